@@ -266,7 +266,9 @@ sg_status sg_sort(sg_ctx* ctx, sg_vector* keys, sg_vector** out);
 
 /* ------------------------------------------------------------------------ */
 /* Matrix product (Sec. 3.4 `multiply`): C = A B.  A: M x K, B: K x N, SG_F32
- * storage; C: M x N SG_F32.  `precision` selects binary32 SIMT arithmetic or
+ * storage; C: M x N SG_F32.  `precision` selects binary32 arithmetic (on the
+ * CUDA cores, or for larger sizes on the tensor cores with every operand split
+ * exactly into three bf16 pieces; products of binary32 accuracy either way) or
  * bf16 / fp16 operands (rounded to nearest even) on the tensor cores with
  * binary32 accumulation.  Built-in postcondition (mode >= PRE_POST):
  * Freivalds' check with 4 Rademacher vectors (see sg_contract). */

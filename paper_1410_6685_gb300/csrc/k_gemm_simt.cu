@@ -17,7 +17,11 @@ template <bool VEC>
 __global__ void __launch_bounds__(256) k_gemm_f32(const float* __restrict__ A, int lda,
                                                   const float* __restrict__ B, int ldb,
                                                   float* __restrict__ C, int ldc, int M, int N,
-                                                  int K, int subtract) {
+                                                  int K, int subtract,
+                                                  const int* only_if) {
+  // queued behind the split product (k_gemm_split.cu): only for operands it
+  // does not take, or (nothing was subtracted yet) after one of its waits gave up
+  if (only_if && only_if[0] == 0 && (subtract || only_if[1] == 0)) return;
   __shared__ __align__(16) float As[2][BK][BM];
   __shared__ __align__(16) float Bs[2][BK][BN];
   const int tid = threadIdx.x;
@@ -117,7 +121,8 @@ __global__ void __launch_bounds__(256) k_gemm_f32(const float* __restrict__ A, i
 }  // namespace
 
 cudaError_t launch_gemm_f32(const float* A, int lda, const float* B, int ldb, float* C, int ldc,
-                            int M, int N, int K, bool subtract, cudaStream_t s, Prof* prof) {
+                            int M, int N, int K, bool subtract, cudaStream_t s, Prof* prof,
+                            const int* only_if) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   const bool vec = (lda % 4 == 0) && (ldb % 4 == 0) && (ldc % 4 == 0) &&
                    ((uintptr_t)A % 16 == 0) && ((uintptr_t)B % 16 == 0) &&
@@ -125,9 +130,11 @@ cudaError_t launch_gemm_f32(const float* A, int lda, const float* B, int ldb, fl
   dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
   prof_begin(prof, "gemm_f32_simt", s);
   if (vec)
-    k_gemm_f32<true><<<grid, 256, 0, s>>>(A, lda, B, ldb, C, ldc, M, N, K, subtract ? 1 : 0);
+    k_gemm_f32<true><<<grid, 256, 0, s>>>(A, lda, B, ldb, C, ldc, M, N, K, subtract ? 1 : 0,
+                                         only_if);
   else
-    k_gemm_f32<false><<<grid, 256, 0, s>>>(A, lda, B, ldb, C, ldc, M, N, K, subtract ? 1 : 0);
+    k_gemm_f32<false><<<grid, 256, 0, s>>>(A, lda, B, ldb, C, ldc, M, N, K, subtract ? 1 : 0,
+                                         only_if);
   prof_end(prof, s);
   return cudaGetLastError();
 }

@@ -1,0 +1,608 @@
+// k_gemm_split.cu -- the binary32 matrix product (Sec. 3.4 `multiply`,
+// SG_PREC_F32_SIMT) of larger sizes on the 5th-generation tensor cores
+// (sm_103a): C = A B (or C = C - A B, the elimination's update).
+//
+// Every binary32 operand is split exactly into three bf16 pieces, x = x1 +
+// x2 + x3 (24 = 8 + 8 + 8 significant bits; x2 and x3 round to nearest what
+// is left), and the product is the sum of the six piece products that matter
+// -- x1 y1, x1 y2, x2 y1, x2 y2, x1 y3, x3 y1 -- each exact in binary32.  What
+// is left out, x2 y3 + x3 y2 + x3 y3, is at most 2^-25.9 of |x y|, about a
+// quarter of one binary32 rounding (2^-24).
+//
+// The tensor core adds into its accumulator by truncation, so a long sum kept
+// there drifts toward zero: 512 steps of K = 16 at K = 8192.  It therefore
+// only sums TK = 32 consecutive k, the smaller products first, so that
+// the accumulator is truncated twice at its full size; the epilogue warps
+// take each chunk's sum out of tensor memory and add it, rounding to
+// nearest, to a running sum in registers while the tensor core fills the
+// other accumulator with the next chunk.
+//
+// The tensor pipe bounds it: six bf16 multiply-adds per binary32 one, so a
+// sixth of the bf16 rate, about 317 TFLOP/s of measured, where the CUDA
+// cores' form (k_gemm_simt.cu) reaches 44-49.
+//
+// Range: pieces and piece products stay normal numbers for |x| = 0 or
+// 2^-50 <= |x| < 2^55.  The cast kernels raise a flag for any other value
+// (subnormals, infinities, NaN, extreme scales); then this kernel does
+// nothing and the CUDA-core form, queued behind it, computes the product.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
+#include <algorithm>
+
+#include "sg_linalg_kernels.h"
+#include "sg_tcgen05.cuh"
+
+namespace sgk {
+namespace {
+
+using namespace tc;
+
+constexpr int TK = 32;        // k per pipeline stage and per tensor-memory accumulation
+constexpr int kEpiWarps = 8;
+constexpr int kThreads = 96 + 32 * kEpiWarps;   // producer, two MMA issuers, epilogue
+constexpr int T_BYTES = kEpiWarps * 16 * 32 * 4;
+
+// Tile forms.  PAIR: a CTA pair computes 256 x TN (each CTA 128 rows of A and
+// TN / 2 rows of B^T per stage); else one CTA computes 128 x TN.
+template <bool PAIR, int TN>
+struct Form {
+  static constexpr int kBRows = PAIR ? TN / 2 : TN;
+  static constexpr int kAPiece = 128 * TK * 2;
+  static constexpr int kBPiece = kBRows * TK * 2;
+  static constexpr int kStageBytes = 3 * (kAPiece + kBPiece);
+  static constexpr int kTileM = PAIR ? 256 : 128;
+  static constexpr int kStages = (232448 - 1024 - 256 - T_BYTES) / kStageBytes;   // 4 or 5
+  static constexpr int kSmem = kStages * kStageBytes + 1024 + 256 + T_BYTES;
+  // kind::f16, D f32, A / B bf16, both K-major
+  static constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) |
+                                     ((uint32_t)(TN >> 3) << 17) |
+                                     ((uint32_t)(kTileM >> 4) << 24);
+};
+
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y,
+                                            int z, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, int x,
+                                                 int y, int z, uint32_t bar_cl) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar_cl)
+      : "memory");
+}
+
+// 16 columns of the warp's 32 tensor-memory lanes (16, not 32: the running
+// sums already hold 128 registers)
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
+        "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// shared-memory descriptor of a K-major tile in the 64-byte swizzle layout
+// (rows of 64 B, 8-row groups 512 B apart)
+__device__ __forceinline__ uint64_t sdesc64(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);   // start address >> 4
+  d |= (uint64_t)1 << 16;                      // leading byte offset (unused here)
+  d |= (uint64_t)(512 >> 4) << 32;             // stride byte offset: 8 rows x 64 B
+  d |= (uint64_t)1 << 46;                      // descriptor version
+  d |= (uint64_t)4 << 61;                      // 64-byte swizzle
+  return d;
+}
+
+// true in one lane of a converged warp
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(p));
+  return p != 0;
+}
+
+// Persistent, roles as in k_gemm_tc / k_gemm_tc2: warp 0 TMA producer, warps 1
+// and 10 MMA issuers, warps 2..9 epilogue (lane quarter warp % 4, column half
+// (warp - 2) / 4).  Chunks of all tiles are numbered in one sequence; chunk
+// it uses accumulator it & 1.  gate[0] != 0: nothing is done.
+template <bool PAIR, int TN, bool SUB>
+__global__ void __launch_bounds__(kThreads, 1)
+    k_gemm_split(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb,
+                 float* __restrict__ C, int ldc, int M, int N, int KB, const int* gate, int* err) {
+  using F = Form<PAIR, TN>;
+  constexpr int HN = TN / 2;                  // columns per epilogue warp
+  constexpr int NC = HN / 32;                 // 32-column groups of the store
+  constexpr int kStages = F::kStages;
+  if (*gate != 0) return;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * F::kStageBytes);
+  // bars[0..S): stage full, [S..2S): stage done (its MMAs have completed),
+  // [2S, 2S+2): accumulator empty, [2S+2]: drain
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 3);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  float* s_t = reinterpret_cast<float*>(smem + kStages * F::kStageBytes + 256);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = PAIR ? cluster_rank() : 0;
+  const int unit = PAIR ? blockIdx.x >> 1 : blockIdx.x;
+  const int nunits = PAIR ? gridDim.x >> 1 : gridDim.x;
+  const int nN = (N + TN - 1) / TN, nM = (M + F::kTileM - 1) / F::kTileM;
+  const int ntiles = nN * nM;
+  const uint32_t stage0 = smem_u32(smem), full0 = smem_u32(bars), done0 = full0 + 8 * kStages;
+  const uint32_t tempty0 = done0 + 8 * kStages, drain_bar = tempty0 + 16;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(full0 + 8 * s, PAIR ? 2 : 1);
+      mbar_init(done0 + 8 * s, 1);
+    }
+    mbar_init(tempty0, (PAIR ? 2 : 1) * kEpiWarps);
+    mbar_init(tempty0 + 8, (PAIR ? 2 : 1) * kEpiWarps);
+    mbar_init(drain_bar, 2);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 2) {
+    if (PAIR) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                       smem_u32(tmem_slot)), "r"(2 * TN) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                       smem_u32(tmem_slot)), "r"(2 * TN) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if (PAIR) cluster_sync(); else __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int it = 0;
+      bool ok = true;
+      for (int t = unit; t < ntiles && ok; t += nunits) {
+        int bm, bn;
+        tile_coords(t, nM, nN, &bm, &bn);
+        const int m0 = bm * F::kTileM + (int)rank * 128;
+        const int n0 = bn * TN + (int)rank * F::kBRows;
+        for (int kb = 0; kb < KB; ++kb, ++it) {
+          const int s = it % kStages;
+          const uint32_t ph = (uint32_t)(it / kStages) & 1u;
+          if (it >= kStages &&
+              !mbar_wait_ab(done0 + 8 * s, ph ^ 1u, err, abort_flag)) {
+            ok = false;
+            break;
+          }
+          const uint32_t dst = stage0 + (uint32_t)(s * F::kStageBytes);
+          if (PAIR) {
+            const uint32_t full = map_rank(full0 + 8 * s, 0);
+            mbar_expect_tx_cl(full, F::kStageBytes);
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+              tma_load_3d_pair(dst + p * F::kAPiece, &ma, kb * TK, m0, p, full);
+              tma_load_3d_pair(dst + 3 * F::kAPiece + p * F::kBPiece, &mb, kb * TK, n0, p, full);
+            }
+          } else {
+            const uint32_t full = full0 + 8 * s;
+            mbar_expect_tx(full, F::kStageBytes);
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+              tma_load_3d(dst + p * F::kAPiece, &ma, kb * TK, m0, p, full);
+              tma_load_3d(dst + 3 * F::kAPiece + p * F::kBPiece, &mb, kb * TK, n0, p, full);
+            }
+          }
+        }
+      }
+    }
+  } else if (warp == 1 || warp == 2 + kEpiWarps) {
+    // Two issuer warps, one per accumulator, taking turns by chunk: a chunk's
+    // two waits and its commit take about 470 clocks, in which the tensor
+    // pipe ran dry behind a single issuer.  The whole warp runs the loop and
+    // one elected lane issues, so that the descriptors stay in uniform
+    // registers: with a lone diverged lane each tcgen05.mma took 68 clocks to
+    // issue, more than a 64-column one takes to run.  A chunk's commit
+    // releases its stage to the producer and hands its accumulator to the
+    // epilogue (both wait on it).
+    if (rank == 0) {
+      const int acc = warp == 1 ? 0 : 1;
+      int it = 0, s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int t = unit; t < ntiles && ok; t += nunits) {
+        for (int kb = 0; kb < KB; ++kb, ++it) {
+          if ((it & 1) != acc) {   // the other issuer's chunk
+            if (++s == kStages) {
+              s = 0;
+              ph ^= 1u;
+            }
+            continue;
+          }
+          ok = mbar_wait_ab(full0 + 8 * s, ph, err, abort_flag) &&
+               (it < 2 || mbar_wait_ab(tempty0 + 8 * acc, (uint32_t)((it >> 1) - 1) & 1u, err,
+                                       abort_flag));
+          ok = __all_sync(0xffffffffu, ok);   // the lanes give up together
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t dacc = tmem + (uint32_t)(acc * TN);
+          const uint64_t da0 = sdesc64(stage0 + (uint32_t)(s * F::kStageBytes));
+          const uint64_t db0 = da0 + (uint64_t)(3 * F::kAPiece >> 4);
+          if (elect_one()) {
+            // the smaller products first, the largest (piece 1 of both) last
+            constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
+#pragma unroll
+            for (int p = 0; p < 6; ++p) {
+#pragma unroll
+              for (int k = 0; k < TK / 16; ++k) {
+                // 16 elements (32 bytes) along K inside the swizzled rows
+                const uint64_t da = da0 + (uint64_t)((pa[p] * F::kAPiece >> 4) + 2 * k);
+                const uint64_t db = db0 + (uint64_t)((pb[p] * F::kBPiece >> 4) + 2 * k);
+                if (PAIR)
+                  umma2(dacc, da, db, F::kIdesc, (p | k) != 0);
+                else
+                  umma(dacc, da, db, F::kIdesc, (p | k) != 0);
+              }
+            }
+            if (PAIR) umma_commit_pair(done0 + 8 * s);
+            else umma_commit(done0 + 8 * s);
+          }
+          __syncwarp();
+          if (++s == kStages) {
+            s = 0;
+            ph ^= 1u;
+          }
+        }
+      }
+      // completes when every MMA issued above has finished
+      if (elect_one()) {
+        if (PAIR) umma_commit_pair(drain_bar);
+        else umma_commit(drain_bar);
+      }
+      __syncwarp();
+    }
+  } else {
+    const int q = warp & 3, hh = (warp - 2) >> 2;
+    float* s_tw = s_t + (warp - 2) * 16 * 32;
+    const uint32_t tempty_cl = PAIR ? map_rank(tempty0, 0) : 0;
+    const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(hh * HN);
+    int ch = 0, s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int t = unit; t < ntiles && ok; t += nunits) {
+      int bm, bn;
+      tile_coords(t, nM, nN, &bm, &bn);
+      const int m0q = bm * F::kTileM + (int)rank * 128 + q * 32, c0 = bn * TN + hh * HN;
+      if (SUB) prefetch_c_row(C, ldc, M, N, m0q + lane, c0, HN);
+      float sum[HN];
+#pragma unroll
+      for (int j = 0; j < HN; ++j) sum[j] = 0.0f;
+#pragma unroll 1
+      for (int i = 0; i < KB; ++i, ++ch) {
+        const int acc = ch & 1;
+        if (!mbar_wait_ab(done0 + 8 * s, ph, err, abort_flag)) {
+          ok = false;
+          break;
+        }
+        if (++s == kStages) {
+          s = 0;
+          ph ^= 1u;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+        for (int c = 0; c < HN / 16; ++c) {
+          uint32_t r[16];
+          tmem_ld16(lane_addr + (uint32_t)(acc * TN + c * 16), r);
+          if (c == HN / 16 - 1) {
+            // this warp's part of the accumulator is drained
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) {
+              if (PAIR) mbar_arrive_cl(tempty_cl + 8 * acc);
+              else mbar_arrive(tempty0 + 8 * acc);
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < 16; ++j) sum[c * 16 + j] += __uint_as_float(r[j]);
+        }
+      }
+      if (!ok) break;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        float4 cv[8];
+        if (SUB) load_c(C, ldc, M, N, m0q, c0 + c * 32, lane, cv);
+        uint32_t r[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(sum[c * 32 + j]);
+        store_chunk(C, ldc, M, N, m0q, c0 + c * 32, r, s_tw, lane, SUB ? 1 : 0, cv);
+      }
+    }
+  }
+  __syncthreads();
+  if (warp == 2) {
+    // every MMA has completed before the tensor memory is released
+    mbar_wait(drain_bar, 0, err);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (PAIR)
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                   "r"(2 * TN) : "memory");
+    else
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                   "r"(2 * TN) : "memory");
+  }
+  // neither CTA leaves while the other may still signal its barriers
+  if (PAIR) cluster_sync();
+}
+
+// x = p[0] + p[1] + p[2], each a bf16 (nearest to what is left); true when x
+// is outside the range in which the pieces and their products are exact
+__device__ __forceinline__ bool split3(float x, uint16_t (&p)[3]) {
+  const uint32_t e = (__float_as_uint(x) >> 23) & 0xFFu;
+  const __nv_bfloat16 h = __float2bfloat16_rn(x);
+  const float r1 = x - __bfloat162float(h);
+  const __nv_bfloat16 m = __float2bfloat16_rn(r1);
+  const float r2 = r1 - __bfloat162float(m);
+  const __nv_bfloat16 l = __float2bfloat16_rn(r2);
+  p[0] = *reinterpret_cast<const uint16_t*>(&h);
+  p[1] = *reinterpret_cast<const uint16_t*>(&m);
+  p[2] = *reinterpret_cast<const uint16_t*>(&l);
+  return x != 0.0f && (e < 127u - 50u || e > 127u + 54u);
+}
+
+// A (rows x cols, leading dimension lda) -> out[3][rows][Kp], zero padded
+__global__ void __launch_bounds__(256) k_split_rows(const float* __restrict__ A, int lda, int rows,
+                                                    int cols, int Kp, uint16_t* __restrict__ out,
+                                                    int* gate, int vec) {
+  const long long total = (long long)rows * (Kp / 8), plane = (long long)rows * Kp;
+  bool bad = false;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
+       t += (long long)gridDim.x * blockDim.x) {
+    const int r = (int)(t / (Kp / 8)), c0 = (int)(t % (Kp / 8)) * 8;
+    const float* src = A + (size_t)r * lda + c0;
+    float x[8];
+    if (vec && c0 + 8 <= cols) {
+      const float4 u = __ldcs(reinterpret_cast<const float4*>(src));
+      const float4 v = __ldcs(reinterpret_cast<const float4*>(src) + 1);
+      x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w;
+      x[4] = v.x; x[5] = v.y; x[6] = v.z; x[7] = v.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) x[j] = c0 + j < cols ? __ldcs(src + j) : 0.0f;
+    }
+    uint32_t w[3][4];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      uint16_t p[3];
+      bad |= split3(x[j], p);
+#pragma unroll
+      for (int z = 0; z < 3; ++z)
+        w[z][j >> 1] = (j & 1) ? w[z][j >> 1] | ((uint32_t)p[z] << 16) : (uint32_t)p[z];
+    }
+#pragma unroll
+    for (int z = 0; z < 3; ++z)
+      *reinterpret_cast<uint4*>(out + z * plane + (long long)r * Kp + c0) =
+          make_uint4(w[z][0], w[z][1], w[z][2], w[z][3]);
+  }
+  if (bad) *gate = 1;
+}
+
+// B (K x N, leading dimension ldb) -> out[3][N][Kp], transposed through a
+// 64 x 64 tile of shared memory: 16-byte loads along n, 16-byte stores along k
+__global__ void __launch_bounds__(256) k_split_transpose(const float* __restrict__ B, int ldb,
+                                                         int K, int N, int Kp,
+                                                         uint16_t* __restrict__ out, int* gate,
+                                                         int vec) {
+  __shared__ float t[64][65];
+  const int k0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
+  const long long plane = (long long)N * Kp;
+  float4 v[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int e = threadIdx.x + 256 * i, k = k0 + (e >> 4), n = n0 + (e & 15) * 4;
+    const float* src = B + (size_t)k * ldb + n;
+    if (vec && k < K && n + 4 <= N) {
+      v[i] = __ldcs(reinterpret_cast<const float4*>(src));
+    } else {
+      float x[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[j] = k < K && n + j < N ? __ldcs(src + j) : 0.0f;
+      v[i] = make_float4(x[0], x[1], x[2], x[3]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int e = threadIdx.x + 256 * i, r = e >> 4, c = (e & 15) * 4;
+    t[r][c] = v[i].x; t[r][c + 1] = v[i].y; t[r][c + 2] = v[i].z; t[r][c + 3] = v[i].w;
+  }
+  __syncthreads();
+  bool bad = false;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int e = threadIdx.x + 256 * i, nn = e >> 3, kc = (e & 7) * 8;
+    if (n0 + nn >= N) continue;
+    uint32_t w[3][4];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      uint16_t p[3];
+      bad |= split3(t[kc + j][nn], p);
+#pragma unroll
+      for (int z = 0; z < 3; ++z)
+        w[z][j >> 1] = (j & 1) ? w[z][j >> 1] | ((uint32_t)p[z] << 16) : (uint32_t)p[z];
+    }
+#pragma unroll
+    for (int z = 0; z < 3; ++z)
+      *reinterpret_cast<uint4*>(out + z * plane + (long long)(n0 + nn) * Kp + k0 + kc) =
+          make_uint4(w[z][0], w[z][1], w[z][2], w[z][3]);
+  }
+  if (bad) *gate = 1;
+}
+
+PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
+  static PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
+                                         &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      p = nullptr;
+    return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+  }();
+  return fn;
+}
+
+// the pieces [3][rows][Kp], boxes of 64 x box_rows of one piece; rows past
+// the end read as zero
+bool make_map3(CUtensorMap* m, const void* base, int rows, int Kp, int box_rows) {
+  auto fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)Kp, (cuuint64_t)rows, 3};
+  cuuint64_t strides[2] = {(cuuint64_t)Kp * 2, (cuuint64_t)rows * Kp * 2};
+  cuuint32_t box[3] = {(cuuint32_t)TK, (cuuint32_t)box_rows, 1};
+  cuuint32_t es[3] = {1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
+            es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+int sm_count() {
+  static int sms = [] {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
+      v = 1;
+    return v;
+  }();
+  return sms;
+}
+
+template <bool PAIR, int TN, bool SUB>
+cudaError_t launch_form(const uint16_t* a3, const uint16_t* b3, int Kp, float* C, int ldc, int M,
+                        int N, int K, const int* gate, int* err, cudaStream_t s) {
+  using F = Form<PAIR, TN>;
+  CUtensorMap ma, mb;
+  if (!make_map3(&ma, a3, M, Kp, 128) || !make_map3(&mb, b3, N, Kp, F::kBRows))
+    return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(k_gemm_split<PAIR, TN, SUB>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, F::kSmem);
+  if (e != cudaSuccess) return e;
+  const long long tiles = (long long)((M + F::kTileM - 1) / F::kTileM) * ((N + TN - 1) / TN);
+  const int units = (int)std::min<long long>(tiles, PAIR ? sm_count() / 2 : sm_count());
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((PAIR ? 2 : 1) * units);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = F::kSmem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  if (PAIR) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+  }
+  return cudaLaunchKernelEx(&cfg, k_gemm_split<PAIR, TN, SUB>, ma, mb, C, ldc, M, N, (K + TK - 1) / TK,
+                            gate, err);
+}
+
+template <bool SUB>
+cudaError_t launch_split(int form, const uint16_t* a3, const uint16_t* b3, int Kp, float* C,
+                         int ldc, int M, int N, int K, const int* gate, int* err, cudaStream_t s) {
+  switch (form) {
+    case 2: return launch_form<true, 256, SUB>(a3, b3, Kp, C, ldc, M, N, K, gate, err, s);
+    case 1: return launch_form<false, 128, SUB>(a3, b3, Kp, C, ldc, M, N, K, gate, err, s);
+    default: return launch_form<false, 64, SUB>(a3, b3, Kp, C, ldc, M, N, K, gate, err, s);
+  }
+}
+
+// Estimated microseconds of the product in each tile form, and the form with
+// the least: waves of tiles times (chunks of 32 k, and the tile's start and
+// store).  Measured per chunk: 0.40 us (128 x 64), 0.48 us (128 x 128), 0.84 us
+// (a pair's 256 x 256), so the larger tiles win once they fill the chip: at
+// 1000^3 20.6 / 22.5 / 39.2 us, at 2048^3 110 / 67.2 / 65.2 us, at 8192^3 5459 /
+// 3774 / 3198 us (344 TFLOP/s; the CUDA cores 22400 us).
+int choose_form(int M, int N, int K, double* us) {
+  const double c = (K + TK - 1) / TK;
+  auto waves = [&](int tm, int tn, int slots) {
+    const long long t = (long long)((M + tm - 1) / tm) * ((N + tn - 1) / tn);
+    return (double)((t + slots - 1) / slots);
+  };
+  const int sms = sm_count();
+  const double t[3] = {6.5 + waves(128, 64, sms) * (0.40 * c + 1.5),
+                       6.5 + waves(128, 128, sms) * (0.48 * c + 3.0),
+                       gemm_pair_available()
+                           ? 7.0 + waves(256, 256, std::max(1, sms / 2)) * (0.84 * c + 5.0)
+                           : 1e300};
+  const int f = (int)(std::min_element(t, t + 3) - t);
+  if (us) *us = t[f];
+  return f;
+}
+
+}  // namespace
+
+// Where the split product gains over the CUDA cores' form, by estimates of
+// both: the casts stream 10 bytes per operand entry and cost two launches,
+// the CUDA cores take 0.145 us per k up to one 128 x 128 tile per SM and 0.71
+// ns per k and tile beyond (1000 x 1000 x 100: 20.3 us on the CUDA cores, 24 us
+// split; 200^3: 34 against 26 us).  Not for K <= 64, where the CUDA cores'
+// sum rounds as rarely, nor where the pieces would take more than 16 GB of
+// scratch.
+bool gemm_split_wanted(int M, int N, int K) {
+  if (M <= 0 || N <= 0 || K <= 64) return false;
+  if (gemm_split_scratch_bytes(M, N, K) > ((size_t)16 << 30)) return false;
+  double split = 0.0;
+  choose_form(M, N, K, &split);
+  split += 11.0 + 10.0 * K * ((double)M + N) / 6.0e6;
+  const double tiles = (double)((M + 127) / 128) * ((N + 127) / 128);
+  const double simt = 3.0 + K * std::max(0.145, 0.00071 * tiles) + 4.0 * M * (double)N / 2.5e6;
+  return split < simt;
+}
+
+size_t gemm_split_scratch_bytes(int M, int N, int K) {
+  const size_t Kp = (size_t)((K + 63) / 64) * 64;
+  return 256 + align256((size_t)M * Kp * 6) + align256((size_t)N * Kp * 6);
+}
+
+cudaError_t launch_gemm_split(const float* A, int lda, const float* B, int ldb, float* C, int ldc,
+                              int M, int N, int K, bool subtract, void* scratch, cudaStream_t s,
+                              Prof* prof, int64_t* kernels, int form) {
+  const int Kp = ((K + 63) / 64) * 64;
+  char* p = static_cast<char*>(scratch);
+  int* gate = reinterpret_cast<int*>(p);   // [0] out of range, [1] a wait gave up
+  uint16_t* a3 = reinterpret_cast<uint16_t*>(p + 256);
+  uint16_t* b3 = reinterpret_cast<uint16_t*>(p + 256 + align256((size_t)M * Kp * 6));
+  const int va = lda % 4 == 0 && (uintptr_t)A % 16 == 0;
+  const int vb = ldb % 4 == 0 && (uintptr_t)B % 16 == 0;
+  prof_begin(prof, "split_operands", s);
+  cudaError_t e = cudaMemsetAsync(gate, 0, 8, s);
+  if (e != cudaSuccess) return e;
+  const long long ca = (long long)M * (Kp / 8);
+  k_split_rows<<<(int)std::min<long long>((ca + 255) / 256, 65535LL * 8), 256, 0, s>>>(
+      A, lda, M, K, Kp, a3, gate, va);
+  k_split_transpose<<<dim3((N + 63) / 64, Kp / 64), 256, 0, s>>>(B, ldb, K, N, Kp, b3, gate, vb);
+  prof_end(prof, s);
+  prof_begin(prof, "gemm_f32_split", s);
+  if (form < 0) form = choose_form(M, N, K, nullptr);
+  e = subtract ? launch_split<true>(form, a3, b3, Kp, C, ldc, M, N, K, gate, gate + 1, s)
+               : launch_split<false>(form, a3, b3, Kp, C, ldc, M, N, K, gate, gate + 1, s);
+  prof_end(prof, s);
+  if (e != cudaSuccess) return e;
+  *kernels += 4;
+  return launch_gemm_f32(A, lda, B, ldb, C, ldc, M, N, K, subtract, s, prof, gate);
+}
+
+}  // namespace sgk

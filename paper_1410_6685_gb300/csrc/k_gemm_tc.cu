@@ -29,9 +29,12 @@
 
 #include "sg_frv.cuh"
 #include "sg_linalg_kernels.h"
+#include "sg_tcgen05.cuh"
 
 namespace sgk {
 namespace {
+
+using namespace tc;
 
 constexpr int TM = 128, TN = 256, TK = 64, STAGES = 4;
 static_assert(kFrvTileC == TN / 2, "the fused check keeps one C r partial per epilogue warp's column half");
@@ -54,199 +57,10 @@ constexpr int R_BYTES = kEpiWarps * (TN / 2) * 16;  // the fused check's r entri
 constexpr int T_BYTES = kEpiWarps * 16 * 32 * 4;    // one 16 x 32 buffer per epilogue warp
 constexpr int SMEM_BYTES =
     STAGES * STAGE_BYTES + 1024 /*align*/ + 256 /*barriers*/ + R_BYTES + T_BYTES;
-constexpr unsigned kWaitLimit = 1u << 26;
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
-}
-
-// bounded wait for the phase with the given parity to complete
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err) {
-  for (unsigned i = 0; i < kWaitLimit; ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
-  }
-  atomicExch(err, 1);
-  return false;
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y,
-                                            uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
-
-// UMMA shared-memory descriptor: K-major tile in the 128-byte swizzle
-// layout (rows of 128 B, 8-row groups 1024 B apart).
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);   // start address >> 4
-  d |= (uint64_t)1 << 16;                      // leading byte offset (unused here)
-  d |= (uint64_t)(1024 >> 4) << 32;            // stride byte offset: 8 rows x 128 B
-  d |= (uint64_t)1 << 46;                      // descriptor version
-  d |= (uint64_t)2 << 61;                      // 128-byte swizzle
-  return d;
-}
-
 // instruction descriptor, kind::f16: D f32, A/B bf16 or f16, both K-major
 __host__ __device__ constexpr uint32_t idesc(bool fp16) {
   return (1u << 4) | ((fp16 ? 0u : 1u) << 7) | ((fp16 ? 0u : 1u) << 10) |
          ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
-}
-
-__device__ __forceinline__ void umma(uint32_t tmem, uint64_t a, uint64_t b, uint32_t id,
-                                     uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-      "l"(a), "l"(b), "r"(id), "r"(accumulate)
-      : "memory");
-}
-
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-      : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-        "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-        "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
-        "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// bounded wait that also gives up as soon as another role of the CTA has
-// raised the abort flag (so one failed wait cannot leave the others spinning
-// through every remaining tile)
-__device__ __forceinline__ bool mbar_wait_ab(uint32_t bar, uint32_t parity, int* err,
-                                             volatile int* abort_flag) {
-  for (unsigned i = 0; i < kWaitLimit; ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
-    if ((i & 255) == 255 && *abort_flag) return false;
-  }
-  atomicExch(err, 1);
-  *abort_flag = 1;
-  return false;
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-// arrive on a barrier anywhere in the cluster
-__device__ __forceinline__ void mbar_arrive_cl(uint32_t bar_cl) {
-  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar_cl) : "memory");
-}
-
-// C rows m0q .. m0q + 31, columns col0 .. col0 + 31, as the epilogue's
-// stores take them: access it, lane l: row m0q + 4 it + l / 8, columns
-// col0 + 4 (l % 8) .. + 3 (zero outside M x N)
-__device__ __forceinline__ void load_c(const float* __restrict__ C, int ldc, int M, int N, int m0q,
-                                       int col0, int lane, float4 (&cv)[8]) {
-#pragma unroll
-  for (int it = 0; it < 8; ++it) {
-    const int grow = m0q + it * 4 + (lane >> 3), gcol = col0 + (lane & 7) * 4;
-    const float* cp = C + (size_t)grow * ldc + gcol;
-    if (grow < M && gcol + 4 <= N && ((reinterpret_cast<uintptr_t>(cp) & 15) == 0)) {
-      cv[it] = *reinterpret_cast<const float4*>(cp);
-    } else {
-      float e[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) e[u] = grow < M && gcol + u < N ? cp[u] : 0.0f;
-      cv[it] = make_float4(e[0], e[1], e[2], e[3]);
-    }
-  }
-}
-
-// Row `row`, columns c0 .. c0 + w - 1 of C (clipped to N) into L2: the
-// subtracting product's epilogue reads them a tile later
-__device__ __forceinline__ void prefetch_c_row(const float* C, int ldc, int M, int N, int row,
-                                               int c0, int w) {
-  if (row >= M || c0 >= N) return;
-  const float* p = C + (size_t)row * ldc + c0;
-  const unsigned bytes = (unsigned)(min(w, N - c0) * 4) & ~15u;
-  if ((reinterpret_cast<uintptr_t>(p) & 15) == 0 && bytes)
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
-// One 32 x 32 chunk of the epilogue: lane l holds row m0q + l, columns
-// col0 .. col0 + 31 (r); C := chunk, or C := cv - chunk when subtracting (cv
-// from load_c), through the warp's transpose buffer s_tw (16 x 32 floats,
-// rows 16 h .. 16 h + 15 in turn); rows outside M and columns outside N are
-// left alone.
-__device__ __forceinline__ void store_chunk(float* __restrict__ C, int ldc, int M, int N, int m0q,
-                                            int col0, const uint32_t (&r)[32], float* s_tw,
-                                            int lane, int subtract, const float4 (&cv)[8]) {
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    if ((lane >> 4) == h) {
-      const int rw = lane & 15;
-      float4* dst = reinterpret_cast<float4*>(s_tw + rw * 32);
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        dst[j ^ (rw & 7)] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
-                                        __uint_as_float(r[4 * j + 2]),
-                                        __uint_as_float(r[4 * j + 3]));
-    }
-    __syncwarp();
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int rr = it * 4 + (lane >> 3), g = lane & 7;
-      const float4 v = reinterpret_cast<const float4*>(s_tw + rr * 32)[g ^ (rr & 7)];
-      const int grow = m0q + 16 * h + rr, gcol = col0 + 4 * g;
-      if (grow >= M) continue;
-      const float4 c4 = cv[4 * h + it];
-      const float4 o =
-          subtract ? make_float4(c4.x - v.x, c4.y - v.y, c4.z - v.z, c4.w - v.w) : v;
-      float* cp = C + (size_t)grow * ldc + gcol;
-      if (gcol + 4 <= N && ((reinterpret_cast<uintptr_t>(cp) & 15) == 0)) {
-        *reinterpret_cast<float4*>(cp) = o;
-      } else {
-        const float oe[4] = {o.x, o.y, o.z, o.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (gcol + u < N) cp[u] = oe[u];
-      }
-    }
-    __syncwarp();
-  }
 }
 
 // The epilogue of one tile by one epilogue warp: tensor-memory lane quarter
@@ -315,22 +129,6 @@ __device__ __forceinline__ bool epilogue_tile(
   }
   if (frv_r && row < M && c0 < N) frv_pw[(size_t)(2 * bn + hh) * M + row] = wacc;
   return true;
-}
-
-// Tile t of the persistent order: groups of kGroupM row blocks; inside a
-// group the row block varies fastest.  The 76 pairs' concurrent 256 x 256
-// tiles then span 8 row blocks x about 10 column blocks, whose A and B
-// slices (some 75 MB at K = 8192) stay in L2 instead of all of B (groups of
-// 8 measured 0.7% faster than 16, and 32 4% slower).
-constexpr int kGroupM = 8;
-__device__ __forceinline__ void tile_coords(int t, int nM, int nN, int* mb, int* nb) {
-  const int per_group = kGroupM * nN;
-  const int g = t / per_group;
-  const int first = g * kGroupM;
-  const int gm = min(kGroupM, nM - first);
-  const int r = t - g * per_group;
-  *mb = first + r % gm;
-  *nb = r / gm;
 }
 
 // Persistent kernel, one CTA per SM, tiles t = blockIdx.x + i * gridDim.x in
@@ -504,54 +302,6 @@ constexpr int SMEM2_BYTES = STAGES2 * STAGE2_BYTES + 1024 + 256 + R_BYTES + T_BY
 __host__ __device__ constexpr uint32_t idesc2(bool fp16) {
   return (1u << 4) | ((fp16 ? 0u : 1u) << 7) | ((fp16 ? 0u : 1u) << 10) |
          ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(TM2 >> 4) << 24);
-}
-
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t map_rank(uint32_t local, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
-               ::: "memory");
-}
-// arrive (with a byte count to expect) on a barrier anywhere in the cluster;
-// CTA-scope release: a cluster-scope one would wait for every earlier global
-// store of the thread
-__device__ __forceinline__ void mbar_expect_tx_cl(uint32_t bar_cl, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;" ::"r"(bar_cl),
-               "r"(bytes) : "memory");
-}
-// TMA load into this CTA's shared memory completing on a barrier of either CTA of the pair
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int x,
-                                                 int y, uint32_t bar_cl) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar_cl)
-      : "memory");
-}
-__device__ __forceinline__ void umma2(uint32_t tmem, uint64_t a, uint64_t b, uint32_t id,
-                                      uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-      "l"(a), "l"(b), "r"(id), "r"(accumulate)
-      : "memory");
-}
-// arrives once on the barrier at this offset in both CTAs of the pair when
-// every MMA issued before it has completed
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
-      " [%0], %1;" ::"r"(bar), "h"((unsigned short)3)
-      : "memory");
 }
 
 __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc2(const __grid_constant__ CUtensorMap ma,
@@ -752,15 +502,6 @@ __global__ void k_cast_transpose(const float* __restrict__ B, int ldb, int K, in
       out[(size_t)n * Kp + k] = h;
     }
   }
-}
-
-__device__ __forceinline__ uint16_t to16(float v, bool fp16) {
-  if (fp16) {
-    const __half x = __float2half_rn(v);
-    return *reinterpret_cast<const uint16_t*>(&x);
-  }
-  const __nv_bfloat16 x = __float2bfloat16_rn(v);
-  return *reinterpret_cast<const uint16_t*>(&x);
 }
 
 // Square B (N x N) -> Bt (N x Kp) 16-bit, with the fused Freivalds partial

@@ -77,9 +77,17 @@ bool sg_linalg_can_fuse(const Node* mm, const Node* chk) {
          mm->in[0]->rows > 0;
 }
 
+bool sg_linalg_split(const Node* n) {
+  return n->kind == NK::MATMUL && n->prec == SG_PREC_F32_SIMT &&
+         sgk::gemm_split_wanted((int)n->in[0]->rows, (int)n->in[1]->cols, (int)n->in[0]->cols);
+}
+
 size_t sg_linalg_scratch(sg_ctx*, Node* n, Node* fused) {
   if (n->kind == NK::MATMUL) {
-    if (n->prec == SG_PREC_F32_SIMT) return 0;
+    if (n->prec == SG_PREC_F32_SIMT)
+      return n->split ? sgk::gemm_split_scratch_bytes((int)n->in[0]->rows, (int)n->in[1]->cols,
+                                                      (int)n->in[0]->cols)
+                      : 0;
     const size_t g = sgk::gemm_tc_scratch_bytes((int)n->in[0]->rows, (int)n->in[1]->cols,
                                                 (int)n->in[0]->cols);
     return fused ? g + sgk::frv_fused_scratch_bytes((int)n->in[0]->rows) : g;
@@ -126,7 +134,10 @@ sg_status sg_exec_linalg(sg_ctx* c, Node* n, Node* fused, void* rec, void* work,
                                        &c->prof, &c->kernels, ir, ic, id, form);
       return SG_OK;
     }
-    if (n->prec == SG_PREC_F32_SIMT) {
+    if (n->split) {
+      *e = sgk::launch_gemm_split(a, K, b, N, cc, N, M, N, K, false, work, c->stream, &c->prof,
+                                  &c->kernels);
+    } else if (n->prec == SG_PREC_F32_SIMT) {
       *e = sgk::launch_gemm_f32(a, K, b, N, cc, N, M, N, K, false, c->stream, &c->prof);
       c->kernels += 1;
     } else {

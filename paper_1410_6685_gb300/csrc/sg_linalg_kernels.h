@@ -8,7 +8,20 @@ namespace sgk {
 // binary32 SIMT product C = A B (or C = C - A B), row-major with leading
 // dimensions (M x K, K x N, M x N).
 cudaError_t launch_gemm_f32(const float* A, int lda, const float* B, int ldb, float* C, int ldc,
-                            int M, int N, int K, bool subtract, cudaStream_t s, Prof* prof);
+                            int M, int N, int K, bool subtract, cudaStream_t s, Prof* prof,
+                            const int* only_if = nullptr);
+
+// The same binary32 product on the tensor cores (k_gemm_split.cu): operands
+// split into three bf16 pieces each, six piece products, sums carried in
+// binary32 registers.  Operands outside its range, found on the device, fall
+// back to launch_gemm_f32 (queued behind, a no-op otherwise).  wanted: the
+// sizes that gain from it.  form: -1 by the sizes, else 0 / 1 / 2 (128 x 64,
+// 128 x 128, a CTA pair's 256 x 256 tiles).
+bool gemm_split_wanted(int M, int N, int K);
+size_t gemm_split_scratch_bytes(int M, int N, int K);
+cudaError_t launch_gemm_split(const float* A, int lda, const float* B, int ldb, float* C, int ldc,
+                              int M, int N, int K, bool subtract, void* scratch, cudaStream_t s,
+                              Prof* prof, int64_t* kernels, int form = -1);
 
 // Tensor-core product: operands rounded (nearest even) to bf16 or fp16,
 // binary32 accumulation in tensor memory.  beta = 0: C = A B; beta = 1:

@@ -16,6 +16,8 @@ sg_status sg_describe_pending(sg_ctx* c, std::string* out);
 // fused: a built-in Freivalds check folded into the product `n` (or nullptr)
 size_t sg_linalg_scratch(sg_ctx* c, Node* n, Node* fused);
 sg_status sg_exec_linalg(sg_ctx* c, Node* n, Node* fused, void* rec, void* work, cudaError_t* e);
+// a binary32 product that gains from the tensor cores (k_gemm_split.cu)
+bool sg_linalg_split(const Node* n);
 // a product whose Freivalds check can be folded into it
 bool sg_linalg_can_fuse(const Node* mm, const Node* chk);
 // True when the node's check failed; fills the violating row and the

@@ -77,6 +77,7 @@ struct Node {
   int nvec = 4;
   double tol = 0.0;
   int prec = 0;                  // MATMUL precision
+  bool split = false;            // MATMUL in binary32: on the tensor cores, operands in bf16 pieces
   bool left = false;             // MATVEC: y = x^T A (in[0] = x, in[1] = A), else y = A x
   // results filled at execution
   int64_t first = -1;
