@@ -114,16 +114,18 @@ __device__ __forceinline__ bool elect_one() {
 // Persistent, roles as in k_gemm_tc / k_gemm_tc2: warp 0 TMA producer, warps 1
 // and 10 MMA issuers, warps 2..9 epilogue (lane quarter warp % 4, column half
 // (warp - 2) / 4).  Chunks of all tiles are numbered in one sequence; chunk
-// it uses accumulator it & 1.  gate[0] != 0: nothing is done.
+// it uses accumulator it & 1.  gate[0] != 0 or
+// skip[0] != 0 (each written by earlier launches): nothing is done.
 template <bool PAIR, int TN, bool SUB>
 __global__ void __launch_bounds__(kThreads, 1)
     k_gemm_split(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb,
-                 float* __restrict__ C, int ldc, int M, int N, int KB, const int* gate, int* err) {
+                 float* __restrict__ C, int ldc, int M, int N, int KB, const int* gate, const int* skip,
+                 int* err) {
   using F = Form<PAIR, TN>;
   constexpr int HN = TN / 2;                  // columns per epilogue warp
   constexpr int NC = HN / 32;                 // 32-column groups of the store
   constexpr int kStages = F::kStages;
-  if (*gate != 0) return;
+  if (*gate != 0 || (skip && *skip != 0)) return;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -346,21 +348,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (PAIR) cluster_sync();
 }
 
-// x = p[0] + p[1] + p[2], each a bf16 (nearest to what is left); true when x
-// is outside the range in which the pieces and their products are exact
-__device__ __forceinline__ bool split3(float x, uint16_t (&p)[3]) {
-  const uint32_t e = (__float_as_uint(x) >> 23) & 0xFFu;
-  const __nv_bfloat16 h = __float2bfloat16_rn(x);
-  const float r1 = x - __bfloat162float(h);
-  const __nv_bfloat16 m = __float2bfloat16_rn(r1);
-  const float r2 = r1 - __bfloat162float(m);
-  const __nv_bfloat16 l = __float2bfloat16_rn(r2);
-  p[0] = *reinterpret_cast<const uint16_t*>(&h);
-  p[1] = *reinterpret_cast<const uint16_t*>(&m);
-  p[2] = *reinterpret_cast<const uint16_t*>(&l);
-  return x != 0.0f && (e < 127u - 50u || e > 127u + 54u);
-}
-
 // A (rows x cols, leading dimension lda) -> out[3][rows][Kp], zero padded
 __global__ void __launch_bounds__(256) k_split_rows(const float* __restrict__ A, int lda, int rows,
                                                     int cols, int Kp, uint16_t* __restrict__ out,
@@ -491,7 +478,7 @@ int sm_count() {
 
 template <bool PAIR, int TN, bool SUB>
 cudaError_t launch_form(const uint16_t* a3, const uint16_t* b3, int Kp, float* C, int ldc, int M,
-                        int N, int K, const int* gate, int* err, cudaStream_t s) {
+                        int N, int K, const int* gate, const int* skip, int* err, cudaStream_t s) {
   using F = Form<PAIR, TN>;
   CUtensorMap ma, mb;
   if (!make_map3(&ma, a3, M, Kp, 128) || !make_map3(&mb, b3, N, Kp, F::kBRows))
@@ -516,16 +503,16 @@ cudaError_t launch_form(const uint16_t* a3, const uint16_t* b3, int Kp, float* C
     cfg.numAttrs = 1;
   }
   return cudaLaunchKernelEx(&cfg, k_gemm_split<PAIR, TN, SUB>, ma, mb, C, ldc, M, N, (K + TK - 1) / TK,
-                            gate, err);
+                            gate, skip, err);
 }
 
 template <bool SUB>
 cudaError_t launch_split(int form, const uint16_t* a3, const uint16_t* b3, int Kp, float* C,
-                         int ldc, int M, int N, int K, const int* gate, int* err, cudaStream_t s) {
+                         int ldc, int M, int N, int K, const int* gate, const int* skip, int* err, cudaStream_t s) {
   switch (form) {
-    case 2: return launch_form<true, 256, SUB>(a3, b3, Kp, C, ldc, M, N, K, gate, err, s);
-    case 1: return launch_form<false, 128, SUB>(a3, b3, Kp, C, ldc, M, N, K, gate, err, s);
-    default: return launch_form<false, 64, SUB>(a3, b3, Kp, C, ldc, M, N, K, gate, err, s);
+    case 2: return launch_form<true, 256, SUB>(a3, b3, Kp, C, ldc, M, N, K, gate, skip, err, s);
+    case 1: return launch_form<false, 128, SUB>(a3, b3, Kp, C, ldc, M, N, K, gate, skip, err, s);
+    default: return launch_form<false, 64, SUB>(a3, b3, Kp, C, ldc, M, N, K, gate, skip, err, s);
   }
 }
 
@@ -597,12 +584,23 @@ cudaError_t launch_gemm_split(const float* A, int lda, const float* B, int ldb, 
   prof_end(prof, s);
   prof_begin(prof, "gemm_f32_split", s);
   if (form < 0) form = choose_form(M, N, K, nullptr);
-  e = subtract ? launch_split<true>(form, a3, b3, Kp, C, ldc, M, N, K, gate, gate + 1, s)
-               : launch_split<false>(form, a3, b3, Kp, C, ldc, M, N, K, gate, gate + 1, s);
+  e = subtract ? launch_split<true>(form, a3, b3, Kp, C, ldc, M, N, K, gate, nullptr, gate + 1, s)
+               : launch_split<false>(form, a3, b3, Kp, C, ldc, M, N, K, gate, nullptr, gate + 1, s);
   prof_end(prof, s);
   if (e != cudaSuccess) return e;
   *kernels += 4;
   return launch_gemm_f32(A, lda, B, ldb, C, ldc, M, N, K, subtract, s, prof, gate);
+}
+
+cudaError_t launch_gemm_split_operands(const uint16_t* a3, const uint16_t* b3, const float* A,
+                                       int lda, const float* B, int ldb, float* C, int ldc, int M,
+                                       int N, int K, const int* gate, const int* skip, int* err,
+                                       cudaStream_t s, int64_t* kernels) {
+  cudaError_t e = launch_split<true>(choose_form(M, N, K, nullptr), a3, b3, K, C, ldc, M, N, K,
+                                     gate, skip, err, s);
+  if (e != cudaSuccess) return e;
+  *kernels += 2;
+  return launch_gemm_f32(A, lda, B, ldb, C, ldc, M, N, K, true, s, nullptr, gate);
 }
 
 }  // namespace sgk

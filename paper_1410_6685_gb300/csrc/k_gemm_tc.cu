@@ -147,7 +147,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc(const __grid_consta
                                                     int N, int KB, uint32_t id, int subtract,
                                                     int* err, const float4* __restrict__ frv_r,
                                                     float4* __restrict__ frv_pw, int inj_row,
-                                                    int inj_col, float inj_delta) {
+                                                    int inj_col, float inj_delta,
+                                                     const int* skip) {
+  if (skip && *skip != 0) return;   // written by earlier launches
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -310,7 +312,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc2(const __grid_const
                                                      int N, int KB, uint32_t id, int subtract,
                                                      int* err, const float4* __restrict__ frv_r,
                                                      float4* __restrict__ frv_pw, int inj_row,
-                                                     int inj_col, float inj_delta) {
+                                                     int inj_col, float inj_delta,
+                                                     const int* skip) {
+  if (skip && *skip != 0) return;   // written by earlier launches
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -750,7 +754,7 @@ bool use_pair() {
 cudaError_t launch_product(const uint16_t* a16, const uint16_t* bt16, int Kp, bool fp16, float* C,
                            int ldc, int M, int N, bool subtract, int* err, const float4* frv_r,
                            float4* frv_pw, int inj_row, int inj_col, float inj_delta,
-                           cudaStream_t s, int form) {
+                           cudaStream_t s, int form, const int* skip = nullptr) {
   CUtensorMap ma, mb;
   if (!make_map(&ma, a16, M, Kp, TM, fp16)) return cudaErrorInvalidValue;
   if (form != 1 && !portable_kernels() && use_pair()) {
@@ -771,7 +775,8 @@ cudaError_t launch_product(const uint16_t* a16, const uint16_t* bt16, int Kp, bo
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k_gemm_tc2, ma, mb, C, ldc, M, N, Kp / TK, idesc2(fp16),
-                              subtract ? 1 : 0, err, frv_r, frv_pw, inj_row, inj_col, inj_delta);
+                              subtract ? 1 : 0, err, frv_r, frv_pw, inj_row, inj_col, inj_delta,
+                              skip);
   }
   static bool attr_done = false;
   if (!attr_done) {
@@ -784,7 +789,7 @@ cudaError_t launch_product(const uint16_t* a16, const uint16_t* bt16, int Kp, bo
   k_gemm_tc<<<persistent_grid(M, N), kGemmThreads, SMEM_BYTES, s>>>(ma, mb, C, ldc, M, N, Kp / TK,
                                                            idesc(fp16), subtract ? 1 : 0, err,
                                                            frv_r, frv_pw, inj_row, inj_col,
-                                                           inj_delta);
+                                                           inj_delta, skip);
   return cudaGetLastError();
 }
 
@@ -894,6 +899,14 @@ cudaError_t launch_gemm_tc(const float* A, int lda, const float* B, int ldb, flo
   prof_end(prof, s);
   *kernels += 3;
   return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t launch_gemm_tc_operands(const uint16_t* a16, const uint16_t* bt16, int K, bool fp16,
+                                    float* C, int ldc, int M, int N, int* err, const int* skip,
+                                    cudaStream_t s, int64_t* kernels) {
+  *kernels += 1;
+  return launch_product(a16, bt16, K, fp16, C, ldc, M, N, true, err, nullptr, nullptr, -1, -1, 0.0f,
+                        s, 0, skip);
 }
 
 cudaError_t launch_gemm_tc_checked(const float* A, const float* B, float* C, int N, bool fp16,

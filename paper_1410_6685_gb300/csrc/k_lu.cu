@@ -39,13 +39,14 @@
 
 #include "sg_lu.h"
 #include "sg_linalg_kernels.h"
+#include "sg_lu_tri.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace sgk {
 namespace {
 
-constexpr int kPB = 32;       // panel width
+constexpr int kPB = kLuPanel;   // panel width
 // CTAs per cluster (PC): 16 where the device schedules clusters of 16
 // (non-portable size), else 8
 constexpr int kPT = 256;      // threads per CTA
@@ -616,35 +617,6 @@ __global__ void __launch_bounds__(128) k_lu_laswp_outer(float* LU, int n, const 
   }
 }
 
-// x := L^-1 x for one column x of 32 entries (stride xs) and the unit lower
-// triangle of L (row stride ls, a multiple of 4; L 16-byte aligned), by
-// forward substitution in registers: row i subtracts L[i][0] x[0], L[i][1]
-// x[1], ... in that order, reading L's row four entries per shared-memory
-// load.
-__device__ __forceinline__ void unit_lower_solve_col4(const float* L, int ls, float* x, int xs) {
-  float v[kPB];
-#pragma unroll
-  for (int i = 0; i < kPB; ++i) v[i] = x[i * xs];
-#pragma unroll
-  for (int i = 1; i < kPB; ++i) {
-    float acc = v[i];
-    const float4* Li = reinterpret_cast<const float4*>(L + i * ls);
-#pragma unroll
-    for (int g = 0; g < i / 4; ++g) {
-      const float4 l = Li[g];
-      acc = fmaf(-l.x, v[4 * g], acc);
-      acc = fmaf(-l.y, v[4 * g + 1], acc);
-      acc = fmaf(-l.z, v[4 * g + 2], acc);
-      acc = fmaf(-l.w, v[4 * g + 3], acc);
-    }
-#pragma unroll
-    for (int q = (i / 4) * 4; q < i; ++q) acc = fmaf(-L[i * ls + q], v[q], acc);
-    v[i] = acc;
-  }
-#pragma unroll
-  for (int i = 1; i < kPB; ++i) x[i * xs] = v[i];
-}
-
 // After panel j inside an outer block, for its columns [c0, c1) to the right
 // of the panel (at most kLuOuter - kPB):
 //   U12 = L11^-1 A12 (rows j..j+32; L11 the panel's unit lower triangle)
@@ -1138,7 +1110,8 @@ __global__ void __launch_bounds__(1024) k_lu_det(const float* __restrict__ LU, i
   }
 }
 
-// |A|_inf (binary64) once per solve
+// |A|_inf (binary64) once per factorisation, and whether every row is
+// diagonally dominant: 2 |a_ii| >= sum_j |a_ij| (NaN: not)
 __global__ void __launch_bounds__(256) k_anorm(const float* __restrict__ A, int n, double* norms) {
   const int lane = threadIdx.x & 31;
   const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
@@ -1151,6 +1124,7 @@ __global__ void __launch_bounds__(256) k_anorm(const float* __restrict__ A, int 
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     mx = fmax(mx, s);
+    if (lane == 0 && !(2.0 * fabs((double)row[i]) >= s)) *reinterpret_cast<int*>(&norms[6]) = 1;
   }
   if (lane == 0) atomicMax(reinterpret_cast<unsigned long long*>(&norms[3]),
                            (unsigned long long)__double_as_longlong(mx));
@@ -1264,6 +1238,7 @@ size_t lu_panel_max_smem(int n) { return panel_smem<8>(n, 0); }
 
 cudaError_t lu_prepare(int n) {
   gemm_tc_prepare();
+  if (cudaError_t de = lu_diag_prepare(); de != cudaSuccess) return de;
   const bool c16 = !portable_kernels() && use_cluster16();
   const size_t ps = c16 ? panel_reg_smem<16>(n, 0) : panel_smem<8>(n, 0);
   cudaError_t e;

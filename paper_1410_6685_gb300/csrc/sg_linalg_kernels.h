@@ -44,6 +44,12 @@ cudaError_t launch_gemm_tc(const float* A, int lda, const float* B, int ldb, flo
                            cudaStream_t s, Prof* prof, int64_t* kernels, int inj_row = -1,
                            int inj_col = -1, float inj_delta = 0.0f, int form = 0);
 bool gemm_pair_available();
+// C -= A16 Bt16^T, the elimination's update with its operands already in
+// K-major 16-bit copies (M x K and N x K, K a multiple of 64); nothing is done
+// when *skip != 0
+cudaError_t launch_gemm_tc_operands(const uint16_t* a16, const uint16_t* bt16, int K, bool fp16,
+                                    float* C, int ldc, int M, int N, int* err, const int* skip,
+                                    cudaStream_t s, int64_t* kernels);
 // Casts the operands once, then times the product C = A B in each of `forms`
 // (a warm-up, then the better of two runs, CUDA events on s, a product
 // under 16 us repeated within a run; waits for s): us[f] microseconds.  C
@@ -51,6 +57,14 @@ bool gemm_pair_available();
 cudaError_t time_gemm_forms(const float* A, int lda, const float* B, int ldb, float* C, int ldc,
                             int M, int N, int K, bool fp16, void* scratch, cudaStream_t s,
                             const int* forms, int nforms, double* us, int64_t* kernels);
+
+// C -= A B with the pieces already formed (a3: 3 x M x K, b3: 3 x N x K bf16,
+// K a multiple of 64); gate[0] != 0 where an entry is out of their range (then
+// the CUDA-core form, from A and B); *skip != 0: nothing is done
+cudaError_t launch_gemm_split_operands(const uint16_t* a3, const uint16_t* b3, const float* A,
+                                       int lda, const float* B, int ldb, float* C, int ldc, int M,
+                                       int N, int K, const int* gate, const int* skip, int* err,
+                                       cudaStream_t s, int64_t* kernels);
 
 // Freivalds' check of C = A B for square N x N matrices with `nvec`
 // Rademacher vectors drawn from SplitMix64 (seed); tau_i = c u_eff sigma_i.

@@ -51,12 +51,29 @@ cudaError_t launch_lu_diag_inv(const float* LU, int n, float* inv, cudaStream_t 
 cudaError_t launch_residual(const float* A, int n, const double* b, const double* x, double* r,
                             double* norms, double thresh, unsigned long long* viol,
                             cudaStream_t s, Prof* prof);
-cudaError_t launch_anorm(const float* A, int n, double* norms, cudaStream_t s);   // norms[3]
+// norms[3] = |A|_inf; the 32-bit word at norms[6] becomes 1 when some row is
+// not diagonally dominant (both zero before)
+cudaError_t launch_anorm(const float* A, int n, double* norms, cudaStream_t s);
 // out[0] = sign of det A (0 if singular), out[1] = log |det A|, from the factors
 cudaError_t launch_lu_det(const float* LU, int n, const int* piv, double* out, cudaStream_t s,
                           Prof* prof);
 // x = d (init) or x += d; norms[1] = max|d|, norms[2] = max|x|, norms[4] = max|b|
 cudaError_t launch_update(double* x, const float* d, const double* b, int n, bool init,
                           double* norms, cudaStream_t s);
+
+
+// Elimination without interchanges (k_lu_diag.cu): the diagonal block at
+// (K, K) with its pivots, then the border of the outer block (KB = kLuOuter),
+// which also writes the trailing update's operands: L21 as a16 (rest x 128)
+// and U12 transposed as bt16 (rest x 128), bf16 or fp16 by prec, or for
+// SG_PREC_F32_SIMT three bf16 planes of each (*gate = 1: an entry out of their
+// range).  A pivot that is not its column's largest entry sets fail[0];
+// with fail[0] set the launches do nothing.  fail[1]: set by an update whose
+// waits gave up, turned into fail[0] by the next diagonal block.
+cudaError_t lu_diag_prepare();
+cudaError_t launch_lu_diag_block(float* LU, int n, int K, int KB, int* piv, int* fail,
+                                 cudaStream_t s);
+cudaError_t launch_lu_border(float* LU, int n, int K, int prec, void* a16, void* bt16, int* gate,
+                             int* fail, cudaStream_t s);
 
 }  // namespace sgk

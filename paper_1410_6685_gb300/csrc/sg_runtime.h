@@ -154,7 +154,8 @@ struct SchedState {
 
 // The blocked factorisation of one size and precision, captured once as a
 // CUDA graph over a workspace the context keeps (factors, pivots, the
-// panels' interchange lists, tensor-core operand copies).
+// panels' interchange lists, tensor-core operand copies); beside it, once a
+// matrix has asked for it, the form without interchanges.
 struct LuCache {
   int n = 0, prec = -1;
   void* base = nullptr;
@@ -166,6 +167,11 @@ struct LuCache {
   cudaGraphExec_t exec = nullptr;
   cudaStream_t cap = nullptr;
   int64_t kernels = 0;          // kernel launches in one replay
+  cudaGraphExec_t exec_diag = nullptr;   // every pivot on the diagonal (k_lu_diag.cu)
+  int64_t kernels_diag = 0;
+  int* gates = nullptr;         // its words per outer block: an entry the pieces do not take
+  int* moves = nullptr;         // the panels' interchange lists, then their counters
+  char* operands = nullptr;     // tensor-core operand copies
   void clear();
   ~LuCache() { clear(); }
 };

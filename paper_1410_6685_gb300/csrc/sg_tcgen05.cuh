@@ -273,5 +273,20 @@ __device__ __forceinline__ uint16_t to16(float v, bool fp16) {
   return *reinterpret_cast<const uint16_t*>(&x);
 }
 
+// x = p[0] + p[1] + p[2], each a bf16 (nearest to what is left); true when x
+// is outside the range in which the pieces and their products are exact
+__device__ __forceinline__ bool split3(float x, uint16_t (&p)[3]) {
+  const uint32_t e = (__float_as_uint(x) >> 23) & 0xFFu;
+  const __nv_bfloat16 h = __float2bfloat16_rn(x);
+  const float r1 = x - __bfloat162float(h);
+  const __nv_bfloat16 m = __float2bfloat16_rn(r1);
+  const float r2 = r1 - __bfloat162float(m);
+  const __nv_bfloat16 l = __float2bfloat16_rn(r2);
+  p[0] = *reinterpret_cast<const uint16_t*>(&h);
+  p[1] = *reinterpret_cast<const uint16_t*>(&m);
+  p[2] = *reinterpret_cast<const uint16_t*>(&l);
+  return x != 0.0f && (e < 127u - 50u || e > 127u + 54u);
+}
+
 }  // namespace tc
 }  // namespace sgk
