@@ -232,9 +232,12 @@ cudaError_t launch_filter_specialised(cudaKernel_t k, const float* x, float* out
   cudaError_t e = cudaMemsetAsync(
       scratch, 0, sizeof(FilterHdr) + (size_t)ntiles * sizeof(unsigned long long) + 256, s);
   if (e != cudaSuccess) return e;
-  (void)num_sms;   // one CTA per tile
   const void* fn = reinterpret_cast<const void*>(k);
-  const int grid = (int)ntiles;
+  // one CTA per tile, or the resident CTAs (one of them scans)
+  const int grid = filter_tile_scans(tile)
+                       ? (int)std::min<long long>((long long)ntiles + 1,
+                                                  (long long)num_sms * filter_tile_occupancy(tile))
+                       : (int)ntiles;
   FilterJitArgs a{};
   a.x = x;
   a.out = out;

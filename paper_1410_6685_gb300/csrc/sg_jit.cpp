@@ -416,25 +416,31 @@ extern "C" __global__ void __launch_bounds__(256) sg_batch(const BatchJitArgs a)
 }
 )SGJIT";
 
-// The filter (Table 2), specialised: a stable compaction, one CTA per tile
-// of 8192 items (or 2048 / 4096: SG_FQ = 2 / 4 float4s per thread, the
-// schedule chooser's filter family) taken from a ticket counter when the CTA starts (so tiles
-// start in ticket order and a look-back seldom waits on a tile that has not
-// started).  Thread t loads float4s t + 256 q (q < 8) of the tile straight
-// into registers; the order of kept items (round q, warp, lane, component)
-// comes from four ballots per round and a scan of the 64 (round, warp)
-// counts that every warp does itself.  The tile's aggregate is published at
-// once, every warp packs its kept items into shared memory (unpredicated
-// stores), warp 0 does the decoupled look-back over the tiles' words, 32
-// tiles per memory round trip, and the packed items are written out
-// contiguously.  Five CTAs per SM (48 registers, a few spilled).  Measured
-// at 2^28 items: 0.41 ms, against 0.48 / 0.49 / 0.55 ms at six / four / three
-// CTAs per SM (40 / 64 / 80 registers), 0.57 ms with 512 threads of 16
-// items, 0.65 ms with 4096-item tiles, 0.71 / 0.85 ms with
-// 64- / 128-tile look-back windows (more words re-polled while a predecessor
-// is unpublished), and 0.92 ms for a persistent form prefetching its next
-// tile by bulk copy (its tickets run ahead of the tiles it is still working
-// on, so look-backs wait on them).
+// The filter (Table 2), specialised: a stable compaction by tiles of 8192 items
+// (or 2048 / 4096: SG_FQ = 2 / 4 float4s per thread, the schedule chooser's
+// filter family) taken from a ticket counter, so that tiles start in ticket
+// order.  Thread t loads float4s t + 256 q of the tile straight into registers;
+// the order of kept items (round q, warp, lane, component) comes from one
+// warp scan of all rounds' counts and a scan of the (round, warp) counts that
+// every warp does itself.  The tile's count is published at once, every warp
+// packs its kept items into shared memory (unpredicated stores), and once the
+// tile's position is known the packed items are written out contiguously.
+//
+// 8192 items (SG_SCAN): persistent, four CTAs per SM (64 registers).  What
+// bounds a tile is the wait for its position: every earlier tile must have
+// been loaded and counted, and the slowest of the 600 in flight decides.  So a
+// CTA packs its tile, loads, counts and publishes the next one, and only then
+// asks for the first one's position; the next tile's ticket is taken early
+// and its memory prefetched into L2; and positions come from one warp (the
+// first ticket's) that sums the published counts, not from each tile's own
+// look-back over hundreds of words.  At 2^28 items, 37.5% kept: 266 us, 5.5 TB/s,
+// 0.81 of the copy rate (one CTA per tile with look-backs: 415 us; persistent
+// without the prefetch 309 us; three / five CTAs per SM 290 / 280 us; a whole CTA
+// scanning 269 us).
+//
+// 2048 and 4096 items: one CTA per tile; warp 0 does the decoupled look-back
+// over the tiles' words, 32 tiles per memory round trip.  They are faster
+// below a few hundred thousand items (7.7 against 9.1 us at 10^5).
 // Layouts below must match FilterResult (sg_internal.h) and FilterJitArgs
 // (sg_jit.h).
 const char* kTemplateFilter = R"SGJIT(
@@ -456,22 +462,69 @@ __device__ __forceinline__ void sg_st_relaxed(unsigned long long* p, unsigned lo
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-extern "C" __global__ void __launch_bounds__(256, SG_FMINB) sg_filter(const FilterJitArgs a) {
-  __shared__ __align__(16) float s_pack[SG_FT];
-  __shared__ float s_spare[256];
-  __shared__ unsigned s_cnt[SG_FQ * 8];
-  __shared__ unsigned s_tile;
-  __shared__ unsigned long long s_excl;
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const long long n = a.n;
-  unsigned lt;
-  asm("mov.u32 %0, %%lanemask_lt;" : "=r"(lt));
-  if (tid == 0) s_tile = atomicAdd(a.tile_ctr, 1u);
-  __syncthreads();
-  const unsigned t = s_tile;
-  const long long base = (long long)t * SG_FT;
-  const int valid = (int)(n - base < SG_FT ? n - base : SG_FT);
-  float v[4 * SG_FQ];
+#if SG_SCAN
+// The scanning warp: turns the tiles' aggregates, as they are published, into
+// exclusive prefixes in the same words: the leading published ones of a
+// window of 256 words per round trip, from the first tile without a prefix
+// on.  (A whole CTA with a window of 1024 and its barriers took twice as long
+// a round.)
+__device__ __forceinline__ void sg_scan_tiles(const FilterJitArgs& a) {
+  const unsigned lane = threadIdx.x & 31;
+  unsigned long long run = 0;
+  unsigned f = 0, spins = 0;
+  while (f < a.ntiles) {
+    unsigned long long wd[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const unsigned i = f + 32 * k + lane;
+      wd[k] = i < a.ntiles ? sg_ld_relaxed(&a.st[i]) : 0ull;
+    }
+    unsigned lead[8], c[8], incl[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const unsigned gap = ~__ballot_sync(0xffffffffu, wd[k] != 0ull);
+      lead[k] = gap ? (unsigned)(__ffs(gap) - 1) : 32u;
+      c[k] = incl[k] = lane < lead[k] ? (unsigned)(wd[k] & SG_CNT) : 0u;
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, incl[k], o);
+        if (lane >= o) incl[k] += y;
+      }
+    unsigned adv = 0;
+    bool open = true;   // every earlier word of the window is published
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (open && lane < lead[k])
+        sg_st_relaxed(&a.st[f + 32 * k + lane], SG_PRE | (run + (incl[k] - c[k])));
+      const unsigned tot = __shfl_sync(0xffffffffu, incl[k], 31);
+      if (open) {
+        run += tot;
+        adv += lead[k];
+      }
+      open = open && lead[k] == 32u;
+    }
+    f += adv;
+    if (adv) {
+      spins = 0;
+    } else if (++spins > a.spin_limit) {
+      if (lane == 0) atomicExch(&a.res->timeout, 1);
+      return;
+    }
+  }
+  if (lane == 0) a.res->count = (long long)run;
+}
+#endif
+
+// The thread's 4 SG_FQ items of the tile at `base` (16-byte loads straight into
+// registers where the tile is whole and aligned) and which of them are kept:
+// bit 4 q + l is component l of round q.
+__device__ __forceinline__ unsigned sg_load_tile(const FilterJitArgs& a, long long base,
+                                                 float (&v)[4 * SG_FQ]) {
+  const int tid = threadIdx.x;
+  const int valid = (int)(a.n - base < SG_FT ? a.n - base : SG_FT);
   if (valid == SG_FT && (((unsigned long long)(a.x + base)) & 15ull) == 0) {
 #pragma unroll
     for (int q = 0; q < SG_FQ; ++q) {
@@ -487,7 +540,6 @@ extern "C" __global__ void __launch_bounds__(256, SG_FMINB) sg_filter(const Filt
         v[4 * q + l] = li < valid ? a.x[base + li] : 0.0f;
       }
   }
-  // predicate on the thread's 32 items, masked to the valid ones
   unsigned keep = 0, vmask = 0;
 #pragma unroll
   for (int q = 0; q < SG_FQ; ++q) {
@@ -504,23 +556,39 @@ extern "C" __global__ void __launch_bounds__(256, SG_FMINB) sg_filter(const Filt
     const int rest = valid - 4 * (q * 256 + tid);
     vmask |= ((1u << min(max(rest, 0), 4)) - 1u) << (4 * q);
   }
-  keep &= vmask;
-  unsigned rbase[SG_FQ];
+  return keep & vmask;
+}
+
+// Kept items of the lanes below, per round (rbase), and of the whole warp, per
+// round (s_cnt[8 q + warp]): one warp scan of all rounds' counts, a byte each
+// (at most 128), instead of four ballots a round.
+__device__ __forceinline__ void sg_count_rounds(unsigned keep, unsigned (&rbase)[SG_FQ],
+                                                unsigned* s_cnt) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  unsigned pk[2] = {0u, 0u};
+#pragma unroll
+  for (int q = 0; q < SG_FQ; ++q)
+    pk[q / 4] |= (unsigned)__popc((keep >> (4 * q)) & 15u) << (8 * (q % 4));
+  unsigned in[2] = {pk[0], pk[1]};
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+    for (int h = 0; h < (SG_FQ + 3) / 4; ++h) {
+      const unsigned y = __shfl_up_sync(0xffffffffu, in[h], o);
+      if (lane >= o) in[h] += y;
+    }
 #pragma unroll
   for (int q = 0; q < SG_FQ; ++q) {
-    unsigned below = 0, cnt = 0;
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      const unsigned m = __ballot_sync(0xffffffffu, (keep >> (4 * q + l)) & 1u);
-      below += __popc(m & lt);
-      cnt += __popc(m);
-    }
-    rbase[q] = below;
-    if (lane == 0) s_cnt[q * 8 + w] = cnt;
+    rbase[q] = ((in[q / 4] - pk[q / 4]) >> (8 * (q % 4))) & 255u;
+    if (lane == 31) s_cnt[q * 8 + w] = (in[q / 4] >> (8 * (q % 4))) & 255u;
   }
-  __syncthreads();
-  // every warp scans the 8 SG_FQ (round, warp) counts, two per lane when
-  // there are 64
+}
+
+// Every warp scans the 8 SG_FQ (round, warp) counts (two per lane when there
+// are 64): rbase becomes each round's first position in the tile; returns the
+// tile's total.
+__device__ __forceinline__ unsigned sg_tile_ranks(const unsigned* s_cnt, unsigned (&rbase)[SG_FQ]) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #if SG_FQ == 8
   const unsigned c0 = s_cnt[2 * lane], c1 = s_cnt[2 * lane + 1];
 #else
@@ -532,25 +600,155 @@ extern "C" __global__ void __launch_bounds__(256, SG_FMINB) sg_filter(const Filt
     const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += y;
   }
-  const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
   const unsigned e0 = incl - c0 - c1;
-  const bool publish = (int)t != a.skip_tile;
-  if (tid == 0 && t > 0 && publish) sg_st_relaxed(&a.st[t], SG_AGG | total);
 #pragma unroll
   for (int q = 0; q < SG_FQ; ++q) {
     const int entry = q * 8 + w;
 #if SG_FQ == 8
-    unsigned r = __shfl_sync(0xffffffffu, (entry & 1) ? e0 + c0 : e0, entry >> 1) + rbase[q];
+    rbase[q] += __shfl_sync(0xffffffffu, (entry & 1) ? e0 + c0 : e0, entry >> 1);
 #else
-    unsigned r = __shfl_sync(0xffffffffu, e0, entry) + rbase[q];
+    rbase[q] += __shfl_sync(0xffffffffu, e0, entry);
 #endif
+  }
+  return __shfl_sync(0xffffffffu, incl, 31);
+}
+
+__device__ __forceinline__ void sg_pack(unsigned keep, const unsigned (&rbase)[SG_FQ],
+                                        const float (&v)[4 * SG_FQ], float* s_pack, float* s_spare) {
+#pragma unroll
+  for (int q = 0; q < SG_FQ; ++q) {
+    unsigned r = rbase[q];
 #pragma unroll
     for (int l = 0; l < 4; ++l) {
       const unsigned bit = (keep >> (4 * q + l)) & 1u;
-      *(bit ? s_pack + r : s_spare + tid) = v[4 * q + l];   // no predicated store
+      *(bit ? s_pack + r : s_spare + threadIdx.x) = v[4 * q + l];   // no predicated store
       r += bit;
     }
   }
+}
+
+// The packed items to their place in the result, with the folded
+// postcondition on each at its output position.
+__device__ __forceinline__ void sg_write_out(const FilterJitArgs& a, const float* s_pack,
+                                             unsigned total, unsigned long long gb) {
+#if SG_POST
+  unsigned long long bad = 0ull;   // ~(lowest violating position), 0: none
+#endif
+  for (unsigned i = threadIdx.x; i < total; i += 256) {
+    const unsigned long long pos = gb + i;
+    if (pos < (unsigned long long)a.n) {
+      const float kv = s_pack[i];
+      a.out[pos] = kv;
+#if SG_POST
+      float x[1], o[1];
+      x[0] = kv;
+      unsigned hit = 0u;
+      float rv = 0.0f;
+      bool rm = false;
+      sg_post(a, x, (long long)pos, o, hit, rv, rm);
+      if (!(rv != 0.0f) && ~pos > bad) bad = ~pos;
+#endif
+    }
+  }
+#if SG_POST
+#pragma unroll
+  for (int o2 = 16; o2 > 0; o2 >>= 1) {
+    const unsigned long long b2 = __shfl_xor_sync(0xffffffffu, bad, o2);
+    bad = b2 > bad ? b2 : bad;
+  }
+  if ((threadIdx.x & 31) == 0 && bad) atomicMax(&a.res->post_enc, bad);
+#endif
+}
+
+#if SG_SCAN
+extern "C" __global__ void __launch_bounds__(256, SG_FMINB) sg_filter(const FilterJitArgs a) {
+  __shared__ __align__(16) float s_pack[SG_FT];
+  __shared__ float s_spare[256];
+  __shared__ unsigned s_cnt[SG_FQ * 8];
+  __shared__ unsigned s_tile;
+  __shared__ unsigned long long s_excl;
+  const int tid = threadIdx.x;
+  if (tid == 0) s_tile = atomicAdd(a.tile_ctr, 1u);
+  __syncthreads();
+  unsigned t = s_tile;
+  if (t == 0) {   // the first ticket scans, the others are the tiles
+    if (tid < 32) sg_scan_tiles(a);
+    return;
+  }
+  --t;
+  // tile `pend` waits packed in shared memory, pend_total items, for its prefix
+  unsigned pend = 0xffffffffu, pend_total = 0u;
+  for (;;) {
+    const bool have = t < a.ntiles;
+    float v[4 * SG_FQ];
+    unsigned rbase[SG_FQ], keep = 0u, total = 0u;
+    if (have) {
+      keep = sg_load_tile(a, (long long)t * SG_FT, v);
+      sg_count_rounds(keep, rbase, s_cnt);
+    }
+    __syncthreads();
+    if (have) {
+      total = sg_tile_ranks(s_cnt, rbase);
+      if (tid == 0 && (int)t != a.skip_tile) sg_st_relaxed(&a.st[t], SG_AGG | total);
+      if (tid == 32) {
+        // the next tile, on its way into L2 while this one is finished
+        const unsigned nt = atomicAdd(a.tile_ctr, 1u) - 1u;
+        s_tile = nt;
+        const float* p = a.x + (long long)nt * SG_FT;
+        if ((long long)(nt + 1u) * SG_FT <= a.n && ((unsigned long long)p & 15ull) == 0)
+          asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(SG_FT * 4) : "memory");
+      }
+    }
+    if (pend != 0xffffffffu) {
+      if (tid == 0) {
+        // the tile's own word turns into its exclusive prefix
+        unsigned long long wd;
+        for (unsigned spins = 0;;) {
+          wd = sg_ld_relaxed(&a.st[pend]);
+          if ((wd & ~SG_CNT) == SG_PRE) break;
+          if (++spins > a.spin_limit ||
+              ((spins & 63u) == 0u && *(volatile const int*)&a.res->timeout)) {
+            atomicExch(&a.res->timeout, 1);
+            wd = ~0ull;
+            break;
+          }
+          if (spins > 32) __nanosleep(64);
+        }
+        s_excl = wd;
+      }
+      __syncthreads();
+      const unsigned long long wd = s_excl;
+      if (wd == ~0ull) return;   // no prefix: nothing is written
+      sg_write_out(a, s_pack, pend_total, wd & SG_CNT);
+    }
+    if (!have) return;
+    __syncthreads();
+    sg_pack(keep, rbase, v, s_pack, s_spare);
+    pend = t;
+    pend_total = total;
+    t = s_tile;
+  }
+}
+#else
+extern "C" __global__ void __launch_bounds__(256, SG_FMINB) sg_filter(const FilterJitArgs a) {
+  __shared__ __align__(16) float s_pack[SG_FT];
+  __shared__ float s_spare[256];
+  __shared__ unsigned s_cnt[SG_FQ * 8];
+  __shared__ unsigned s_tile;
+  __shared__ unsigned long long s_excl;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (tid == 0) s_tile = atomicAdd(a.tile_ctr, 1u);
+  __syncthreads();
+  const unsigned t = s_tile;
+  float v[4 * SG_FQ];
+  unsigned rbase[SG_FQ];
+  const unsigned keep = sg_load_tile(a, (long long)t * SG_FT, v);
+  sg_count_rounds(keep, rbase, s_cnt);
+  __syncthreads();
+  const unsigned total = sg_tile_ranks(s_cnt, rbase);
+  const bool publish = (int)t != a.skip_tile;
+  if (tid == 0 && t > 0 && publish) sg_st_relaxed(&a.st[t], SG_AGG | total);
+  sg_pack(keep, rbase, v, s_pack, s_spare);
   if (w == 0) {
     unsigned long long excl = 0;
     if (t == 0) {
@@ -590,36 +788,9 @@ extern "C" __global__ void __launch_bounds__(256, SG_FMINB) sg_filter(const Filt
     }
   }
   __syncthreads();
-  const unsigned long long gb = s_excl;
-#if SG_POST
-  unsigned long long bad = 0ull;   // ~(lowest violating position), 0: none
-#endif
-  for (unsigned i = tid; i < total; i += 256) {
-    const unsigned long long pos = gb + i;
-    if (pos < (unsigned long long)n) {
-      const float kv = s_pack[i];
-      a.out[pos] = kv;
-#if SG_POST
-      // the folded postcondition on the kept item at its output position
-      float x[1], o[1];
-      x[0] = kv;
-      unsigned hit = 0u;
-      float rv = 0.0f;
-      bool rm = false;
-      sg_post(a, x, (long long)pos, o, hit, rv, rm);
-      if (!(rv != 0.0f) && ~pos > bad) bad = ~pos;
-#endif
-    }
-  }
-#if SG_POST
-#pragma unroll
-  for (int o2 = 16; o2 > 0; o2 >>= 1) {
-    const unsigned long long b2 = __shfl_xor_sync(0xffffffffu, bad, o2);
-    bad = b2 > bad ? b2 : bad;
-  }
-  if (lane == 0 && bad) atomicMax(&a.res->post_enc, bad);
-#endif
+  sg_write_out(a, s_pack, total, s_excl);
 }
+#endif
 )SGJIT";
 
 // ---- body generation: symbolic execution of the postfix program -----------
@@ -883,12 +1054,12 @@ bool filter_source(const Prog& pred, int tile, std::string* src, std::string* lo
       return false;
     }
   }
-  // resident CTAs per SM the compiler plans for: 48 registers at 8192
+  // resident CTAs per SM the compiler plans for: 64 registers at 8192
   // items, 40 at 4096, 32 at 2048
   char defs[160];
   snprintf(defs, sizeof defs, "#define SG_MINMAX 0\n#define SG_FT %d\n#define SG_FQ %d\n"
-           "#define SG_FMINB %d\n#define SG_POST %d\n", tile, tile / 1024,
-           filter_tile_occupancy(tile), post ? 1 : 0);
+           "#define SG_FMINB %d\n#define SG_POST %d\n#define SG_SCAN %d\n", tile, tile / 1024,
+           filter_tile_occupancy(tile), post ? 1 : 0, filter_tile_scans(tile) ? 1 : 0);
   *src = std::string(defs) + kTemplateHead + body_fn(body) +
          (post ? body_fn(post_body, "sg_post") : std::string()) + kTemplateFilter;
   return true;
@@ -896,7 +1067,9 @@ bool filter_source(const Prog& pred, int tile, std::string* src, std::string* lo
 
 }  // namespace
 
-int filter_tile_occupancy(int tile) { return tile >= 8192 ? 5 : tile >= 4096 ? 6 : 8; }
+bool filter_tile_scans(int tile) { return tile >= 8192; }
+
+int filter_tile_occupancy(int tile) { return tile >= 8192 ? 4 : tile >= 4096 ? 6 : 8; }
 
 cudaKernel_t jit_filter_kernel(const Prog& pred, std::string* log, int tile, const Prog* post) {
   std::string src;

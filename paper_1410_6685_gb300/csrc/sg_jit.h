@@ -70,14 +70,17 @@ cudaKernel_t jit_stream_kernel(const Prog& pr, int nin, int nout, int npred, boo
                                bool minmax, uint32_t pred_exists, std::string* log);
 // the batched map -> for_all -> masked sum chain of one program (k_batch.cu)
 cudaKernel_t jit_batch_kernel(const Prog& pr, std::string* log);
-// the stable compaction of one predicate (one input slot), one CTA per
-// tile of `tile` items: 2048, 4096 or 8192 (k_filter.cu launches it)
+// the stable compaction of one predicate (one input slot), by
+// tiles of `tile` items: 2048, 4096 or 8192 (k_filter.cu launches it)
 // post: a for_all postcondition (one input slot) on the kept items, checked
 // as they are written (FilterResult::post_enc), or null
 cudaKernel_t jit_filter_kernel(const Prog& pred, std::string* log, int tile = kJitFilterTile,
                                const Prog* post = nullptr);
 // index of the postcondition's first constant in FilterJitArgs::cst
 inline int jit_filter_post_base(const Prog& pred) { return pred.nops + 1; }
+// whether that filter kernel is persistent, with a CTA of its own that forms
+// the tiles' prefixes (else one CTA per tile, and look-backs)
+bool filter_tile_scans(int tile);
 // resident CTAs per SM that filter kernel is compiled for
 int filter_tile_occupancy(int tile);
 // the smallest tile of the specialised filter (sizes its look-back scratch)
