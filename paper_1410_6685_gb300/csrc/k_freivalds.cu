@@ -320,7 +320,7 @@ cudaError_t launch_freivalds(const float* A, const float* B, const float* C, int
   return cudaGetLastError();
 }
 
-FrvFused frv_fused_layout(void* scratch, int N) {
+FrvFused frv_fused_layout(void* scratch, int N, int tile_c) {
   FrvFused f;
   char* p = static_cast<char*>(scratch);
   const size_t one = align256((size_t)N * sizeof(float4));
@@ -330,7 +330,7 @@ FrvFused frv_fused_layout(void* scratch, int N) {
   p += 3 * one;
   f.nsb = (N + kFrvStripeB - 1) / kFrvStripeB;
   f.nsa = (N + kFrvStripeA - 1) / kFrvStripeA;
-  f.nsc = (N + kFrvTileC - 1) / kFrvTileC;
+  f.nsc = (N + tile_c - 1) / tile_c;
   f.pb = reinterpret_cast<float*>(p);
   p += align256((size_t)f.nsb * N * 5 * sizeof(float));
   f.pzq = reinterpret_cast<float*>(p);
@@ -341,7 +341,7 @@ FrvFused frv_fused_layout(void* scratch, int N) {
   return f;
 }
 
-size_t frv_fused_scratch_bytes(int N) { return frv_fused_layout(nullptr, N).bytes; }
+size_t frv_fused_scratch_bytes(int N) { return frv_fused_layout(nullptr, N, kFrvMinTileC).bytes; }
 
 cudaError_t launch_frv_vectors(const FrvFused& f, int N, int nvec, unsigned long long seed,
                                cudaStream_t st) {

@@ -103,14 +103,6 @@ __device__ __forceinline__ uint64_t sdesc64(uint32_t saddr) {
   return d;
 }
 
-// true in one lane of a converged warp
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-               : "=r"(p));
-  return p != 0;
-}
-
 // Persistent, roles as in k_gemm_tc / k_gemm_tc2: warp 0 TMA producer, warps 1
 // and 10 MMA issuers, warps 2..9 epilogue (lane quarter warp % 4, column half
 // (warp - 2) / 4).  Chunks of all tiles are numbered in one sequence; chunk
@@ -348,94 +340,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (PAIR) cluster_sync();
 }
 
-// A (rows x cols, leading dimension lda) -> out[3][rows][Kp], zero padded
-__global__ void __launch_bounds__(256) k_split_rows(const float* __restrict__ A, int lda, int rows,
-                                                    int cols, int Kp, uint16_t* __restrict__ out,
-                                                    int* gate, int vec) {
-  const long long total = (long long)rows * (Kp / 8), plane = (long long)rows * Kp;
-  bool bad = false;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(t / (Kp / 8)), c0 = (int)(t % (Kp / 8)) * 8;
-    const float* src = A + (size_t)r * lda + c0;
-    float x[8];
-    if (vec && c0 + 8 <= cols) {
-      const float4 u = __ldcs(reinterpret_cast<const float4*>(src));
-      const float4 v = __ldcs(reinterpret_cast<const float4*>(src) + 1);
-      x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w;
-      x[4] = v.x; x[5] = v.y; x[6] = v.z; x[7] = v.w;
-    } else {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) x[j] = c0 + j < cols ? __ldcs(src + j) : 0.0f;
-    }
-    uint32_t w[3][4];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      uint16_t p[3];
-      bad |= split3(x[j], p);
-#pragma unroll
-      for (int z = 0; z < 3; ++z)
-        w[z][j >> 1] = (j & 1) ? w[z][j >> 1] | ((uint32_t)p[z] << 16) : (uint32_t)p[z];
-    }
-#pragma unroll
-    for (int z = 0; z < 3; ++z)
-      *reinterpret_cast<uint4*>(out + z * plane + (long long)r * Kp + c0) =
-          make_uint4(w[z][0], w[z][1], w[z][2], w[z][3]);
-  }
-  if (bad) *gate = 1;
-}
-
-// B (K x N, leading dimension ldb) -> out[3][N][Kp], transposed through a
-// 64 x 64 tile of shared memory: 16-byte loads along n, 16-byte stores along k
-__global__ void __launch_bounds__(256) k_split_transpose(const float* __restrict__ B, int ldb,
-                                                         int K, int N, int Kp,
-                                                         uint16_t* __restrict__ out, int* gate,
-                                                         int vec) {
-  __shared__ float t[64][65];
-  const int k0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  const long long plane = (long long)N * Kp;
-  float4 v[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int e = threadIdx.x + 256 * i, k = k0 + (e >> 4), n = n0 + (e & 15) * 4;
-    const float* src = B + (size_t)k * ldb + n;
-    if (vec && k < K && n + 4 <= N) {
-      v[i] = __ldcs(reinterpret_cast<const float4*>(src));
-    } else {
-      float x[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) x[j] = k < K && n + j < N ? __ldcs(src + j) : 0.0f;
-      v[i] = make_float4(x[0], x[1], x[2], x[3]);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int e = threadIdx.x + 256 * i, r = e >> 4, c = (e & 15) * 4;
-    t[r][c] = v[i].x; t[r][c + 1] = v[i].y; t[r][c + 2] = v[i].z; t[r][c + 3] = v[i].w;
-  }
-  __syncthreads();
-  bool bad = false;
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int e = threadIdx.x + 256 * i, nn = e >> 3, kc = (e & 7) * 8;
-    if (n0 + nn >= N) continue;
-    uint32_t w[3][4];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      uint16_t p[3];
-      bad |= split3(t[kc + j][nn], p);
-#pragma unroll
-      for (int z = 0; z < 3; ++z)
-        w[z][j >> 1] = (j & 1) ? w[z][j >> 1] | ((uint32_t)p[z] << 16) : (uint32_t)p[z];
-    }
-#pragma unroll
-    for (int z = 0; z < 3; ++z)
-      *reinterpret_cast<uint4*>(out + z * plane + (long long)(n0 + nn) * Kp + k0 + kc) =
-          make_uint4(w[z][0], w[z][1], w[z][2], w[z][3]);
-  }
-  if (bad) *gate = 1;
-}
-
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
     void* p = nullptr;
@@ -572,15 +476,11 @@ cudaError_t launch_gemm_split(const float* A, int lda, const float* B, int ldb, 
   int* gate = reinterpret_cast<int*>(p);   // [0] out of range, [1] a wait gave up
   uint16_t* a3 = reinterpret_cast<uint16_t*>(p + 256);
   uint16_t* b3 = reinterpret_cast<uint16_t*>(p + 256 + align256((size_t)M * Kp * 6));
-  const int va = lda % 4 == 0 && (uintptr_t)A % 16 == 0;
-  const int vb = ldb % 4 == 0 && (uintptr_t)B % 16 == 0;
   prof_begin(prof, "split_operands", s);
   cudaError_t e = cudaMemsetAsync(gate, 0, 8, s);
+  if (e == cudaSuccess)
+    e = launch_cast_operands<SG_PREC_F32_SIMT>(A, lda, B, ldb, M, N, K, Kp, a3, b3, gate, s);
   if (e != cudaSuccess) return e;
-  const long long ca = (long long)M * (Kp / 8);
-  k_split_rows<<<(int)std::min<long long>((ca + 255) / 256, 65535LL * 8), 256, 0, s>>>(
-      A, lda, M, K, Kp, a3, gate, va);
-  k_split_transpose<<<dim3((N + 63) / 64, Kp / 64), 256, 0, s>>>(B, ldb, K, N, Kp, b3, gate, vb);
   prof_end(prof, s);
   prof_begin(prof, "gemm_f32_split", s);
   if (form < 0) form = choose_form(M, N, K, nullptr);
@@ -588,7 +488,7 @@ cudaError_t launch_gemm_split(const float* A, int lda, const float* B, int ldb, 
                : launch_split<false>(form, a3, b3, Kp, C, ldc, M, N, K, gate, nullptr, gate + 1, s);
   prof_end(prof, s);
   if (e != cudaSuccess) return e;
-  *kernels += 4;
+  *kernels += 3;
   return launch_gemm_f32(A, lda, B, ldb, C, ldc, M, N, K, subtract, s, prof, gate);
 }
 

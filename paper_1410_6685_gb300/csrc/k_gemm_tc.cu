@@ -4,21 +4,22 @@
 // accumulation in tensor memory.
 //
 // Operands are first cast (and B transposed) into K-major 16-bit copies whose
-// K extent is padded to a multiple of 64.  The product runs on CTA pairs
-// (k_gemm_tc2, tcgen05 cta_group::2, 256 x 256 tiles, described there) where
-// the device schedules clusters of two, else on single CTAs (k_gemm_tc), each
-// computing a 128 x 256 tile of C:
-//   warp 0, one lane : TMA producer -- 2-D tiled bulk-tensor loads of a 128x64
-//                      A slice and a 256x64 B slice per stage (128-byte
-//                      swizzle, no multicast), completion on a "full" mbarrier;
-//   warp 1, one lane : MMA issuer -- four tcgen05.mma (M=128, N=256, K=16) per
-//                      stage, accumulator in 256 TMEM columns, tcgen05.commit
-//                      to the stage's "empty" mbarrier, and to "done" at the end;
+// K extent is padded to a multiple of 64, both in one launch.  The product runs
+// on CTA pairs (k_gemm_tc2, tcgen05 cta_group::2, 256 x 256 tiles, described
+// there) or on single CTAs (k_gemm_tc), each computing a 128 x 256, 128 x 128 or
+// 128 x 64 tile of C:
+//   warp 0, one lane : TMA producer -- 2-D tiled bulk-tensor loads of the A and
+//                      B slices of a 64-deep stage (128-byte swizzle, no
+//                      multicast), completion on a "full" mbarrier;
+//   warp 1           : MMA issuer (one elected lane) -- four tcgen05.mma (M=128,
+//                      N = the tile's, K=16) per stage, accumulators in TMEM,
+//                      tcgen05.commit to the stage's "empty" mbarrier, and to
+//                      "done" at the end;
 //   warp 2           : allocates / frees the tensor memory;
-//   all four warps   : epilogue -- tcgen05.ld of their 32 TMEM lanes (rows),
+//   warps 2..9       : epilogue -- tcgen05.ld of their 32 TMEM lanes (rows),
 //                      binary32 stores (or read-modify-write for C - A B).
-// Four pipeline stages of 48 KB.  Every mbarrier wait is bounded: on a
-// timeout the kernel raises an error flag and finishes without hanging.
+// Every mbarrier wait is bounded: on a timeout the kernel raises an error flag
+// and finishes without hanging.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -36,18 +37,14 @@ namespace {
 
 using namespace tc;
 
-constexpr int TM = 128, TN = 256, TK = 64, STAGES = 4;
-static_assert(kFrvTileC == TN / 2, "the fused check keeps one C r partial per epilogue warp's column half");
+constexpr int TM = 128, TN = 256, TK = 64;
 constexpr int A_BYTES = TM * TK * 2;            // 16 KB
-constexpr int B_BYTES = TN * TK * 2;            // 32 KB
-constexpr int STAGE_BYTES = A_BYTES + B_BYTES;  // 48 KB
 // Eight epilogue warps, two per quarter of the tensor memory's lanes, each
 // draining one 128-column half of a tile (with four, each alone on its SM
 // sub-partition, the dependent steps of the epilogue bounded short-K
 // products such as the elimination's updates)
 constexpr int kEpiWarps = 8;
 constexpr int kGemmThreads = 64 + 32 * kEpiWarps;   // producer, MMA issuer, epilogue
-constexpr int R_BYTES = kEpiWarps * (TN / 2) * 16;  // the fused check's r entries of each warp's half
 // The epilogue turns each 32 x 32 chunk (lane = row, from the tensor
 // memory) around in shared memory, 16 rows at a time, so that eight lanes
 // cover one row's 128 bytes: a warp's access touches 4 rows instead of 32,
@@ -55,32 +52,48 @@ constexpr int R_BYTES = kEpiWarps * (TN / 2) * 16;  // the fused check's r entri
 // g of row r sits at group g ^ (r & 7): conflict-free writes (lane = row)
 // and reads (eight lanes = one row).
 constexpr int T_BYTES = kEpiWarps * 16 * 32 * 4;    // one 16 x 32 buffer per epilogue warp
-constexpr int SMEM_BYTES =
-    STAGES * STAGE_BYTES + 1024 /*align*/ + 256 /*barriers*/ + R_BYTES + T_BYTES;
+// the fused check's r entries of each warp's column half
+constexpr int r_bytes(int tn) { return kEpiWarps * (tn / 2) * 16; }
+
+// The one-CTA form with TNv-column tiles: 64-deep stages, or 128-deep ones for
+// the narrower tiles (a stage's wait, commit and eight MMAs' issue take about as
+// long as the MMAs run; with four per stage the issuer fell behind), as many
+// as fit
+template <int TNv>
+struct One {
+  static constexpr int kSlices = TNv == 256 ? 1 : 2;
+  static constexpr int kBBytes = TNv * TK * 2;
+  static constexpr int kStageBytes = kSlices * (A_BYTES + kBBytes);
+  static constexpr int kRest = 1024 /*align*/ + 256 /*barriers*/ + r_bytes(TNv) + T_BYTES;
+  static constexpr int kFit = (232448 - kRest) / kStageBytes;
+  static constexpr int kStages = kFit < 8 ? kFit : 8;
+  static constexpr int kSmem = kStages * kStageBytes + kRest;
+};
+
 // instruction descriptor, kind::f16: D f32, A/B bf16 or f16, both K-major
-__host__ __device__ constexpr uint32_t idesc(bool fp16) {
+__host__ __device__ constexpr uint32_t idesc(bool fp16, int tn) {
   return (1u << 4) | ((fp16 ? 0u : 1u) << 7) | ((fp16 ? 0u : 1u) << 10) |
-         ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+         ((uint32_t)(tn >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
 }
 
 // The epilogue of one tile by one epilogue warp: tensor-memory lane quarter
-// q (rows m0q .. m0q + 31), column half hh (columns n0 + 128 hh .. + 127,
-// four 32-column chunks) of accumulator acc.  The warp releases the
+// q (rows m0q .. m0q + 31), column half hh (columns n0 + TNv / 2 hh on, TNv / 64
+// 32-column chunks) of accumulator acc.  The warp releases the
 // accumulator with one arrival on `tempty` (a cluster address when CL) once
 // its last chunk is read; the fused check's partial C r of its rows over its
 // half goes to column tile 2 bn + hh of frv_pw.  false: the wait for the
 // accumulator gave up.
-template <bool CL>
+template <bool CL, int TNv>
 __device__ __forceinline__ bool epilogue_tile(
     uint32_t tmem, int acc, int tl, uint32_t tfull, uint32_t tempty, int q, int hh, int m0q,
     int n0, int bn, float* __restrict__ C, int ldc, int M, int N, int subtract,
     const float4* __restrict__ frv_r, float4* __restrict__ frv_pw, int inj_row, int inj_col,
     float inj_delta, float4* s_rw, float* s_tw, int lane, int* err, volatile int* abort_flag) {
-  const int c0 = n0 + hh * (TN / 2);
+  const int c0 = n0 + hh * (TNv / 2);
   if (frv_r) {
     // each epilogue warp keeps its own copy, so no barrier spans the warps
     __syncwarp();
-    for (int j = lane; j < TN / 2; j += 32)
+    for (int j = lane; j < TNv / 2; j += 32)
       s_rw[j] = c0 + j < N ? frv_r[c0 + j] : make_float4(0.f, 0.f, 0.f, 0.f);
     __syncwarp();
   }
@@ -89,13 +102,13 @@ __device__ __forceinline__ bool epilogue_tile(
   const int row = m0q + lane;
   float4 wacc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
-  for (int c = 0; c < TN / 64; ++c) {
+  for (int c = 0; c < TNv / 64; ++c) {
     const int col0 = c0 + c * 32;
     float4 cv[8];
     if (subtract) load_c(C, ldc, M, N, m0q, col0, lane, cv);
     uint32_t r[32];
-    tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * TN + col0 - n0), r);
-    if (c == TN / 64 - 1) {
+    tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * TNv + col0 - n0), r);
+    if (c == TNv / 64 - 1) {
       // this warp's part of the accumulator is drained
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -134,13 +147,14 @@ __device__ __forceinline__ bool epilogue_tile(
 // Persistent kernel, one CTA per SM, tiles t = blockIdx.x + i * gridDim.x in
 // the grouped order of tile_coords:
 //   warp 0, one lane : TMA producer over all of the CTA's tiles;
-//   warp 1, one lane : MMA issuer; accumulators alternate between two
-//                      256-column halves of the 512 TMEM columns, so the
-//                      epilogue of one tile overlaps the main loop of the next;
+//   warp 1           : MMA issuer (one elected lane); two accumulators of the
+//                      tile's columns alternate, so the epilogue of one tile
+//                      overlaps the main loop of the next;
 //   warps 2..9       : epilogue, warp w reads TMEM lanes 32 (w % 4) .. + 31
-//                      and the 128-column half (w - 2) / 4 of the tile;
+//                      and the column half (w - 2) / 4 of the tile;
 //                      after draining an accumulator they release it to the
 //                      MMA issuer through an mbarrier.
+template <int TNv>
 __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc(const __grid_constant__ CUtensorMap ma,
                                                     const __grid_constant__ CUtensorMap mb,
                                                     float* __restrict__ C, int ldc, int M,
@@ -150,6 +164,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc(const __grid_consta
                                                     int inj_col, float inj_delta,
                                                      const int* skip) {
   if (skip && *skip != 0) return;   // written by earlier launches
+  constexpr int STAGES = One<TNv>::kStages, STAGE_BYTES = One<TNv>::kStageBytes;
+  constexpr int SL = One<TNv>::kSlices;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -160,12 +176,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc(const __grid_consta
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 5);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   float4* s_r = reinterpret_cast<float4*>(smem + STAGES * STAGE_BYTES + 256);
-  float* s_t = reinterpret_cast<float*>(smem + STAGES * STAGE_BYTES + 256 + R_BYTES);
+  float* s_t = reinterpret_cast<float*>(smem + STAGES * STAGE_BYTES + 256 + r_bytes(TNv));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nN = (N + TN - 1) / TN, nM = (M + TM - 1) / TM;
+  const int nN = (N + TNv - 1) / TNv, nM = (M + TM - 1) / TM;
   const int ntiles = nN * nM;
   const uint32_t tfull0 = smem_u32(&bars[2 * STAGES]), tempty0 = smem_u32(&bars[2 * STAGES + 2]);
   const uint32_t drain_bar = smem_u32(&bars[2 * STAGES + 4]);
+  const uint32_t full0 = smem_u32(bars), stage0 = smem_u32(smem);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < 2 * STAGES; ++s) mbar_init(smem_u32(&bars[s]), 1);
@@ -181,7 +198,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc(const __grid_consta
   if (warp == 2) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)),
-                 "r"(2 * TN)
+                 "r"(2 * TNv)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -198,7 +215,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc(const __grid_consta
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
         int bm, bn;
         tile_coords(t, nM, nN, &bm, &bn);
-        const int m0 = bm * TM, n0 = bn * TN;
+        const int m0 = bm * TM, n0 = bn * TNv;
         for (int kb = 0; kb < KB; ++kb, ++it) {
           const int s = it % STAGES;
           const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
@@ -210,49 +227,64 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc(const __grid_consta
           const uint32_t full = smem_u32(&bars[s]);
           mbar_expect_tx(full, STAGE_BYTES);
           const uint32_t a_dst = smem_u32(smem + s * STAGE_BYTES);
-          tma_load_2d(a_dst, &ma, kb * TK, m0, full);
-          tma_load_2d(a_dst + A_BYTES, &mb, kb * TK, n0, full);
+          // (past Kp a slice reads zeros)
+#pragma unroll
+          for (int u = 0; u < SL; ++u) {
+            tma_load_2d(a_dst + u * A_BYTES, &ma, (kb * SL + u) * TK, m0, full);
+            tma_load_2d(a_dst + SL * A_BYTES + u * One<TNv>::kBBytes, &mb, (kb * SL + u) * TK, n0,
+                        full);
+          }
         }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // MMA issuer
-      int it = 0, tl = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tl) {
-        const int acc = tl & 1;
-        if (tl >= 2 && !mbar_wait_ab(tempty0 + 8 * acc, (uint32_t)((tl >> 1) - 1) & 1u, err,
-                                     abort_flag))
-          break;
+    // MMA issuer: the whole warp runs the loop and one elected lane issues, so
+    // that the descriptors stay in uniform registers (from a lone diverged
+    // lane a tcgen05.mma takes 68 clocks to issue, longer than a 64-column one
+    // takes to run)
+    int it = 0, tl = 0, s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tl) {
+      const int acc = tl & 1;
+      ok = tl < 2 || mbar_wait_ab(tempty0 + 8 * acc, (uint32_t)((tl >> 1) - 1) & 1u, err,
+                                  abort_flag);
+      ok = __all_sync(0xffffffffu, ok);   // the lanes give up together
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t dacc = tmem + (uint32_t)(acc * TNv);
+      for (int kb = 0; kb < KB; ++kb, ++it) {
+        ok = __all_sync(0xffffffffu, mbar_wait_ab(full0 + 8 * s, ph, err, abort_flag));
+        if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t dacc = tmem + (uint32_t)(acc * TN);
-        for (int kb = 0; kb < KB; ++kb, ++it) {
-          const int s = it % STAGES;
-          const uint32_t ph = (uint32_t)(it / STAGES) & 1u;
-          if (!mbar_wait_ab(smem_u32(&bars[s]), ph, err, abort_flag)) {
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t a_base = smem_u32(smem + s * STAGE_BYTES);
-          const uint64_t da = sdesc(a_base), db = sdesc(a_base + A_BYTES);
+        const uint64_t da = sdesc(stage0 + (uint32_t)(s * STAGE_BYTES));
+        const uint64_t db = da + (uint64_t)(SL * A_BYTES >> 4);
+        if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < TK / 16; ++k) {
-            // advance 16 elements (32 bytes) along K inside the swizzled rows
-            umma(dacc, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), id, (kb | k) != 0);
-          }
-          umma_commit(smem_u32(&bars[STAGES + s]));
+          for (int u = 0; u < SL; ++u)
+#pragma unroll
+            for (int k = 0; k < TK / 16; ++k) {
+              // advance 16 elements (32 bytes) along K inside the swizzled rows
+              umma(dacc, da + (uint64_t)((u * A_BYTES >> 4) + k * 2),
+                   db + (uint64_t)((u * One<TNv>::kBBytes >> 4) + k * 2), id, (kb | u | k) != 0);
+            }
+          umma_commit(full0 + 8 * (STAGES + s));
+          if (kb == KB - 1) umma_commit(tfull0 + 8 * acc);
         }
-        if (ok) umma_commit(tfull0 + 8 * acc);
+        __syncwarp();
+        if (++s == STAGES) {
+          s = 0;
+          ph ^= 1u;
+        }
       }
-      // completes when every MMA issued above has finished
-      umma_commit(drain_bar);
     }
+    // completes when every MMA issued above has finished
+    if (elect_one()) umma_commit(drain_bar);
+    __syncwarp();
   } else {
     // epilogue warps 2..9: lane quarter warp % 4, column half (warp - 2) / 4
     const int q = warp & 3, hh = (warp - 2) >> 2;
-    float4* s_rw = s_r + (warp - 2) * (TN / 2);
+    float4* s_rw = s_r + (warp - 2) * (TNv / 2);
     float* s_tw = s_t + (warp - 2) * 16 * 32;
     int tl = 0;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++tl) {
@@ -262,10 +294,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc(const __grid_consta
       if (subtract && t + (int)gridDim.x < ntiles) {
         int bm2, bn2;
         tile_coords(t + (int)gridDim.x, nM, nN, &bm2, &bn2);
-        prefetch_c_row(C, ldc, M, N, bm2 * TM + q * 32 + lane, bn2 * TN + hh * (TN / 2), TN / 2);
+        prefetch_c_row(C, ldc, M, N, bm2 * TM + q * 32 + lane, bn2 * TNv + hh * (TNv / 2), TNv / 2);
       }
-      if (!epilogue_tile<false>(tmem, acc, tl, tfull0 + 8 * acc, tempty0 + 8 * acc, q, hh,
-                                bm * TM + q * 32, bn * TN, bn, C, ldc, M, N, subtract, frv_r,
+      if (!epilogue_tile<false, TNv>(tmem, acc, tl, tfull0 + 8 * acc, tempty0 + 8 * acc, q, hh,
+                                bm * TM + q * 32, bn * TNv, bn, C, ldc, M, N, subtract, frv_r,
                                 frv_pw, inj_row, inj_col, inj_delta, s_rw, s_tw, lane, err,
                                 abort_flag))
         break;
@@ -276,7 +308,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc(const __grid_consta
     // every MMA has completed before the tensor memory is released
     mbar_wait(drain_bar, 0, err);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * TN)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * TNv)
                  : "memory");
   }
 }
@@ -299,7 +331,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc(const __grid_consta
 // Six stages of 32 KB.  Every mbarrier wait is bounded, as in k_gemm_tc.
 constexpr int TM2 = 256, TH = 128, STAGES2 = 6;
 constexpr int STAGE2_BYTES = TH * TK * 2 * 2;   // 128 A rows + 128 B rows
-constexpr int SMEM2_BYTES = STAGES2 * STAGE2_BYTES + 1024 + 256 + R_BYTES + T_BYTES;
+constexpr int SMEM2_BYTES = STAGES2 * STAGE2_BYTES + 1024 + 256 + r_bytes(TN) + T_BYTES;
 
 __host__ __device__ constexpr uint32_t idesc2(bool fp16) {
   return (1u << 4) | ((fp16 ? 0u : 1u) << 7) | ((fp16 ? 0u : 1u) << 10) |
@@ -324,7 +356,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc2(const __grid_const
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES2 + 5);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   float4* s_r = reinterpret_cast<float4*>(smem + STAGES2 * STAGE2_BYTES + 256);
-  float* s_t = reinterpret_cast<float*>(smem + STAGES2 * STAGE2_BYTES + 256 + R_BYTES);
+  float* s_t = reinterpret_cast<float*>(smem + STAGES2 * STAGE2_BYTES + 256 + r_bytes(TN));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
   const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
@@ -332,6 +364,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc2(const __grid_const
   const int ntiles = nN * nM;
   const uint32_t tfull0 = smem_u32(&bars[2 * STAGES2]), tempty0 = smem_u32(&bars[2 * STAGES2 + 2]);
   const uint32_t drain_bar = smem_u32(&bars[2 * STAGES2 + 4]);
+  const uint32_t full0 = smem_u32(bars), stage0 = smem_u32(smem);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES2; ++s) {
@@ -384,35 +417,47 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc2(const __grid_const
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
-      int it = 0, tl = 0;
-      bool ok = true;
-      for (int t = pair; t < ntiles && ok; t += npairs, ++tl) {
-        const int acc = tl & 1;
-        if (tl >= 2 && !mbar_wait_ab(tempty0 + 8 * acc, (uint32_t)((tl >> 1) - 1) & 1u, err,
-                                     abort_flag))
-          break;
+    // MMA issuer: the whole warp runs the loop and one elected lane issues, so
+    // that the descriptors stay in uniform registers (from a lone diverged
+    // lane a tcgen05.mma takes 68 clocks to issue, longer than a 64-column one
+    // takes to run)
+    if (rank == 0) {
+    int it = 0, tl = 0, s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int t = pair; t < ntiles && ok; t += npairs, ++tl) {
+      const int acc = tl & 1;
+      ok = tl < 2 || mbar_wait_ab(tempty0 + 8 * acc, (uint32_t)((tl >> 1) - 1) & 1u, err,
+                                  abort_flag);
+      ok = __all_sync(0xffffffffu, ok);   // the lanes give up together
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t dacc = tmem + (uint32_t)(acc * TN);
+      for (int kb = 0; kb < KB; ++kb, ++it) {
+        ok = __all_sync(0xffffffffu, mbar_wait_ab(full0 + 8 * s, ph, err, abort_flag));
+        if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t dacc = tmem + (uint32_t)(acc * TN);
-        for (int kb = 0; kb < KB; ++kb, ++it) {
-          const int s = it % STAGES2;
-          const uint32_t ph = (uint32_t)(it / STAGES2) & 1u;
-          if (!mbar_wait_ab(smem_u32(&bars[s]), ph, err, abort_flag)) {
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t a_base = smem_u32(smem + s * STAGE2_BYTES);
-          const uint64_t da = sdesc(a_base), db = sdesc(a_base + TH * TK * 2);
+        const uint64_t da = sdesc(stage0 + (uint32_t)(s * STAGE2_BYTES));
+        const uint64_t db = da + (uint64_t)(TH * TK * 2 >> 4);
+        if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < TK / 16; ++k)
+          for (int k = 0; k < TK / 16; ++k) {
+            // advance 16 elements (32 bytes) along K inside the swizzled rows
             umma2(dacc, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), id, (kb | k) != 0);
-          umma_commit_pair(smem_u32(&bars[STAGES2 + s]));
+          }
+          umma_commit_pair(full0 + 8 * (STAGES2 + s));
+          if (kb == KB - 1) umma_commit_pair(tfull0 + 8 * acc);
         }
-        if (ok) umma_commit_pair(tfull0 + 8 * acc);
+        __syncwarp();
+        if (++s == STAGES2) {
+          s = 0;
+          ph ^= 1u;
+        }
       }
-      // completes, in both CTAs, when every MMA issued above has finished
-      umma_commit_pair(drain_bar);
+    }
+    // completes, in both CTAs, when every MMA issued above has finished
+    if (elect_one()) umma_commit_pair(drain_bar);
+    __syncwarp();
     }
   } else {
     // epilogue warps 2..9: lane quarter warp % 4, column half (warp - 2) / 4
@@ -431,7 +476,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc2(const __grid_const
         prefetch_c_row(C, ldc, M, N, bm2 * TM2 + (int)rank * TH + q * 32 + lane,
                        bn2 * TN + hh * (TN / 2), TN / 2);
       }
-      if (!epilogue_tile<true>(tmem, acc, tl, tfull0 + 8 * acc, tempty_leader + 8 * acc, q, hh,
+      if (!epilogue_tile<true, TN>(tmem, acc, tl, tfull0 + 8 * acc, tempty_leader + 8 * acc, q, hh,
                                bm * TM2 + (int)rank * TH + q * 32, bn * TN, bn, C, ldc, M, N,
                                subtract, frv_r, frv_pw, inj_row, inj_col, inj_delta, s_rw, s_tw,
                                lane, err, abort_flag))
@@ -447,65 +492,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc2(const __grid_const
   }
   // neither CTA leaves while the other may still signal its barriers
   cluster_sync();
-}
-
-// binary32 (rows x cols, leading dim ld) -> 16-bit rows x Kp, zero padded
-template <bool FP16>
-__global__ void k_cast_rows(const float* __restrict__ A, int lda, int rows, int cols, int Kp,
-                            void* out) {
-  const long long total = (long long)rows * (Kp / 8);
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(t / (Kp / 8));
-    const int c0 = (int)(t % (Kp / 8)) * 8;
-    const float* src = A + (size_t)r * lda + c0;
-    uint16_t h[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float v = (c0 + j < cols) ? src[j] : 0.0f;
-      if (FP16) {
-        const __half x = __float2half_rn(v);
-        h[j] = *reinterpret_cast<const uint16_t*>(&x);
-      } else {
-        const __nv_bfloat16 x = __float2bfloat16_rn(v);
-        h[j] = *reinterpret_cast<const uint16_t*>(&x);
-      }
-    }
-    uint4 pk;
-    pk.x = h[0] | ((uint32_t)h[1] << 16);
-    pk.y = h[2] | ((uint32_t)h[3] << 16);
-    pk.z = h[4] | ((uint32_t)h[5] << 16);
-    pk.w = h[6] | ((uint32_t)h[7] << 16);
-    reinterpret_cast<uint4*>(out)[t] = pk;
-  }
-}
-
-// B (K x N, leading dim ldb) -> Bt (N x Kp) 16-bit, transposed via 32x32 tiles
-template <bool FP16>
-__global__ void k_cast_transpose(const float* __restrict__ B, int ldb, int K, int N, int Kp,
-                                 uint16_t* out) {
-  __shared__ float t[32][33];
-  const int k0 = blockIdx.y * 32, n0 = blockIdx.x * 32;
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const int k = k0 + i, n = n0 + threadIdx.x;
-    t[i][threadIdx.x] = (k < K && n < N) ? B[(size_t)k * ldb + n] : 0.0f;
-  }
-  __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const int n = n0 + i, k = k0 + threadIdx.x;
-    if (n < N && k < Kp) {
-      const float v = t[threadIdx.x][i];
-      uint16_t h;
-      if (FP16) {
-        const __half x = __float2half_rn(v);
-        h = *reinterpret_cast<const uint16_t*>(&x);
-      } else {
-        const __nv_bfloat16 x = __float2bfloat16_rn(v);
-        h = *reinterpret_cast<const uint16_t*>(&x);
-      }
-      out[(size_t)n * Kp + k] = h;
-    }
-  }
 }
 
 // Square B (N x N) -> Bt (N x Kp) 16-bit, with the fused Freivalds partial
@@ -707,19 +693,16 @@ bool make_map(CUtensorMap* m, const void* base, int rows, int Kp, int box_rows, 
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// one CTA per SM (the pipeline's shared memory allows no second), at most
-// one per tile
-int persistent_grid(int M, int N) {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
+// one CTA per SM (the pipeline's shared memory allows no second)
+int sm_count() {
+  static const int sms = [] {
+    int dev = 0, v = 0;
     cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        sms <= 0)
-      sms = 1;
-  }
-  const long long tiles = (long long)((M + TM - 1) / TM) * ((N + TN - 1) / TN);
-  return (int)std::max<long long>(1, std::min<long long>(tiles, sms));
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
+      v = 1;
+    return v;
+  }();
+  return sms;
 }
 
 // the CTA-pair kernel where the device schedules clusters of two with its
@@ -749,6 +732,42 @@ bool use_pair() {
   return v == 1;
 }
 
+bool takes_pair(int form) { return form != 1 && !portable_kernels() && use_pair(); }
+
+// Columns of the one-CTA form's tiles: the width with the shortest estimate,
+// waves of tiles times (64-deep slices, and the tile's start and store).
+// Measured per slice: 0.18 us (64 columns), 0.24 us (128), 0.41 us (256); the narrow
+// tiles are bound by their operands' shared-memory traffic but fill the chip
+// sooner: 1024^3 12.2 / 12.2 / 16.9 us, 1537 x 1023 x 2049 22.2 / 17.4 / 22.9 us (a
+// pair's 256 x 256 tiles 22.2 us), 2048^3 34.6 / 25.2 / 23.2 us, 3000 x 300 x 8000
+// 32.4 / 36.5 / 51 us.
+int one_cta_columns(int M, int N, int Kp) {
+  const double c = Kp / TK;
+  auto us = [&](int tn, double per_stage, double per_tile) {
+    const long long t = (long long)((M + TM - 1) / TM) * ((N + tn - 1) / tn);
+    return (double)((t + sm_count() - 1) / sm_count()) * (per_stage * c + per_tile);
+  };
+  const double t64 = us(64, 0.18, 1.0), t128 = us(128, 0.24, 1.5), t256 = us(256, 0.41, 2.5);
+  return t64 <= t128 && t64 <= t256 ? 64 : t128 <= t256 ? 128 : 256;
+}
+
+template <int TNv>
+cudaError_t launch_one(const CUtensorMap& ma, const uint16_t* bt16, int Kp, bool fp16, float* C,
+                       int ldc, int M, int N, bool subtract, int* err, const float4* frv_r,
+                       float4* frv_pw, int inj_row, int inj_col, float inj_delta, cudaStream_t s,
+                       const int* skip) {
+  CUtensorMap mb;
+  if (!make_map(&mb, bt16, N, Kp, TNv, fp16)) return cudaErrorInvalidValue;
+  const cudaError_t e = cudaFuncSetAttribute(
+      k_gemm_tc<TNv>, cudaFuncAttributeMaxDynamicSharedMemorySize, One<TNv>::kSmem);
+  if (e != cudaSuccess) return e;
+  const long long tiles = (long long)((M + TM - 1) / TM) * ((N + TNv - 1) / TNv);
+  k_gemm_tc<TNv><<<(int)std::min<long long>(tiles, sm_count()), kGemmThreads, One<TNv>::kSmem, s>>>(
+      ma, mb, C, ldc, M, N, (Kp / TK + One<TNv>::kSlices - 1) / One<TNv>::kSlices, idesc(fp16, TNv), subtract ? 1 : 0, err, frv_r, frv_pw,
+      inj_row, inj_col, inj_delta, skip);
+  return cudaGetLastError();
+}
+
 // C (+)= A16 Bt16^T on the tensor cores: the CTA-pair kernel (form 2, or 0
 // where the device schedules pairs), else the one-CTA kernel
 cudaError_t launch_product(const uint16_t* a16, const uint16_t* bt16, int Kp, bool fp16, float* C,
@@ -757,11 +776,11 @@ cudaError_t launch_product(const uint16_t* a16, const uint16_t* bt16, int Kp, bo
                            cudaStream_t s, int form, const int* skip = nullptr) {
   CUtensorMap ma, mb;
   if (!make_map(&ma, a16, M, Kp, TM, fp16)) return cudaErrorInvalidValue;
-  if (form != 1 && !portable_kernels() && use_pair()) {
+  if (takes_pair(form)) {
     if (!make_map(&mb, bt16, N, Kp, TH, fp16)) return cudaErrorInvalidValue;
     const long long tiles = (long long)((M + TM2 - 1) / TM2) * ((N + TN - 1) / TN);
     const int pairs = (int)std::max<long long>(
-        1, std::min<long long>(tiles, persistent_grid(1 << 30, TN) / 2));   // SMs / 2
+        1, std::min<long long>(tiles, sm_count() / 2));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * pairs);
     cfg.blockDim = dim3(kGemmThreads);
@@ -778,19 +797,14 @@ cudaError_t launch_product(const uint16_t* a16, const uint16_t* bt16, int Kp, bo
                               subtract ? 1 : 0, err, frv_r, frv_pw, inj_row, inj_col, inj_delta,
                               skip);
   }
-  static bool attr_done = false;
-  if (!attr_done) {
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         SMEM_BYTES);
-    if (e != cudaSuccess) return e;
-    attr_done = true;
+  switch (one_cta_columns(M, N, Kp)) {
+    case 64: return launch_one<64>(ma, bt16, Kp, fp16, C, ldc, M, N, subtract, err, frv_r, frv_pw,
+                                   inj_row, inj_col, inj_delta, s, skip);
+    case 128: return launch_one<128>(ma, bt16, Kp, fp16, C, ldc, M, N, subtract, err, frv_r,
+                                     frv_pw, inj_row, inj_col, inj_delta, s, skip);
+    default: return launch_one<256>(ma, bt16, Kp, fp16, C, ldc, M, N, subtract, err, frv_r, frv_pw,
+                                    inj_row, inj_col, inj_delta, s, skip);
   }
-  if (!make_map(&mb, bt16, N, Kp, TN, fp16)) return cudaErrorInvalidValue;
-  k_gemm_tc<<<persistent_grid(M, N), kGemmThreads, SMEM_BYTES, s>>>(ma, mb, C, ldc, M, N, Kp / TK,
-                                                           idesc(fp16), subtract ? 1 : 0, err,
-                                                           frv_r, frv_pw, inj_row, inj_col,
-                                                           inj_delta, skip);
-  return cudaGetLastError();
 }
 
 }  // namespace
@@ -803,7 +817,6 @@ bool portable_kernels() { return g_portable; }
 
 void gemm_tc_prepare() {
   use_pair();
-  cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
   cudaGetLastError();
 }
 
@@ -817,18 +830,12 @@ size_t gemm_tc_scratch_bytes(int M, int N, int K) {
 namespace {
 
 // the bf16 / fp16 operand copies: A by rows, B transposed (K padded to Kp)
-void cast_operands(const float* A, int lda, const float* B, int ldb, int M, int N, int K, int Kp,
-                   bool fp16, uint16_t* a16, uint16_t* bt16, cudaStream_t s) {
-  const long long ca = (long long)M * (Kp / 8);
-  const int ga = (int)std::min<long long>((ca + 255) / 256, 65535LL * 8);
-  dim3 gt((N + 31) / 32, (Kp + 31) / 32), bt(32, 8);
-  if (fp16) {
-    k_cast_rows<true><<<ga, 256, 0, s>>>(A, lda, M, K, Kp, a16);
-    k_cast_transpose<true><<<gt, bt, 0, s>>>(B, ldb, K, N, Kp, bt16);
-  } else {
-    k_cast_rows<false><<<ga, 256, 0, s>>>(A, lda, M, K, Kp, a16);
-    k_cast_transpose<false><<<gt, bt, 0, s>>>(B, ldb, K, N, Kp, bt16);
-  }
+cudaError_t cast_operands(const float* A, int lda, const float* B, int ldb, int M, int N, int K,
+                          int Kp, bool fp16, uint16_t* a16, uint16_t* bt16, cudaStream_t s) {
+  return fp16 ? launch_cast_operands<SG_PREC_F16_TC>(A, lda, B, ldb, M, N, K, Kp, a16, bt16,
+                                                     nullptr, s)
+              : launch_cast_operands<SG_PREC_BF16_TC>(A, lda, B, ldb, M, N, K, Kp, a16, bt16,
+                                                      nullptr, s);
 }
 
 }  // namespace
@@ -842,10 +849,10 @@ cudaError_t time_gemm_forms(const float* A, int lda, const float* B, int ldb, fl
   int* err = reinterpret_cast<int*>(p);
   uint16_t* a16 = reinterpret_cast<uint16_t*>(p + 256);
   uint16_t* bt16 = reinterpret_cast<uint16_t*>(p + 256 + align256((size_t)M * Kp * 2));
-  cast_operands(A, lda, B, ldb, M, N, K, Kp, fp16, a16, bt16, s);
-  *kernels += 2;
+  cudaError_t e = cast_operands(A, lda, B, ldb, M, N, K, Kp, fp16, a16, bt16, s);
+  *kernels += 1;
   cudaEvent_t ev[2] = {nullptr, nullptr};
-  cudaError_t e = cudaEventCreate(&ev[0]);
+  if (e == cudaSuccess) e = cudaEventCreate(&ev[0]);
   if (e == cudaSuccess) e = cudaEventCreate(&ev[1]);
   for (int f = 0; f < nforms && e == cudaSuccess; ++f) {
     // a warm-up, then the better of two timed runs; a product shorter than
@@ -891,13 +898,14 @@ cudaError_t launch_gemm_tc(const float* A, int lda, const float* B, int ldb, flo
   uint16_t* a16 = reinterpret_cast<uint16_t*>(p + 256);
   uint16_t* bt16 = reinterpret_cast<uint16_t*>(p + 256 + align256((size_t)M * Kp * 2));
   prof_begin(prof, "cast_operands", s);
-  cast_operands(A, lda, B, ldb, M, N, K, Kp, fp16, a16, bt16, s);
+  cudaError_t e = cast_operands(A, lda, B, ldb, M, N, K, Kp, fp16, a16, bt16, s);
   prof_end(prof, s);
+  if (e != cudaSuccess) return e;
   prof_begin(prof, fp16 ? "gemm_tc_f16" : "gemm_tc_bf16", s);
-  const cudaError_t e = launch_product(a16, bt16, Kp, fp16, C, ldc, M, N, subtract, err, nullptr,
+  e = launch_product(a16, bt16, Kp, fp16, C, ldc, M, N, subtract, err, nullptr,
                                        nullptr, inj_row, inj_col, inj_delta, s, form);
   prof_end(prof, s);
-  *kernels += 3;
+  *kernels += 2;
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -920,7 +928,9 @@ cudaError_t launch_gemm_tc_checked(const float* A, const float* B, float* C, int
   int* err = reinterpret_cast<int*>(p);
   uint16_t* a16 = reinterpret_cast<uint16_t*>(p + 256);
   uint16_t* bt16 = reinterpret_cast<uint16_t*>(p + 256 + align256((size_t)N * Kp * 2));
-  const FrvFused f = frv_fused_layout(p + gemm_tc_scratch_bytes(N, N, N), N);
+  // one C r partial per epilogue warp's half of a tile
+  const FrvFused f = frv_fused_layout(p + gemm_tc_scratch_bytes(N, N, N), N,
+                                      (takes_pair(form) ? TN : one_cta_columns(N, N, Kp)) / 2);
   prof_begin(prof, "cast_operands", s);
   cudaError_t e = launch_frv_vectors(f, N, nvec, seed, s);
   if (e != cudaSuccess) return e;

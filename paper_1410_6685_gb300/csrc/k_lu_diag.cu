@@ -203,29 +203,6 @@ __global__ void __launch_bounds__(kDiagThreads) k_lu_diag_block(float* __restric
   if (bad) *fail = 1;
 }
 
-// eight consecutive entries as the update's operands: bf16, fp16, or the three
-// bf16 pieces in planes `plane` apart (true: an entry they do not take)
-template <int PREC>
-__device__ __forceinline__ bool store_operand(uint16_t* dst, size_t plane, const float (&v)[8]) {
-  bool bad = false;
-  uint32_t h[3][4];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    uint16_t p[3];
-    if (PREC == SG_PREC_F32_SIMT)
-      bad |= tc::split3(v[j], p);
-    else
-      p[0] = tc::to16(v[j], PREC == SG_PREC_F16_TC);
-#pragma unroll
-    for (int z = 0; z < (PREC == SG_PREC_F32_SIMT ? 3 : 1); ++z)
-      h[z][j >> 1] = (j & 1) ? h[z][j >> 1] | ((uint32_t)p[z] << 16) : (uint32_t)p[z];
-  }
-#pragma unroll
-  for (int z = 0; z < (PREC == SG_PREC_F32_SIMT ? 3 : 1); ++z)
-    *reinterpret_cast<uint4*>(dst + z * plane) = make_uint4(h[z][0], h[z][1], h[z][2], h[z][3]);
-  return bad;
-}
-
 // The outer block's border.  The first CTAs take 64 rows each of A21 (L21 =
 // A21 U11^-1), the others 64 columns each of A12 (U12 = L11^-1 A12); both hold
 // the whole factored diagonal block in shared memory and go through it by 32
@@ -342,7 +319,7 @@ __global__ void __launch_bounds__(kBorderThreads, 2)
       float v[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = X[r * kS + c + j];
-      if (r < cnt) out |= store_operand<PREC>(a16 + (size_t)(first - K - kNB + r) * kNB + c, plane, v);
+      if (r < cnt) out |= tc::store_operand<PREC>(a16 + (size_t)(first - K - kNB + r) * kNB + c, plane, v);
     }
     if (bad) *fail = 1;
   } else {
@@ -355,7 +332,7 @@ __global__ void __launch_bounds__(kBorderThreads, 2)
       float v[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = X[(k + j) * kXS + c];
-      if (c < cnt) out |= store_operand<PREC>(bt16 + (size_t)(first - K - kNB + c) * kNB + k, plane, v);
+      if (c < cnt) out |= tc::store_operand<PREC>(bt16 + (size_t)(first - K - kNB + c) * kNB + k, plane, v);
     }
   }
   if (PREC == SG_PREC_F32_SIMT && out) *gate = 1;

@@ -83,11 +83,11 @@ cudaError_t launch_freivalds(const float* A, const float* B, const float* C, int
 // matrices: the cast of B also forms the partial sums of B r and |B_k|^2,
 // the cast of A those of A (B r) and (A.A) t, and the GEMM epilogue those of
 // C r, so the check reads no matrix a second time.  Partial sums are over
-// column stripes (kFrvStripeB of B, kFrvStripeA of A, kFrvTileC of C) and are
+// column stripes (kFrvStripeB of B, kFrvStripeA of A, tile_c of C) and are
 // added in a fixed order by the final per-row test.
 constexpr int kFrvStripeB = 512;
 constexpr int kFrvStripeA = 1024;
-constexpr int kFrvTileC = 128;
+constexpr int kFrvMinTileC = 32;
 struct FrvFused {
   float4* r4;      // [N] the nvec Rademacher vectors, entry j of each
   float4* br4;     // [N] B r
@@ -98,7 +98,7 @@ struct FrvFused {
   int nsb, nsa, nsc;
   size_t bytes;
 };
-FrvFused frv_fused_layout(void* scratch, int N);
+FrvFused frv_fused_layout(void* scratch, int N, int tile_c);
 size_t frv_fused_scratch_bytes(int N);
 cudaError_t launch_frv_vectors(const FrvFused& f, int N, int nvec, unsigned long long seed,
                                cudaStream_t st);

@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "safegpu.h"
+
 namespace sgk {
 namespace tc {
 
@@ -273,6 +275,14 @@ __device__ __forceinline__ uint16_t to16(float v, bool fp16) {
   return *reinterpret_cast<const uint16_t*>(&x);
 }
 
+// true in one lane of a converged warp
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(p));
+  return p != 0;
+}
+
 // x = p[0] + p[1] + p[2], each a bf16 (nearest to what is left); true when x
 // is outside the range in which the pieces and their products are exact
 __device__ __forceinline__ bool split3(float x, uint16_t (&p)[3]) {
@@ -286,6 +296,108 @@ __device__ __forceinline__ bool split3(float x, uint16_t (&p)[3]) {
   p[1] = *reinterpret_cast<const uint16_t*>(&m);
   p[2] = *reinterpret_cast<const uint16_t*>(&l);
   return x != 0.0f && (e < 127u - 50u || e > 127u + 54u);
+}
+
+// eight consecutive entries as a product's operands (PREC: an sg_precision):
+// bf16, fp16, or the three bf16 pieces in planes `plane` apart (true: an entry they do not take)
+template <int PREC>
+__device__ __forceinline__ bool store_operand(uint16_t* dst, size_t plane, const float (&v)[8]) {
+  bool bad = false;
+  uint32_t h[3][4];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    uint16_t p[3];
+    if (PREC == SG_PREC_F32_SIMT)
+      bad |= split3(v[j], p);
+    else
+      p[0] = to16(v[j], PREC == SG_PREC_F16_TC);
+#pragma unroll
+    for (int z = 0; z < (PREC == SG_PREC_F32_SIMT ? 3 : 1); ++z)
+      h[z][j >> 1] = (j & 1) ? h[z][j >> 1] | ((uint32_t)p[z] << 16) : (uint32_t)p[z];
+  }
+#pragma unroll
+  for (int z = 0; z < (PREC == SG_PREC_F32_SIMT ? 3 : 1); ++z)
+    *reinterpret_cast<uint4*>(dst + z * plane) = make_uint4(h[z][0], h[z][1], h[z][2], h[z][3]);
+  return bad;
+}
+
+
+// Both operands of a product in one launch: A (M x K, leading dimension lda) ->
+// a16 (M x Kp) and B (K x N) -> b16 (N x Kp), K-major 16-bit copies (PREC: bf16,
+// fp16, or three bf16 planes), zero padded to Kp, a multiple of 64.  The first
+// na CTAs take A, eight entries a thread; the others 64 x 64 tiles of B, turned
+// around in shared memory: 16-byte loads along n, 16-byte stores along k.
+// *gate = 1: an entry the pieces do not take.
+template <int PREC>
+__global__ void __launch_bounds__(256) k_cast_operands(const float* __restrict__ A, int lda, int M,
+                                                       const float* __restrict__ B, int ldb, int N,
+                                                       int K, int Kp, uint16_t* __restrict__ a16,
+                                                       uint16_t* __restrict__ b16, int* gate,
+                                                       unsigned na, int va, int vb) {
+  __shared__ float t[64][65];
+  bool bad = false;
+  if (blockIdx.x < na) {
+    const long long u = blockIdx.x * 256LL + threadIdx.x, r = u / (Kp / 8);
+    const int c0 = (int)(u % (Kp / 8)) * 8;
+    if (r >= M) return;
+    const float* src = A + r * lda + c0;
+    float x[8];
+    if (va && c0 + 8 <= K) {
+      const float4 p = __ldcs(reinterpret_cast<const float4*>(src));
+      const float4 q = __ldcs(reinterpret_cast<const float4*>(src) + 1);
+      x[0] = p.x; x[1] = p.y; x[2] = p.z; x[3] = p.w;
+      x[4] = q.x; x[5] = q.y; x[6] = q.z; x[7] = q.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) x[j] = c0 + j < K ? __ldcs(src + j) : 0.0f;
+    }
+    bad = store_operand<PREC>(a16 + r * Kp + c0, (size_t)M * Kp, x);
+  } else {
+    const unsigned b = blockIdx.x - na, nt = (unsigned)(N + 63) / 64;
+    const int k0 = (int)(b / nt) * 64, n0 = (int)(b % nt) * 64;
+    float4 v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int e = threadIdx.x + 256 * i, k = k0 + (e >> 4), n = n0 + (e & 15) * 4;
+      const float* src = B + (size_t)k * ldb + n;
+      if (vb && k < K && n + 4 <= N) {
+        v[i] = __ldcs(reinterpret_cast<const float4*>(src));
+      } else {
+        float x[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x[j] = k < K && n + j < N ? __ldcs(src + j) : 0.0f;
+        v[i] = make_float4(x[0], x[1], x[2], x[3]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int e = threadIdx.x + 256 * i, r = e >> 4, c = (e & 15) * 4;
+      t[r][c] = v[i].x; t[r][c + 1] = v[i].y; t[r][c + 2] = v[i].z; t[r][c + 3] = v[i].w;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int e = threadIdx.x + 256 * i, nn = e >> 3, kc = (e & 7) * 8;
+      if (n0 + nn >= N) continue;
+      float x[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) x[j] = t[kc + j][nn];
+      bad |= store_operand<PREC>(b16 + (size_t)(n0 + nn) * Kp + k0 + kc, (size_t)N * Kp, x);
+    }
+  }
+  if (PREC == SG_PREC_F32_SIMT && bad) *gate = 1;
+}
+
+template <int PREC>
+cudaError_t launch_cast_operands(const float* A, int lda, const float* B, int ldb, int M, int N,
+                                 int K, int Kp, uint16_t* a16, uint16_t* b16, int* gate,
+                                 cudaStream_t s) {
+  const long long na = ((long long)M * (Kp / 8) + 255) / 256;
+  const long long nb = (long long)((N + 63) / 64) * (Kp / 64);
+  k_cast_operands<PREC><<<(unsigned)(na + nb), 256, 0, s>>>(
+      A, lda, M, B, ldb, N, K, Kp, a16, b16, gate, (unsigned)na,
+      lda % 4 == 0 && (uintptr_t)A % 16 == 0, ldb % 4 == 0 && (uintptr_t)B % 16 == 0);
+  return cudaGetLastError();
 }
 
 }  // namespace tc
