@@ -8,7 +8,8 @@
 //      histograms and the input's multiset fingerprint; its last block turns
 //      the histograms into per-digit global start offsets.
 //   2. k_onesweep x4: each CTA takes the next tile (a global atomic ticket,
-//      so tiles start in order; 6144 keys, 24 per thread), prefetches the
+//      so tiles start in order; 6144 keys, 24 per thread, or fewer for
+//      small sorts), prefetches the
 //      tile one resident wave ahead into L2 (cp.async.bulk.prefetch), ranks its keys
 //      stably inside the tile (warp-private counters; the lanes sharing a
 //      digit are found by match_any or by ballots), publishes its per-digit tile
@@ -27,6 +28,7 @@
 #include <stdint.h>
 
 #include <climits>
+#include <type_traits>
 
 #include "sg_internal.h"
 
@@ -35,20 +37,15 @@ namespace {
 
 constexpr int kSortBlock = 256;
 constexpr int kSortMinBlocks = 4;   // resident CTAs per SM the registers are sized for
-constexpr int kKpt = 24;
-constexpr int kTile = kSortBlock * kKpt;   // 6144 keys
 constexpr int kMatchEvery = 8;
 constexpr int kRadix = 256;
 constexpr int kWarps = kSortBlock / 32;
-constexpr int kWarpKeys = 32 * kKpt;
 constexpr unsigned kSpinLimit = 1u << 22;
-// look-back window: the words of this many preceding tiles are loaded
-// together and then taken in order, so one memory round trip covers several
-// steps of the walk (4 for the 32-bit words, 2 for the 64-bit words of the
-// checked last pass: the fastest of 1, 2, 4 and 8 for each, 15% and 8% faster
-// passes than one word at a time)
-constexpr int kLook = 4;
-constexpr int kLookWide = 2;
+// Look-back window (LOOK; half of it for the 64-bit words of the checked last
+// pass): the words of this many preceding tiles are loaded together and then
+// taken in order, so one memory round trip covers several steps of the walk (4
+// and 2 for large sorts: the fastest of 1, 2, 4 and 8 for each, 15% and 8% faster
+// passes than one word at a time; small sorts: keys_per_thread)
 
 constexpr unsigned kCntMask = (1u << 30) - 1;
 constexpr unsigned kAgg = 1u;
@@ -275,8 +272,9 @@ __global__ void __launch_bounds__(256) k_radix_hist(const int* __restrict__ in, 
 }
 
 // ---------------------------------------------------------------------------
-template <bool CK>
+template <bool CK, int KPT>
 struct SortSmem {
+  static constexpr int kTile = kSortBlock * KPT;
   int keys[kTile + 1];   // + a sentinel after the tile's keys (checked pass)
   unsigned whist[kWarps][kRadix];
   // checked pass: the last key of each warp's keys of each digit, so that a
@@ -293,12 +291,14 @@ struct SortSmem {
 
 // One tile of one pass.  FULL: the tile holds kTile keys (every tile but the
 // last), so no index is checked against n.
-template <bool LAST, bool CHECK, bool FULL, bool FLT>
-__device__ __forceinline__ void onesweep_tile(SortSmem<LAST && CHECK>& sm, const int* __restrict__ in,
+template <bool LAST, bool CHECK, bool FULL, bool FLT, int KPT, int LOOK>
+__device__ __forceinline__ void onesweep_tile(SortSmem<LAST && CHECK, KPT>& sm, const int* __restrict__ in,
                                               int* __restrict__ out, long long n, int pass,
                                               SortHdr* h, unsigned* st32,
                                               unsigned long long* st64, SortResult* res,
                                               unsigned tile, const LookbackCtl lb) {
+  constexpr int kKpt = KPT, kTile = kSortBlock * KPT, kWarpKeys = 32 * KPT;
+  constexpr int kLook = LOOK, kLookWide = LOOK / 2;
   int* const s_keys = sm.keys;
   unsigned (*const s_whist)[kRadix] = sm.whist;
   int* const s_gbase = sm.gbase;
@@ -546,12 +546,13 @@ __device__ __forceinline__ void onesweep_tile(SortSmem<LAST && CHECK>& sm, const
   }
 }
 
-template <bool LAST, bool CHECK, bool FLT>
+template <bool LAST, bool CHECK, bool FLT, int KPT, int LOOK>
 __global__ void __launch_bounds__(kSortBlock, kSortMinBlocks) k_onesweep(
     const int* __restrict__ in, int* __restrict__ out, long long n, int pass, SortHdr* h,
     unsigned* st32, unsigned long long* st64, SortResult* res, unsigned ahead,
     const LookbackCtl lb) {
-  __shared__ SortSmem<LAST && CHECK> sm;
+  __shared__ SortSmem<LAST && CHECK, KPT> sm;
+  constexpr int kTile = kSortBlock * KPT;
   const int tid = threadIdx.x;
   if (tid == 0) {
     // an earlier pass whose look-back gave up left its output incomplete:
@@ -573,9 +574,9 @@ __global__ void __launch_bounds__(kSortBlock, kSortMinBlocks) k_onesweep(
                    : "memory");
   }
   if ((long long)(tile + 1) * kTile <= n)
-    onesweep_tile<LAST, CHECK, true, FLT>(sm, in, out, n, pass, h, st32, st64, res, tile, lb);
+    onesweep_tile<LAST, CHECK, true, FLT, KPT, LOOK>(sm, in, out, n, pass, h, st32, st64, res, tile, lb);
   else
-    onesweep_tile<LAST, CHECK, false, FLT>(sm, in, out, n, pass, h, st32, st64, res, tile, lb);
+    onesweep_tile<LAST, CHECK, false, FLT, KPT, LOOK>(sm, in, out, n, pass, h, st32, st64, res, tile, lb);
 }
 
 // ---------------------------------------------------------------------------
@@ -626,9 +627,20 @@ struct Layout {
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// Keys per thread, and with them the tile (256 threads) and the look-back window.
+// Large sorts are bound by what the SMs do per tile, which 24 keys per thread
+// spread over the most keys (pass at 2^26: 217 us; 16 keys 247, 8 keys 365).  A
+// sort whose tiles are all resident at once is a chain of latencies, the
+// ranking of a thread's keys and a look-back over tiles none of which has a
+// prefix yet: smaller tiles, and 16 words per round trip instead of 4.  Whole
+// sort by kernel times, 24 keys / as chosen: 61 / 44 us at 30000, 57 / 49 us at 10^5, 67
+// / 62 us at 10^6, equal at 2 10^6.
+int keys_per_thread(long long n) { return n <= 200000 ? 8 : n <= 2000000 ? 16 : 24; }
+
 Layout layout(long long n) {
   Layout L;
-  const size_t ntiles = (size_t)((n + kTile - 1) / kTile);
+  const size_t tile = (size_t)kSortBlock * keys_per_thread(n);
+  const size_t ntiles = ((size_t)n + tile - 1) / tile;
   size_t off = align256(sizeof(SortHdr));
   for (int p = 0; p < 3; ++p) {
     L.st32[p] = off;
@@ -656,7 +668,7 @@ size_t sort_scratch_bytes(long long n) { return layout(n).total; }
 
 namespace {
 
-template <bool FLT>
+template <bool FLT, int KPT, int LOOK>
 cudaError_t sort_impl(const int32_t* in, int32_t* out, long long n, bool contracts,
                         void* scratch, SortResult* res, cudaStream_t s, int num_sms,
                         int64_t* kernels, const SortInject* inject, Prof* prof,
@@ -677,16 +689,17 @@ cudaError_t sort_impl(const int32_t* in, int32_t* out, long long n, bool contrac
   else
     k_radix_hist<FLT, false><<<grid_for((n + 3) / 4 / 8, num_sms, 8), 256, 0, s>>>(in, n, h, res);
   prof_end(prof, s);
+  constexpr int kTile = kSortBlock * KPT;
   const unsigned ntiles = (unsigned)((n + kTile - 1) / kTile);
   const unsigned ahead = (unsigned)num_sms * kSortMinBlocks;
   prof_begin(prof, "onesweep", s);
-  k_onesweep<false, false, FLT><<<ntiles, kSortBlock, 0, s>>>(in, tmp, n, 0, h, st32[0], st64, res, ahead, lb);
+  k_onesweep<false, false, FLT, KPT, LOOK><<<ntiles, kSortBlock, 0, s>>>(in, tmp, n, 0, h, st32[0], st64, res, ahead, lb);
   prof_end(prof, s);
   prof_begin(prof, "onesweep", s);
-  k_onesweep<false, false, FLT><<<ntiles, kSortBlock, 0, s>>>(tmp, out, n, 1, h, st32[1], st64, res, ahead, lb);
+  k_onesweep<false, false, FLT, KPT, LOOK><<<ntiles, kSortBlock, 0, s>>>(tmp, out, n, 1, h, st32[1], st64, res, ahead, lb);
   prof_end(prof, s);
   prof_begin(prof, "onesweep", s);
-  k_onesweep<false, false, FLT><<<ntiles, kSortBlock, 0, s>>>(out, tmp, n, 2, h, st32[2], st64, res, ahead, lb);
+  k_onesweep<false, false, FLT, KPT, LOOK><<<ntiles, kSortBlock, 0, s>>>(out, tmp, n, 2, h, st32[2], st64, res, ahead, lb);
   prof_end(prof, s);
   if (inject && inject->mode == 1 && inject->i < n && inject->j < n) {
     // swap through the (now free) output buffer: stream-ordered host copies
@@ -707,9 +720,9 @@ cudaError_t sort_impl(const int32_t* in, int32_t* out, long long n, bool contrac
   unsigned* st_last = reinterpret_cast<unsigned*>(st64);
   prof_begin(prof, contracts ? "onesweep_last_checked" : "onesweep", s);
   if (contracts)
-    k_onesweep<true, true, FLT><<<ntiles, kSortBlock, 0, s>>>(tmp, out, n, 3, h, st_last, st64, res, ahead, lb);
+    k_onesweep<true, true, FLT, KPT, LOOK><<<ntiles, kSortBlock, 0, s>>>(tmp, out, n, 3, h, st_last, st64, res, ahead, lb);
   else
-    k_onesweep<true, false, FLT><<<ntiles, kSortBlock, 0, s>>>(tmp, out, n, 3, h, st_last, st64, res, ahead, lb);
+    k_onesweep<true, false, FLT, KPT, LOOK><<<ntiles, kSortBlock, 0, s>>>(tmp, out, n, 3, h, st_last, st64, res, ahead, lb);
   prof_end(prof, s);
   *kernels += 5;
   return cudaGetLastError();
@@ -721,10 +734,19 @@ cudaError_t launch_sort(const int32_t* in, int32_t* out, long long n, bool contr
                         void* scratch, SortResult* res, cudaStream_t s, int num_sms,
                         int64_t* kernels, const SortInject* inject, Prof* prof, bool flt,
                         const LookbackCtl& lb) {
-  return flt ? sort_impl<true>(in, out, n, contracts, scratch, res, s, num_sms, kernels, inject,
-                               prof, lb)
-             : sort_impl<false>(in, out, n, contracts, scratch, res, s, num_sms, kernels, inject,
-                                prof, lb);
+  auto go = [&](auto flag, auto kpt, auto look) {
+    return sort_impl<decltype(flag)::value, decltype(kpt)::value, decltype(look)::value>(
+        in, out, n, contracts, scratch, res, s, num_sms, kernels, inject, prof, lb);
+  };
+  auto by_size = [&](auto flag) {
+    using std::integral_constant;
+    switch (keys_per_thread(n)) {
+      case 8: return go(flag, integral_constant<int, 8>{}, integral_constant<int, 16>{});
+      case 16: return go(flag, integral_constant<int, 16>{}, integral_constant<int, 16>{});
+      default: return go(flag, integral_constant<int, 24>{}, integral_constant<int, 4>{});
+    }
+  };
+  return flt ? by_size(std::true_type{}) : by_size(std::false_type{});
 }
 
 size_t check_scratch_bytes() { return 0; }
