@@ -969,8 +969,58 @@ bool jit_available() { return nvrtc().ok; }
 
 // Returns the specialised kernel, compiling it on first use; nullptr when it
 // cannot be built (then the caller uses the interpreting kernel).
+namespace {
+
+// The kernels already asked for, by what their source depends on (the
+// program's operators and slots, not its constants, and the template's
+// parameters): writing the source out to look it up in compile_cached took 4 us
+// of every flush.
+class KernelMemo {
+ public:
+  std::string key;
+  explicit KernelMemo(char kind) : key(1, kind) {}
+  void add(int v) { key.append(reinterpret_cast<const char*>(&v), sizeof v); }
+  void add(const Prog& p) {
+    const int n = p.nops < 0 ? 0 : p.nops > kMaxProg ? kMaxProg : p.nops;
+    add((int)p.nops);
+    key.append(reinterpret_cast<const char*>(p.op), (size_t)n);
+    key.append(reinterpret_cast<const char*>(p.arg), (size_t)n);
+  }
+  bool find(cudaKernel_t* k) const {
+    std::lock_guard<std::mutex> lk(mu());
+    const auto it = map().find(key);
+    if (it == map().end()) return false;
+    *k = it->second;
+    return true;
+  }
+  cudaKernel_t keep(cudaKernel_t k) const {
+    if (k) {
+      std::lock_guard<std::mutex> lk(mu());
+      map()[key] = k;
+    }
+    return k;
+  }
+
+ private:
+  static std::mutex& mu() {
+    static std::mutex m;
+    return m;
+  }
+  static std::unordered_map<std::string, cudaKernel_t>& map() {
+    static std::unordered_map<std::string, cudaKernel_t> m;
+    return m;
+  }
+};
+
+}  // namespace
+
 cudaKernel_t jit_stream_kernel(const Prog& pr, int nin, int nout, int npred, bool reduce,
                                bool minmax, uint32_t pred_exists, std::string* log) {
+  KernelMemo memo('s');
+  memo.add(pr);
+  for (int v : {nin, nout, npred, (int)reduce, (int)minmax, (int)pred_exists}) memo.add(v);
+  cudaKernel_t found;
+  if (memo.find(&found)) return found;
   if (!nvrtc().ok) {
     if (log) *log = "NVRTC library not found";
     return nullptr;
@@ -987,7 +1037,7 @@ cudaKernel_t jit_stream_kernel(const Prog& pr, int nin, int nout, int npred, boo
            nin, nin > 0 ? nin : 1, nout, nout > 0 ? nout : 1, npred, reduce ? 1 : 0,
            minmax ? 1 : 0);
   const std::string src = std::string(defs) + kTemplateHead + body_fn(body) + kTemplateKernel;
-  return compile_cached(src, "sg_fused", log);
+  return memo.keep(compile_cached(src, "sg_fused", log));
 }
 
 cudaKernel_t jit_batch_kernel(const Prog& pr, std::string* log) {
@@ -1072,9 +1122,16 @@ bool filter_tile_scans(int tile) { return tile >= 8192; }
 int filter_tile_occupancy(int tile) { return tile >= 8192 ? 4 : tile >= 4096 ? 6 : 8; }
 
 cudaKernel_t jit_filter_kernel(const Prog& pred, std::string* log, int tile, const Prog* post) {
+  KernelMemo memo('f');
+  memo.add(pred);
+  memo.add(tile);
+  memo.add(post ? 1 : 0);
+  if (post) memo.add(*post);
+  cudaKernel_t found;
+  if (memo.find(&found)) return found;
   std::string src;
   if (!filter_source(pred, tile, &src, log, post)) return nullptr;
-  return compile_cached(src, "sg_filter", log);
+  return memo.keep(compile_cached(src, "sg_filter", log));
 }
 
 bool jit_check_filter(const Prog& pred, std::string* log, const Prog* post) {

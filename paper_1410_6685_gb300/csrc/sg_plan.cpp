@@ -729,10 +729,8 @@ cudaError_t launch_stream_scheduled(sg_ctx* c, cudaKernel_t jk, const sgk::Strea
   const std::vector<sg_sched_choice> cand = sg_stream_candidates(w.n, c->num_sms);
   const sg_sched_choice d = sg_stream_default();
   const int gd = sg_stream_grid(w.n, d, c->num_sms);
-  std::vector<float> X(cand.size() * kSchedFeatures);
   int def = -1;
   for (size_t i = 0; i < cand.size(); ++i) {
-    sg_stream_features(w, cand[i], c->num_sms, &X[i * kSchedFeatures]);
     if (def < 0 && cand[i].chunk == d.chunk && sg_stream_grid(w.n, cand[i], c->num_sms) == gd)
       def = (int)i;
   }
@@ -744,7 +742,14 @@ cudaError_t launch_stream_scheduled(sg_ctx* c, cudaKernel_t jk, const sgk::Strea
   int learned = -1;
   std::vector<float> pred;
   std::vector<double> us;
-  int idx = sg_sched_lookup(c, SG_SCHED_STREAM, key, X, def, &learned, &pred, &us);
+  int idx = -1;
+  std::vector<float> X;
+  if (!sg_sched_settled(c, SG_SCHED_STREAM, key, cand.size(), &idx, &learned, &us)) {
+    X.resize(cand.size() * kSchedFeatures);
+    for (size_t i = 0; i < cand.size(); ++i)
+      sg_stream_features(w, cand[i], c->num_sms, &X[i * kSchedFeatures]);
+    idx = sg_sched_lookup(c, SG_SCHED_STREAM, key, X, def, &learned, &pred, &us);
+  }
   cudaError_t e = cudaSuccess;
   if (idx < 0) {
     bool in_place = false;
@@ -790,19 +795,23 @@ cudaError_t launch_filter_scheduled(sg_ctx* c, const sgk::Prog& pr, const float*
   FilterWork w;
   w.n = n;
   w.ops = pr.nops;
-  std::vector<float> X(cand.size() * kSchedFeatures);
   int def = 0;
-  for (size_t i = 0; i < cand.size(); ++i) {
-    sg_filter_features(w, cand[i], sgk::filter_tile_occupancy((int)cand[i].chunk), c->num_sms,
-                       &X[i * kSchedFeatures]);
+  for (size_t i = 0; i < cand.size(); ++i)
     if (cand[i].chunk == d.chunk) def = (int)i;
-  }
   const uint64_t key = sg_sched_key(SG_SCHED_FILTER, {(uint64_t)n, prog_shape(pr),
                                                       post ? prog_shape(*post) + 1 : 0});
   int learned = -1;
   std::vector<float> pred;
   std::vector<double> us;
-  int idx = sg_sched_lookup(c, SG_SCHED_FILTER, key, X, def, &learned, &pred, &us);
+  int idx = -1;
+  std::vector<float> X;
+  if (!sg_sched_settled(c, SG_SCHED_FILTER, key, cand.size(), &idx, &learned, &us)) {
+    X.resize(cand.size() * kSchedFeatures);
+    for (size_t i = 0; i < cand.size(); ++i)
+      sg_filter_features(w, cand[i], sgk::filter_tile_occupancy((int)cand[i].chunk), c->num_sms,
+                         &X[i * kSchedFeatures]);
+    idx = sg_sched_lookup(c, SG_SCHED_FILTER, key, X, def, &learned, &pred, &us);
+  }
   cudaError_t e = cudaSuccess;
   auto kernel = [&](int i) {
     return sgk::jit_filter_kernel(pr, nullptr, (int)cand[i].chunk, post);
@@ -939,7 +948,17 @@ sg_status run_flush(sg_ctx* c, bool fuse, bool commit, double* us) {
       default: need_records = true; break;
     }
   }
-  cudaError_t e = need_records ? cudaMemsetAsync(dres, 0, res_bytes, c->stream) : cudaSuccess;
+  // A flush whose only records are stream passes' lets their last block store
+  // the whole record into the pinned host buffer: no clearing and no copy (3.5
+  // us of a flush of one small pass).  Other kernels add to their records with
+  // atomics, in device memory.
+  bool direct = need_records && commit && c->host_res_mapped;
+  for (Pass& P : passes)
+    direct &= P.kind == PK::STREAM || P.kind == PK::TRANSPOSE || P.kind == PK::MATVEC ||
+              P.kind == PK::CONCAT || (P.kind == PK::MATMUL && !P.chk_frv);
+  if (direct) dres = static_cast<char*>(c->host_res);
+  const bool copy_back = need_records && !direct;
+  cudaError_t e = copy_back ? cudaMemsetAsync(dres, 0, res_bytes, c->stream) : cudaSuccess;
   sg_status status = SG_OK;
   cudaEvent_t tev[2] = {nullptr, nullptr};
   if (us && e == cudaSuccess) {
@@ -1150,7 +1169,7 @@ sg_status run_flush(sg_ctx* c, bool fuse, bool commit, double* us) {
   if (us && e == cudaSuccess && !status) e = cudaEventRecord(tev[1], c->stream);
   // while an asynchronous read is still on the copy engine, the records are
   // stored by a kernel instead of queueing a copy behind it
-  if (e == cudaSuccess && !status && need_records) {
+  if (e == cudaSuccess && !status && copy_back) {
     if (dl_busy) {
       e = sgk::launch_copy(c->host_res, dres, passes.size() * sgk::kResultBytes, c->num_sms,
                            c->stream);

@@ -288,6 +288,19 @@ void sg_sched_note(sg_ctx* c, int family, const std::vector<sg_sched_choice>& ca
   c->schedst.has_last[family] = true;
 }
 
+bool sg_sched_settled(const sg_ctx* c, int family, uint64_t key, size_t ncand, int* idx,
+                      int* learned, std::vector<double>* us) {
+  *learned = -1;
+  const int f = c->schedst.forced[family];
+  if (f >= 0 && f < (int)ncand) {
+    *idx = f;
+    return true;
+  }
+  if (c->sched == SG_SCHED_LEARNED && c->schedst.model[family].trained) return false;
+  *idx = sg_sched_tuned(c, key, us, learned);
+  return *idx >= 0;
+}
+
 int sg_sched_lookup(sg_ctx* c, int family, uint64_t key, const std::vector<float>& X, int def,
                     int* learned, std::vector<float>* pred, std::vector<double>* us) {
   *learned = -1;

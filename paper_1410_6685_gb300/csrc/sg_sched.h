@@ -123,3 +123,8 @@ void sg_sched_note(sg_ctx* c, int family, const std::vector<sg_sched_choice>& ca
 // choice when it was measured.
 int sg_sched_lookup(sg_ctx* c, int family, uint64_t key, const std::vector<float>& X, int def,
                     int* learned, std::vector<float>* pred, std::vector<double>* us);
+// The same decision where it needs no features (a forced index, or an
+// autotuned one outside the learned scheduler): true with *idx, asked before
+// the features of `ncand` candidates are computed.
+bool sg_sched_settled(const sg_ctx* c, int family, uint64_t key, size_t ncand, int* idx,
+                      int* learned, std::vector<double>* us);
