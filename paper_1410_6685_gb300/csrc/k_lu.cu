@@ -30,8 +30,8 @@
 // Solve: pivots on the right-hand side, then forward / backward substitution
 // by steps of 128 rows in one launch each: CTAs take steps in order
 // (ticket) and wait, with a bounded spin, for the steps they depend on; each
-// step's diagonal block is applied through its inverse (assembled from the
-// 64 x 64 inverses formed once per factorisation), one short product
+// step's diagonal block is applied through its inverse (formed once per
+// factorisation), one short product
 // instead of 128 dependent steps.
 // Refinement: residual r = b - A x in binary64 from the binary32 A, and the
 // update x += d with the norms the stopping test needs.
@@ -572,48 +572,80 @@ __global__ void __launch_bounds__(kPT, 1)
 
 // The interchanges of an outer block's panels (moves lists m0, m0 + 1, ...,
 // in order) on the columns outside it, [0, K) and [K + KB, n), and on the
-// row permutation perm: one thread per column; for each list every load of
-// the column precedes its stores.
-__global__ void __launch_bounds__(128) k_lu_laswp_outer(float* LU, int n, const int* __restrict__ moves,
+// row permutation perm.  Every CTA first composes the lists into one (entry: a
+// position's last move, its source followed back through the earlier lists;
+// each list is a permutation of its rows, at most 64), then moves its 32
+// columns through shared memory, all loads before any store.  One load and
+// one store phase instead of one per list: 27 -> 7 us at n = 1000.
+constexpr int kSwapCols = 32;
+constexpr int kSwapMax = kLuOuter / kPB * 2 * kPB;   // entries of all lists
+__global__ void __launch_bounds__(256) k_lu_laswp_outer(float* LU, int n, const int* __restrict__ moves,
                                                         int nlists, int K, int KB, int* perm) {
-  __shared__ int s_cnt[kLuOuter / kPB], s_src[kLuOuter / kPB][2 * kPB],
-      s_dst[kLuOuter / kPB][2 * kPB];
-  for (int q = 0; q < nlists; ++q) {
-    const int* m = moves + (size_t)q * kLuMoveInts;
-    const int cnt = min(m[0], 2 * kPB);
-    if (threadIdx.x == 0) s_cnt[q] = cnt;
-    for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-      s_src[q][t] = m[1 + t];
-      s_dst[q][t] = m[1 + 2 * kPB + t];
+  __shared__ int s_src[kSwapMax], s_dst[kSwapMax];   // unused entries: -1
+  __shared__ int f_src[kSwapMax], f_dst[kSwapMax], f_n;
+  __shared__ float s_val[kSwapMax][kSwapCols];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  // entry e: list e / 64, move e % 64
+  const int q0 = tid / (2 * kPB), t0 = tid % (2 * kPB);
+  int src = -1, dst = -1;
+  if (q0 < nlists) {
+    const int* m = moves + (size_t)q0 * kLuMoveInts;
+    const int ms = m[1 + t0], md = m[1 + 2 * kPB + t0];   // loaded with the count
+    if (t0 < min(m[0], 2 * kPB)) {
+      src = ms;
+      dst = md;
+    }
+  }
+  s_src[tid] = src;
+  s_dst[tid] = dst;
+  if (tid == 0) f_n = 0;
+  __syncthreads();
+  if (dst >= 0) {
+    bool last = true;
+    for (int q = q0 + 1; q < nlists; ++q) {
+#pragma unroll 16
+      for (int t = 0; t < 2 * kPB; ++t) last &= s_dst[q * 2 * kPB + t] != dst;
+    }
+    if (last) {
+      for (int q = q0 - 1; q >= 0; --q) {
+        int hit = -1;
+#pragma unroll 16
+        for (int t = 0; t < 2 * kPB; ++t) hit = s_dst[q * 2 * kPB + t] == src ? t : hit;
+        if (hit >= 0) src = s_src[q * 2 * kPB + hit];
+      }
+      if (src != dst) {
+        const int k = atomicAdd(&f_n, 1);
+        f_src[k] = src;
+        f_dst[k] = dst;
+      }
     }
   }
   __syncthreads();
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g == n - KB) {
+  const int ne = f_n;
+  if (blockIdx.x == gridDim.x - 1) {
     // one more column: the row permutation itself
-    for (int q = 0; q < nlists; ++q) {
-      const int cnt = s_cnt[q];
-      int v[2 * kPB];
-#pragma unroll
-      for (int t = 0; t < 2 * kPB; ++t)
-        if (t < cnt) v[t] = perm[s_src[q][t]];
-#pragma unroll
-      for (int t = 0; t < 2 * kPB; ++t)
-        if (t < cnt) perm[s_dst[q][t]] = v[t];
-    }
+    int v = 0;
+    if (tid < ne) v = perm[f_src[tid]];
+    __syncthreads();
+    if (tid < ne) perm[f_dst[tid]] = v;
     return;
   }
-  const int c = g < K ? g : g + KB;
-  if (c >= n) return;
-  for (int q = 0; q < nlists; ++q) {
-    const int cnt = s_cnt[q];
-    float v[2 * kPB];
+  const int g = blockIdx.x * kSwapCols + lane, c = g < K ? g : g + KB;
+  if (c < n) {
+    for (int e0 = w; e0 < ne; e0 += 128) {
+      float v[16];
 #pragma unroll
-    for (int t = 0; t < 2 * kPB; ++t)
-      if (t < cnt) v[t] = LU[(size_t)s_src[q][t] * n + c];
+      for (int i = 0; i < 16; ++i)
+        if (e0 + 8 * i < ne) v[i] = LU[(size_t)f_src[e0 + 8 * i] * n + c];
 #pragma unroll
-    for (int t = 0; t < 2 * kPB; ++t)
-      if (t < cnt) LU[(size_t)s_dst[q][t] * n + c] = v[t];
+      for (int i = 0; i < 16; ++i)
+        if (e0 + 8 * i < ne) s_val[e0 + 8 * i][lane] = v[i];
+    }
+  }
+  __syncthreads();
+  if (c < n) {
+#pragma unroll 8
+    for (int e = w; e < ne; e += 8) LU[(size_t)f_dst[e] * n + c] = s_val[e][lane];
   }
 }
 
@@ -806,152 +838,188 @@ __global__ void k_apply_perm(const double* __restrict__ rhs, float* y, int n,
     y[i] = (float)rhs[perm[i]];
 }
 
-// Inverses of the 64x64 diagonal blocks of L (unit lower) and U (upper),
-// once per factorisation, for the blocked substitutions: inv[0][b] = L_bb^-1,
-// inv[1][b] = U_bb^-1, row-major; a block cut by n is padded with the
-// identity.  One CTA per block: thread j < 64 forms column j of L_bb^-1 by
-// forward substitution, thread 64 + j column j of U_bb^-1 by back
-// substitution, both in registers.
-constexpr int kTB = 64;   // rows of a substitution block
-__global__ void __launch_bounds__(2 * kTB) k_lu_diag_inv(const float* __restrict__ LU, int n,
-                                                         float* __restrict__ inv) {
-  __shared__ float D[kTB][kTB + 1];
-  const int b = blockIdx.x, row0 = b * kTB, tid = threadIdx.x;
-  for (int t = tid; t < kTB * kTB; t += 2 * kTB) {
-    const int r = t / kTB, c = t % kTB;
-    D[r][c] = (row0 + r < n && row0 + c < n) ? LU[(size_t)(row0 + r) * n + row0 + c]
-                                             : (r == c ? 1.0f : 0.0f);
+// Inverses of the 128 x 128 diagonal blocks of L (unit lower) and U (upper),
+// once per factorisation, for the blocked substitutions; a block cut by n is
+// padded with the identity.  One CTA per block: first the two 64 x 64 diagonal
+// blocks' inverses by substitution, 256 threads each with 16 rows of a column
+// in registers, a finished row passed on through shared memory; then, with f the block
+// solved first (the upper one for L, the lower one for U), s the other and X
+// the rows of s over the columns of f, -inv_s X inv_f takes the place of X.
+// (The substitutions used to form this product from the 64 x 64 inverses at
+// the start of every step of every solve: 10 us of each launch.)
+// Layout, as the substitutions read it: the row r of step c, columns 32 g + 4 k ..
+// + 3, is float4 ((c 4 + g) 8 + k) 128 + r; the steps of L, then those of U.
+constexpr int kTB = 64;              // rows of a diagonal block
+constexpr int kRB = 2 * kTB;         // rows of a step
+constexpr int kDS = kTB + 4;         // 16-byte rows
+constexpr int kInvThreads = 512;
+constexpr size_t kInvSmem = (size_t)6 * kTB * kDS * sizeof(float);
+__global__ void __launch_bounds__(kInvThreads) k_lu_diag_inv(const float* __restrict__ LU, int n,
+                                                             float4* __restrict__ inv) {
+  extern __shared__ __align__(16) float ism[];
+  float* dt = ism;                     // [2][kTB][kDS] the diagonal blocks, transposed
+  float* iv = dt + 2 * kTB * kDS;      // [2][kTB][kDS] their inverses
+  float* xa = iv + 2 * kTB * kDS;      // [kTB][kDS] X, then inv_s X inv_f
+  float* xb = xa + kTB * kDS;          // [kTB][kDS] X inv_f
+  const int c = blockIdx.x, tid = threadIdx.x, row0 = c * kRB;
+  const bool lower = blockIdx.y == 0;
+  const bool two = row0 + kTB < n;
+  const int kf = lower || !two ? 0 : 1, ks = 1 - kf;
+  // eight loads in flight per thread (one after the other they took 20 us)
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int t = tid + (8 * h + i) * kInvThreads, k = h, r = t / kTB % kTB, q = t % kTB;
+      const int b0 = row0 + kTB * k;
+      v[i] = (b0 + r < n && b0 + q < n) ? __ldg(LU + (size_t)(b0 + r) * n + b0 + q)
+                                        : (r == q ? 1.0f : 0.0f);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int t = tid + (8 * h + i) * kInvThreads;
+      dt[(h * kTB + t % kTB) * kDS + t / kTB % kTB] = v[i];
+    }
+  }
+  {
+    float v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int t = tid + i * kInvThreads;
+      const int r = row0 + kTB * ks + t / kTB, q = row0 + kTB * kf + t % kTB;
+      v[i] = two && r < n && q < n ? __ldg(LU + (size_t)r * n + q) : 0.0f;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int t = tid + i * kInvThreads;
+      xa[t / kTB * kDS + t % kTB] = v[i];
+    }
   }
   __syncthreads();
-  const int nb = gridDim.x;
-  const int j = tid % kTB;
-  float x[kTB];
-  if (tid < kTB) {
+  {
+    // 256 threads per block: thread (j, rg) holds rows 16 rg .. + 15 of column j
+    const int j = tid % kTB, rg = tid / kTB % 4, blk = tid / (4 * kTB);
+    const float* D = dt + blk * kTB * kDS;   // D[q * kDS + r]: entry (r, q)
+    float* xs = iv + blk * kTB * kDS;        // row q of the inverse, once final
+    float x[16];
 #pragma unroll
-    for (int i = 0; i < kTB; ++i) {
-      float acc = i == j ? 1.0f : 0.0f;
+    for (int i = 0; i < 16; ++i) x[i] = 16 * rg + i == j ? 1.0f : 0.0f;
+#pragma unroll 1
+    for (int h = 0; h < 4; ++h) {
+      const int og = lower ? h : 3 - h;      // rows 16 og .. + 15 become final
 #pragma unroll
-      for (int q = 0; q < i; ++q) acc = fmaf(-D[i][q], x[q], acc);
-      x[i] = acc;
+      for (int u = 0; u < 16; ++u) {
+        const int v = lower ? u : 15 - u, q = 16 * og + v;
+        if (rg == og) {
+          // (x[v] with v known only through `lower`: both are constants here)
+          float xv = lower ? x[u] : x[15 - u];
+          if (!lower) xv /= D[q * kDS + q];
+          xs[q * kDS + j] = xv;
+        }
+        __syncthreads();
+        const float xq = xs[q * kDS + j];
+        const bool all = lower ? rg > og : rg < og;
+        if (all || rg == og) {
+          const float4* Dq = reinterpret_cast<const float4*>(D + q * kDS + 16 * rg);
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            const float4 d = Dq[g];
+            const float dd[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int i = 4 * g + e;
+              const bool after = lower ? i > u : i < 15 - u;
+              if (all || after) x[i] = fmaf(-dd[e], xq, x[i]);
+            }
+          }
+        }
+      }
     }
+  }
+  __syncthreads();
+  if (two) {
+    // X inv_f, then inv_s (X inv_f): thread = one column, eight rows
+    const int jj = tid % kTB, r8 = (tid / kTB) * 8;
+    auto product = [&](const float* P, const float* Q, float* R) {
+      float a[8];
 #pragma unroll
-    for (int i = 0; i < kTB; ++i) inv[((size_t)b * kTB + i) * kTB + j] = x[i];
-  } else {
+      for (int i = 0; i < 8; ++i) a[i] = 0.0f;
+#pragma unroll 2
+      for (int m = 0; m < kTB; m += 4) {
+        float q[4];
 #pragma unroll
-    for (int i = kTB - 1; i >= 0; --i) {
-      float acc = i == j ? 1.0f : 0.0f;
+        for (int e = 0; e < 4; ++e) q[e] = Q[(m + e) * kDS + jj];
 #pragma unroll
-      for (int q = i + 1; q < kTB; ++q) acc = fmaf(-D[i][q], x[q], acc);
-      x[i] = acc / D[i][i];
-    }
+        for (int i = 0; i < 8; ++i) {
+          const float4 p = *reinterpret_cast<const float4*>(P + (r8 + i) * kDS + m);
+          a[i] = fmaf(p.x, q[0], a[i]);
+          a[i] = fmaf(p.y, q[1], a[i]);
+          a[i] = fmaf(p.z, q[2], a[i]);
+          a[i] = fmaf(p.w, q[3], a[i]);
+        }
+      }
 #pragma unroll
-    for (int i = 0; i < kTB; ++i) inv[((size_t)(nb + b) * kTB + i) * kTB + j] = x[i];
+      for (int i = 0; i < 8; ++i) R[(r8 + i) * kDS + jj] = a[i];
+      __syncthreads();
+    };
+    product(xa, iv + kf * kTB * kDS, xb);
+    product(iv + ks * kTB * kDS, xb, xa);
+  }
+  float4* out = inv + ((size_t)blockIdx.y * gridDim.x + c) * (kRB * kRB / 4);
+  for (int t = tid; t < kRB * kRB / 4; t += kInvThreads) {
+    const int r = t % kRB, c4 = t / kRB * 4, kr = r / kTB, kc = c4 / kTB;
+    const int o = r % kTB * kDS + c4 % kTB;
+    const float* p = kr == kc ? iv + kr * kTB * kDS + o : xa + o;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (kr == kc ? (kr == 0 || two) : (two && kr == ks))
+      v = kr == kc ? make_float4(p[0], p[1], p[2], p[3]) : make_float4(-p[0], -p[1], -p[2], -p[3]);
+    out[t] = v;
   }
 }
 
-// Triangular solve by steps of 128 rows (two 64-row blocks).  LOWER: unit
-// lower L, steps in increasing order; else upper U with its diagonal, in
-// decreasing order.  Each step first forms, in shared memory, the inverse of
-// its 128 x 128 diagonal block from the two 64 x 64 inverses: with f the
-// block solved first (the upper one for L, the lower one for U), s the
-// other and X the rows of s over the columns of f, the inverse holds f's and
-// s's inverses on its diagonal and -inv_s X inv_f in place of X.  This is
-// done while earlier steps run, and each thread then keeps a 32-column
-// quarter of one row of it in registers.  A step's 128 rows form four
-// groups of 32, four warps per group sharing the step's dependencies in
-// 32-column pieces (warp q of a group takes every fourth, in the order they
-// are solved), each loading its piece row by row, coalesced (lane =
-// column), before waiting, with a bounded spin, for the flag of the step the
-// piece belongs to; one transposing warp reduction then gives lane r the sum
-// of row r.  The right-hand sides minus those sums times the inverse give
-// the step's solution, published with one flag (a release store).  The
-// chain of global waits from step to step (a few microseconds each, the
-// same at every size) bounds the solve.
-constexpr int kRB = 2 * kTB;         // rows of a step
+// Triangular solve by steps of 128 rows.  LOWER: unit lower L, steps in
+// increasing order; else upper U with its diagonal, in decreasing order.  A
+// step's diagonal block is applied through its inverse (k_lu_diag_inv), each
+// thread keeping a 32-column quarter of one row of it in registers, loaded
+// while earlier steps run.  A step's 128 rows form four groups of 32, four
+// warps per group sharing the step's dependencies in 32-column pieces (warp q
+// of a group takes every fourth, in the order they are solved), each loading
+// its piece row by row, coalesced (lane = column), before waiting, with a
+// bounded spin, for the flag of the step the piece belongs to; one transposing
+// warp reduction then gives lane r the sum of row r.  The right-hand sides
+// minus those sums times the inverse give the step's solution, published with
+// one flag (a release store).  The chain of global waits from step to step (a
+// few microseconds each, the same at every size) bounds the solve.
 constexpr int kTrsvThreads = 512;
-constexpr int kTS = kTB + 1;         // shared row strides (conflict-free lane = row reads)
-constexpr int kRS = kRB + 1;
-constexpr size_t kTrsvSmem =
-    (kRB * kRS + 2 * kTB * kTS + (kTrsvThreads / 32) * 32 + kRB + 4 * kRB) * sizeof(float) + 16;
 template <bool LOWER>
 __global__ void __launch_bounds__(kTrsvThreads, 1) k_trsv(const float* __restrict__ LU,
-                                                          const float* __restrict__ inv, int n,
+                                                          const float4* __restrict__ inv, int n,
                                                           float* y, unsigned* flags,
                                                           unsigned epoch, unsigned* ticket,
                                                           int* err) {
-  extern __shared__ float tsm[];
-  float* ib = tsm;                                     // [kRB][kRS] the step's inverse
-  float* xa = ib + kRB * kRS;                          // [kTB][kTS] X
-  float* xb = xa + kTB * kTS;                          // [kTB][kTS] X inv_f
-  float* part = xb + kTB * kTS;                        // [16][32]
-  float* vsh = part + (kTrsvThreads / 32) * 32;        // [kRB]
-  float* xp = vsh + kRB;                               // [4][kRB] quarter sums
-  unsigned* s_b = reinterpret_cast<unsigned*>(xp + 4 * kRB);
+  __shared__ float part[kTrsvThreads];
+  __shared__ __align__(16) float vsh[kRB];
+  __shared__ float xp[4 * kRB];   // quarter sums
+  __shared__ unsigned s_b;
   const int tid = threadIdx.x;
-  const int nb = (n + kTB - 1) / kTB;
   const int nst = (n + kRB - 1) / kRB;
-  if (tid == 0) *s_b = atomicAdd(ticket, 1u);
+  if (tid == 0) s_b = atomicAdd(ticket, 1u);
   __syncthreads();
-  const int t = (int)*s_b;
+  const int t = (int)s_b;
   const int c = LOWER ? t : nst - 1 - t;
   const int row0 = c * kRB;
   const int lane = tid & 31, w = tid >> 5;
   const int g = w >> 2, wq = w & 3;              // row group, and the warp's share of it
-  const bool two = 2 * c + 1 < nb;
-  const int nblk = two ? 2 : 1;
-  const int kf = LOWER || !two ? 0 : 1, ks = 1 - kf;
   // warps 0-3 (lane + 32 w = row of the step) read their right-hand side now
   const int rs = 32 * (w & 3) + lane;
   const float bv = (w < 4 && row0 + rs < n) ? __ldcg(&y[row0 + rs]) : 0.0f;
-  // the diagonal inverses (zero elsewhere), and X
-  for (int e = tid; e < kRB * kRB; e += kTrsvThreads) {
-    const int r = e / kRB, jj = e % kRB, kr = r / kTB;
-    ib[r * kRS + jj] = (kr == jj / kTB && kr < nblk)
-                           ? inv[((size_t)(2 * c + kr) * kTB + r % kTB) * kTB + jj % kTB]
-                           : 0.0f;
-  }
-  if (two)
-    for (int e = tid; e < kTB * kTB; e += kTrsvThreads) {
-      const int r = e / kTB, jj = e % kTB;
-      const int gr = row0 + kTB * ks + r, gc = (2 * c + kf) * kTB + jj;
-      xa[r * kTS + jj] = (gr < n && gc < n) ? LU[(size_t)gr * n + gc] : 0.0f;
-    }
-  __syncthreads();
-  if (two) {
-    // X inv_f, then -inv_s (X inv_f): thread = one column, eight rows
-    const int jj = tid % kTB, r8 = (tid / kTB) * 8;
-    const float* fi = ib + (kTB * kf) * kRS + kTB * kf + jj;
-    float a[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) a[i] = 0.0f;
-#pragma unroll 8
-    for (int m = 0; m < kTB; ++m) {
-      const float bm = fi[m * kRS];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) a[i] = fmaf(xa[(r8 + i) * kTS + m], bm, a[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) xb[(r8 + i) * kTS + jj] = a[i];
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 8; ++i) a[i] = 0.0f;
-    const float* si = ib + (kTB * ks) * kRS + kTB * ks;
-#pragma unroll 8
-    for (int m = 0; m < kTB; ++m) {
-      const float bm = xb[m * kTS + jj];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) a[i] = fmaf(si[(r8 + i) * kRS + m], bm, a[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) ib[(kTB * ks + r8 + i) * kRS + kTB * kf + jj] = -a[i];
-    __syncthreads();
-  }
-  // this thread's quarter of row rs of the inverse
+  // this thread's quarter of row rs of the step's inverse
   float iv[32];
-  {
-    const float* ir = ib + rs * kRS + 32 * g;
 #pragma unroll
-    for (int jj = 0; jj < 32; ++jj) iv[jj] = ir[jj];
+  for (int k = 0; k < 8; ++k) {
+    const float4 q = __ldg(inv + ((size_t)(c * 4 + g) * 8 + k) * kRB + rs);
+    iv[4 * k] = q.x; iv[4 * k + 1] = q.y; iv[4 * k + 2] = q.z; iv[4 * k + 3] = q.w;
   }
   // the dependencies: lane = column, one transposing reduction at the end
   float acc[32];
@@ -1060,7 +1128,20 @@ __global__ void __launch_bounds__(256) k_residual(const float* __restrict__ A, i
   for (long long i = warp; i < n; i += nw) {
     const float* row = A + i * (long long)n;
     double s = 0.0;
-    for (int j = lane; j < n; j += 32) s = fma(f32_to_f64(__ldcs(row + j)), x[j], s);
+    // eight columns' loads in flight, then their multiply-adds in order (one
+    // at a time the loads' latency made 23 us of n = 1000, 164 us of 8192)
+    for (int j = lane; j < n; j += 256) {
+      float av[8];
+      double xv[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const bool in = j + 32 * u < n;
+        av[u] = in ? __ldcs(row + j + 32 * u) : 0.0f;
+        xv[u] = in ? x[j + 32 * u] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) s = fma(f32_to_f64(av[u]), xv[u], s);
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     const double ri = b[i] - s;
@@ -1120,7 +1201,13 @@ __global__ void __launch_bounds__(256) k_anorm(const float* __restrict__ A, int 
   for (long long i = warp; i < n; i += nw) {
     const float* row = A + i * (long long)n;
     double s = 0.0;
-    for (int j = lane; j < n; j += 32) s += fabs(f32_to_f64(row[j]));
+    for (int j = lane; j < n; j += 256) {
+      float av[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) av[u] = j + 32 * u < n ? __ldg(row + j + 32 * u) : 0.0f;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) s += fabs(f32_to_f64(av[u]));
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     mx = fmax(mx, s);
@@ -1270,9 +1357,10 @@ cudaError_t launch_lu_panel(float* LU, int n, int k, int jb, int* piv, int* info
 
 cudaError_t launch_lu_laswp_outer(float* LU, int n, const int* moves, int nlists, int K, int KB,
                                   int* perm, cudaStream_t s, Prof* prof) {
-  const int cols = n - KB + 1;   // and the permutation
+  static_assert(kSwapMax == 256, "one thread per entry");
+  const int ctas = (n - KB + kSwapCols - 1) / kSwapCols + 1;   // and the permutation
   prof_begin(prof, "lu_laswp", s);
-  k_lu_laswp_outer<<<(cols + 127) / 128, 128, 0, s>>>(LU, n, moves, nlists, K, KB, perm);
+  k_lu_laswp_outer<<<ctas, 256, 0, s>>>(LU, n, moves, nlists, K, KB, perm);
   prof_end(prof, s);
   return cudaGetLastError();
 }
@@ -1302,11 +1390,15 @@ cudaError_t launch_lu_iota(int* perm, int n, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-size_t lu_diag_inv_bytes(int n) { return (size_t)2 * ((n + kTB - 1) / kTB) * kTB * kTB * 4; }
+size_t lu_diag_inv_bytes(int n) { return (size_t)2 * ((n + kRB - 1) / kRB) * kRB * kRB * 4; }
 
 cudaError_t launch_lu_diag_inv(const float* LU, int n, float* inv, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_lu_diag_inv<<<(n + kTB - 1) / kTB, 2 * kTB, 0, s>>>(LU, n, inv);
+  const cudaError_t e = cudaFuncSetAttribute(
+      k_lu_diag_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInvSmem);
+  if (e != cudaSuccess) return e;
+  k_lu_diag_inv<<<dim3((n + kRB - 1) / kRB, 2), kInvThreads, kInvSmem, s>>>(
+      LU, n, reinterpret_cast<float4*>(inv));
   return cudaGetLastError();
 }
 
@@ -1315,24 +1407,14 @@ cudaError_t launch_lu_solve(const float* LU, const float* inv, int n, const int*
                             unsigned epoch, unsigned* tickets, int* err, cudaStream_t s,
                             Prof* prof) {
   (void)rhs_is_residual;
-  const int nb = (n + kTB - 1) / kTB;
   const int nst = (n + kRB - 1) / kRB;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(k_trsv<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kTrsvSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_trsv<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kTrsvSmem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  const float4* i4 = reinterpret_cast<const float4*>(inv);
   prof_begin(prof, "lu_trsv", s);
   k_apply_perm<<<(n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024, 256, 0, s>>>(rhs, y, n, perm);
   cudaMemsetAsync(tickets, 0, 2 * sizeof(unsigned), s);
-  k_trsv<true><<<nst, kTrsvThreads, kTrsvSmem, s>>>(LU, inv, n, y, flags, epoch, tickets, err);
-  k_trsv<false><<<nst, kTrsvThreads, kTrsvSmem, s>>>(LU, inv + (size_t)nb * kTB * kTB, n, y,
-                                                     flags + nb, epoch, tickets + 1, err);
+  k_trsv<true><<<nst, kTrsvThreads, 0, s>>>(LU, i4, n, y, flags, epoch, tickets, err);
+  k_trsv<false><<<nst, kTrsvThreads, 0, s>>>(LU, i4 + (size_t)nst * (kRB * kRB / 4), n, y,
+                                             flags + nst, epoch, tickets + 1, err);
   prof_end(prof, s);
   return cudaGetLastError();
 }

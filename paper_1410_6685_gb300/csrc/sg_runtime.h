@@ -162,7 +162,7 @@ struct LuCache {
   float* lu = nullptr;
   int* piv = nullptr;
   int* perm = nullptr;          // row i of the factors is row perm[i] of A
-  float* inv = nullptr;         // inverses of the factors' 32x32 diagonal blocks
+  float* inv = nullptr;         // inverses of the factors' 128 x 128 diagonal blocks
   int* info = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaStream_t cap = nullptr;
