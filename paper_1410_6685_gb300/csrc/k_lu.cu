@@ -570,6 +570,202 @@ __global__ void __launch_bounds__(kPT, 1)
   }
 }
 
+// The panel with one row per thread: PC CTAs (one, or a cluster), T threads
+// each, rows r0 .. r0 + rs - 1 (rs <= T) of the panel in registers, in the shifted
+// layout of k_lu_panel_reg.  Per column: each warp's best candidate (larger
+// magnitude, then lower position) stages its row in shared memory; one CTA barrier; every warp finds the best of the
+// warps' keys the same way.  One CTA: that is the pivot.  A cluster: warp q
+// sends the CTA's key and row to CTA q by asynchronous remote stores that
+// complete on the receiver's mbarrier, and the best of the CTAs' keys is the
+// pivot.  Then every row is updated from the pivot row in shared memory.  The
+// interchanges, the zero-pivot rule, the write-back and the lists are
+// k_lu_panel_reg's, and so are the operations and their order.
+template <int PC, int T>
+struct PanelSmem {
+  static constexpr int kWarps = T / 32;
+  float stage[2][kWarps][kPB];
+  float crow[PC > 1 ? 2 : 1][PC][kPB];
+  static constexpr int kXC = (kLuOuter - kPB + PC - 1) / PC;   // other columns of the block per CTA
+  int mv[4 * kPB];                                             // the moved rows, then where to
+  unsigned long long wkey[2][kWarps];
+  unsigned long long cand[2][PC];
+  unsigned long long bar[2];
+  int fpos[T];
+  float lbuf[T * kStride];
+};
+template <int PC, int T>
+__global__ void __launch_bounds__(T, 1)
+    k_lu_panel_rows(float* __restrict__ LU, int n, int k, int jb, int* __restrict__ piv,
+                    int* __restrict__ info, int* __restrict__ moves, int c_lo, int c_hi) {
+  constexpr int kW = T / 32;
+  extern __shared__ __align__(16) unsigned char smem[];
+  PanelSmem<PC, T>& sm = *reinterpret_cast<PanelSmem<PC, T>*>(smem);
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int rank = PC > 1 ? (int)cg::this_cluster().block_rank() : 0;
+  const int m = n - k, rs = (m + PC - 1) / PC, r0 = rank * rs, r1 = min(m, r0 + rs);
+  const int r = r0 + tid;
+  bool act = r < r1;
+  int lp = r;
+  float x[kPB];
+  {
+    const float* src = LU + (size_t)(k + (act ? r : 0)) * n + k;
+    if (((n | k) & 3) == 0) {   // then jb is a multiple of 4 too
+#pragma unroll
+      for (int q = 0; q < kPB / 4; ++q) {
+        const float4 v = act && 4 * q < jb ? __ldg(reinterpret_cast<const float4*>(src) + q)
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+        x[4 * q] = v.x; x[4 * q + 1] = v.y; x[4 * q + 2] = v.z; x[4 * q + 3] = v.w;
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < kPB; ++c) x[c] = act && c < jb ? __ldg(src + c) : 0.0f;
+    }
+  }
+  if (PC > 1) {
+    if (tid < 2)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sm_addr(&sm.bar[tid])) : "memory");
+    if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    cg::this_cluster().sync();   // every CTA's barriers exist before anyone sends
+  }
+  // The lane with the best of one key per lane, -1 when there is none.  (One
+  // maximum and a ballot, with the second maximum for ties alone, was 5%
+  // slower a column: the branch.)
+  auto winner_of = [](unsigned long long u) {
+    const unsigned hi = (unsigned)(u >> 32), lo = (unsigned)u;
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    const unsigned eq = __ballot_sync(0xffffffffu, u != 0ull && hi == mh && lo == ml);
+    return eq ? __ffs(eq) - 1 : -1;
+  };
+  int my_info = 0;
+  bool failed = false;
+#pragma unroll 1
+  for (int j = 0; j < jb; ++j) {
+    const int par = j & 1;
+    // (the top bit: a row's key is never 0)
+    const unsigned long long mine = act ? key_of(x[0], lp, r) | (1ull << 63) : 0ull;
+    const int wl = winner_of(mine);
+    if (lane == wl) {
+      float4* st = reinterpret_cast<float4*>(sm.stage[par][w]);
+#pragma unroll
+      for (int q = 0; q < kPB / 4; ++q)
+        st[q] = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
+      sm.wkey[par][w] = mine;
+    }
+    if (wl < 0 && lane == 0) sm.wkey[par][w] = 0ull;
+    const uint32_t mbar = sm_addr(&sm.bar[par]);
+    if (PC > 1 && tid == 0)   // this column's bytes from the cluster complete bar[par]
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar),
+                   "r"(col_bytes<PC>()) : "memory");
+    __syncthreads();
+    unsigned long long u = lane < kW ? sm.wkey[par][lane] : 0ull;
+    int best = winner_of(u);
+    const float* prow = sm.stage[par][best < 0 ? 0 : best];
+    unsigned long long g;
+    if (PC > 1) {
+      // A CTA sends column j + 2 only after it has all of column j + 1, which
+      // every CTA sends only after reading column j: two slots suffice.
+      g = best < 0 ? 0ull : sm.wkey[par][best];
+      for (int q = w; q < PC; q += kW) {
+        if (lane < kPB / 4)
+          st_async_v4(cl_addr(sm_addr(&sm.crow[par][rank][4 * lane]), q),
+                      g ? reinterpret_cast<const float4*>(prow)[lane]
+                        : make_float4(0.f, 0.f, 0.f, 0.f), cl_addr(mbar, q));
+        else if (lane == kPB / 4)
+          st_async_b64(cl_addr(sm_addr(&sm.cand[par][rank]), q), g, cl_addr(mbar, q));
+      }
+      // after a wait gave up nothing is written back; later columns do not wait
+      if (!failed && !bar_wait(mbar, (uint32_t)(j >> 1) & 1u)) failed = true;
+      u = lane < PC ? sm.cand[par][lane] : 0ull;
+      best = winner_of(u);
+      prow = sm.crow[par][best < 0 ? 0 : best];
+    }
+    float pv[kPB];
+#pragma unroll
+    for (int q = 0; q < kPB / 4; ++q) {
+      const float4 v = reinterpret_cast<const float4*>(prow)[q];
+      pv[4 * q] = v.x; pv[4 * q + 1] = v.y; pv[4 * q + 2] = v.z; pv[4 * q + 3] = v.w;
+    }
+    const float d = pv[0];
+    const bool pzero = d == 0.0f;
+    const float rd = 1.0f / d;
+    const float l = pzero ? x[0] : x[0] * rd;
+    if (pzero) {   // the row is only shifted
+#pragma unroll
+      for (int c = 0; c + 1 < kPB; ++c) x[c] = x[c + 1];
+      if (my_info == 0) my_info = k + j + 1;
+    } else {
+#pragma unroll
+      for (int c = 0; c + 1 < kPB; ++c) x[c] = fmaf(-l, pv[c + 1], x[c + 1]);
+    }
+    x[kPB - 1] = 0.0f;
+    g = __shfl_sync(0xffffffffu, u, best < 0 ? 0 : best);
+    const int p = (int)(0xFFFFu - (unsigned)((g >> 16) & 0xFFFFu));   // winning position
+    const int gp = (int)(g & 0xFFFFu);                                // its row in the panel
+    // interchange of positions j and p; the pivot row retires (what its
+    // registers hold no longer matters), its U part, columns j .. jb - 1, copied
+    // out by one warp
+    if (lp == j) lp = p;
+    if (act && r == gp) {
+      lp = j;
+      act = false;
+    }
+    if (act) sm.lbuf[tid * kStride + j] = l;
+    if (w == (j & (kW - 1)) && gp >= r0 && gp < r1 && lane < jb - j)
+      sm.lbuf[(gp - r0) * kStride + j + lane] = prow[lane];
+    if (tid == 0 && rank == 0) piv[k + j] = k + p;
+  }
+  if (PC > 1 && failed) atomicCAS(info, 0, -1);   // a wait gave up: report, write nothing
+  const bool any_failed = __syncthreads_or(failed);
+  if (PC > 1) cg::this_cluster().sync();   // no CTA reads another's shared memory after this
+  // list the rows that moved (at most 2 jb); every row's final position
+  if (!any_failed && r < r1) {
+    sm.fpos[tid] = lp;
+    if (lp != r) {
+      const int t = atomicAdd(&moves[0], 1);
+      if (t < 2 * kPB) {
+        moves[1 + t] = k + r;
+        moves[1 + 2 * kPB + t] = k + lp;
+      }
+    }
+  }
+  __syncthreads();
+  // write the panel back in its final row order, one row per warp store
+  if (!any_failed) {
+    for (int q = w; q < r1 - r0; q += kW)
+      if (lane < jb) LU[(size_t)(k + sm.fpos[q]) * n + k + lane] = sm.lbuf[q * kStride + lane];
+  }
+  if (tid == 0 && rank == 0 && my_info) atomicCAS(info, 0, my_info);
+  if (PC > 1) cg::this_cluster().sync();   // every CTA's moves are listed
+  else __syncthreads();
+  // the interchanges on the outer block's other columns [c_lo, k) and
+  // [k + jb, c_hi), CTA `rank` the columns rank, rank + PC, ...: the lists once
+  // into shared memory, then all loads before any store
+  constexpr int kXC = PanelSmem<PC, T>::kXC;
+  const int nl = k - c_lo, nc = nl + (c_hi - k - jb);
+  const int nci = nc > rank ? (nc - rank + PC - 1) / PC : 0;
+  if (!any_failed && nci > 0) {
+    const int cnt = min(__ldcg(&moves[0]), 2 * kPB);
+    for (int t = tid; t < 4 * kPB; t += T) sm.mv[t] = __ldcg(&moves[1 + t]);
+    __syncthreads();
+    constexpr int kPer = (2 * kPB * kXC + T - 1) / T;   // entries per thread
+    float v[kPer];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      const int e = tid + i * T, t = e / kXC, g2 = rank + e % kXC * PC;
+      if (t < cnt && e % kXC < nci)
+        v[i] = __ldcg(LU + (size_t)sm.mv[t] * n + (g2 < nl ? c_lo + g2 : k + jb + (g2 - nl)));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      const int e = tid + i * T, t = e / kXC, g2 = rank + e % kXC * PC;
+      if (t < cnt && e % kXC < nci)
+        LU[(size_t)sm.mv[2 * kPB + t] * n + (g2 < nl ? c_lo + g2 : k + jb + (g2 - nl))] = v[i];
+    }
+  }
+}
+
 // The interchanges of an outer block's panels (moves lists m0, m0 + 1, ...,
 // in order) on the columns outside it, [0, K) and [K + KB, n), and on the
 // row permutation perm.  Every CTA first composes the lists into one (entry: a
@@ -1344,13 +1540,52 @@ cudaError_t lu_prepare(int n) {
   return cudaFuncSetAttribute(k_lu_trsm_outer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx);
 }
 
+namespace {
+template <int PC, int T>
+cudaError_t launch_rows(float* LU, int n, int k, int jb, int* piv, int* info, int* moves, int c_lo,
+                        int c_hi, cudaStream_t s) {
+  auto fn = k_lu_panel_rows<PC, T>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(PanelSmem<PC, T>));
+  if (e == cudaSuccess && PC > 8)
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(PC);
+  cfg.blockDim = dim3(T);
+  cfg.dynamicSmemBytes = sizeof(PanelSmem<PC, T>);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = PC;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = PC > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, fn, LU, n, k, jb, piv, info, moves, c_lo, c_hi);
+}
+}  // namespace
+
 cudaError_t launch_lu_panel(float* LU, int n, int k, int jb, int* piv, int* info, int* moves,
                             int c_lo, int c_hi, cudaStream_t s, Prof* prof) {
   prof_begin(prof, "lu_panel", s);
-  const cudaError_t e =
-      !portable_kernels() && use_cluster16()
-          ? launch_panel<16>(LU, n, k, jb, piv, info, moves, c_lo, c_hi, s)
-                      : launch_panel<8>(LU, n, k, jb, piv, info, moves, c_lo, c_hi, s);
+  // One row per thread up to 4096 rows: one CTA up to 256 rows (no exchange; 1130
+  // clocks a column), 8 up to 2048 (1470), 16 up to 4096 (1700).  More CTAs cost
+  // more per exchange, more rows per CTA more per update, each thread reading
+  // the whole pivot row from shared memory (16 CTAs of 576 rows: 2900 clocks at
+  // 8192 rows, where two or three rows per thread of k_lu_panel_reg take 2300).
+  const int m = n - k;
+  cudaError_t e;
+  if (portable_kernels() || !use_cluster16())
+    e = launch_panel<8>(LU, n, k, jb, piv, info, moves, c_lo, c_hi, s);
+  else if (m <= 256)
+    e = launch_rows<1, 256>(LU, n, k, jb, piv, info, moves, c_lo, c_hi, s);
+  else if (m <= 2048)
+    e = launch_rows<8, 256>(LU, n, k, jb, piv, info, moves, c_lo, c_hi, s);
+  else if (m <= 4096)
+    e = launch_rows<16, 256>(LU, n, k, jb, piv, info, moves, c_lo, c_hi, s);
+  else
+    e = launch_panel<16>(LU, n, k, jb, piv, info, moves, c_lo, c_hi, s);
   prof_end(prof, s);
   return e;
 }
