@@ -1027,9 +1027,14 @@ __global__ void k_lu_iota(int* perm, int n) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) perm[i] = i;
 }
 
-// y = P rhs (binary64 in, binary32 out): y[i] = rhs[perm[i]]
+// y = P rhs (binary64 in, binary32 out): y[i] = rhs[perm[i]].  Also clears the
+// substitutions' tickets and the norms the update after them forms.
 __global__ void k_apply_perm(const double* __restrict__ rhs, float* y, int n,
-                             const int* __restrict__ perm) {
+                             const int* __restrict__ perm, unsigned* tickets, double* norms) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    tickets[0] = tickets[1] = 0u;
+    norms[1] = norms[2] = 0.0;
+  }
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
     y[i] = (float)rhs[perm[i]];
 }
@@ -1638,15 +1643,14 @@ cudaError_t launch_lu_diag_inv(const float* LU, int n, float* inv, cudaStream_t 
 }
 
 cudaError_t launch_lu_solve(const float* LU, const float* inv, int n, const int* perm,
-                            const double* rhs, bool rhs_is_residual, float* y, unsigned* flags,
-                            unsigned epoch, unsigned* tickets, int* err, cudaStream_t s,
+                            const double* rhs, float* y, unsigned* flags, unsigned epoch,
+                            unsigned* tickets, double* norms, int* err, cudaStream_t s,
                             Prof* prof) {
-  (void)rhs_is_residual;
   const int nst = (n + kRB - 1) / kRB;
   const float4* i4 = reinterpret_cast<const float4*>(inv);
   prof_begin(prof, "lu_trsv", s);
-  k_apply_perm<<<(n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024, 256, 0, s>>>(rhs, y, n, perm);
-  cudaMemsetAsync(tickets, 0, 2 * sizeof(unsigned), s);
+  k_apply_perm<<<(n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024, 256, 0, s>>>(rhs, y, n, perm, tickets,
+                                                                           norms);
   k_trsv<true><<<nst, kTrsvThreads, 0, s>>>(LU, i4, n, y, flags, epoch, tickets, err);
   k_trsv<false><<<nst, kTrsvThreads, 0, s>>>(LU, i4 + (size_t)nst * (kRB * kRB / 4), n, y,
                                              flags + nst, epoch, tickets + 1, err);

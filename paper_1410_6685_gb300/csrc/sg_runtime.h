@@ -172,6 +172,7 @@ struct LuCache {
   int* gates = nullptr;         // its words per outer block: an entry the pieces do not take
   int* moves = nullptr;         // the panels' interchange lists, then their counters
   char* operands = nullptr;     // tensor-core operand copies
+  void* host = nullptr;         // pinned, for the solve's small read-backs
   void clear();
   ~LuCache() { clear(); }
 };

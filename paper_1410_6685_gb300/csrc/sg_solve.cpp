@@ -207,6 +207,11 @@ sg_status lu_factor(sg_ctx* c, const float* A, int n, sg_precision prec, const d
     L.moves = reinterpret_cast<int*>(base + o_moves);
     L.gates = reinterpret_cast<int*>(base + o_gates);
     L.operands = base + o_gemm;
+    if (cudaMallocHost(&L.host, 128) != cudaSuccess) {
+      cudaGetLastError();
+      L.clear();
+      return err(c, SG_ERR_OOM, "pinned result buffer allocation failed");
+    }
     L.n = n;
     L.prec = (int)prec;
   }
@@ -246,22 +251,22 @@ sg_status lu_factor(sg_ctx* c, const float* A, int n, sg_precision prec, const d
     cudaError_t e = cudaGraphLaunch(exec, s);
     sgk::prof_end(&c->prof, s);
     c->kernels += kernels;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(hi, L.info, sizeof hi, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(L.host, L.info, sizeof hi, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
       cudaGetLastError();
       return err(c, SG_ERR_CUDA, cudaGetErrorString(e));
     }
+    memcpy(hi, L.host, sizeof hi);
     *hinfo = hi[0];
     return diag && hi[1] ? SG_ERR_NOT_CONVERGED : SG_OK;   // only seen below
   };
   const size_t bytes = (size_t)n * n * 4;
-  double hdom = 0.0;
-  cudaError_t e = cudaMemcpyAsync(&hdom, norms + 6, sizeof hdom, cudaMemcpyDeviceToHost, s);
+  cudaError_t e = cudaMemcpyAsync(L.host, norms + 6, 8, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(L.lu, A, bytes, cudaMemcpyDeviceToDevice, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   int not_dominant = 0;
-  memcpy(&not_dominant, &hdom, sizeof not_dominant);
+  memcpy(&not_dominant, L.host, sizeof not_dominant);
   if (e == cudaSuccess && !not_dominant) {
     const sg_status st = run(true);
     if (st != SG_ERR_NOT_CONVERGED) return st;
@@ -327,9 +332,7 @@ extern "C" sg_status sg_solve(sg_ctx* c, sg_matrix* A, sg_vector* b, const sg_so
   const size_t o_r = take((size_t)n * 8);
   const size_t o_flags = take((size_t)2 * nb * 4);
   const size_t o_tk = take(64);
-  const size_t o_err = take(64);
-  const size_t o_norms = take(8 * 8);
-  const size_t o_viol = take(8);
+  const size_t o_norms = take(8 * 8 + 16);   // norms, then viol and dev_err: read back together
   char* base = nullptr;
   cudaError_t e = cudaMallocAsync((void**)&base, off, c->stream);
   if (e != cudaSuccess) {
@@ -341,9 +344,9 @@ extern "C" sg_status sg_solve(sg_ctx* c, sg_matrix* A, sg_vector* b, const sg_so
   w.r = reinterpret_cast<double*>(base + o_r);
   w.flags = reinterpret_cast<unsigned*>(base + o_flags);
   w.tickets = reinterpret_cast<unsigned*>(base + o_tk);
-  w.dev_err = reinterpret_cast<int*>(base + o_err);
   w.norms = reinterpret_cast<double*>(base + o_norms);
-  w.viol = reinterpret_cast<unsigned long long*>(base + o_viol);
+  w.viol = reinterpret_cast<unsigned long long*>(w.norms + 8);
+  w.dev_err = reinterpret_cast<int*>(w.norms + 9);
 
   // the solution vector (owned by the returned handle)
   auto xv = std::make_shared<Value>();
@@ -370,21 +373,25 @@ extern "C" sg_status sg_solve(sg_ctx* c, sg_matrix* A, sg_vector* b, const sg_so
 
   sg_solve_info inf{0, 0, 0.0, 0.0};
   sg_status status = SG_OK;
-  double hn[8];
+  double hn[10] = {};
   unsigned long long hviol = 0;
   int hinfo = 0, herr = 0;
   unsigned epoch = 0;
+  // One copy to pinned memory brings norms, violation and error: three to
+  // pageable memory and the memsets between the steps, now k_apply_perm's, took
+  // 20 us of an iteration's 60 at n = 1000.
   auto sync_read = [&]() -> bool {
-    e = cudaMemcpyAsync(hn, w.norms, sizeof hn, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, w.dev_err, sizeof herr, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&hviol, w.viol, sizeof hviol, cudaMemcpyDeviceToHost, s);
+    e = cudaMemcpyAsync(c->lu.host, w.norms, sizeof hn, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    return e == cudaSuccess;
+    if (e != cudaSuccess) return false;
+    memcpy(hn, c->lu.host, sizeof hn);
+    memcpy(&hviol, &hn[8], sizeof hviol);
+    memcpy(&herr, &hn[9], sizeof herr);
+    return true;
   };
 
   // 1. factorisation of a copy of A (the context's cached graph)
-  e = cudaMemsetAsync(base + o_flags, 0, o_norms + 64 - o_flags, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(w.viol, 0, 8, s);
+  e = cudaMemsetAsync(base + o_flags, 0, o_norms + sizeof hn - o_flags, s);
   if (e == cudaSuccess) e = sgk::launch_anorm(a, n, w.norms, s);
   if (e == cudaSuccess) {
     status = lu_factor(c, a, n, o.precision, w.norms, &hinfo);
@@ -409,17 +416,16 @@ extern "C" sg_status sg_solve(sg_ctx* c, sg_matrix* A, sg_vector* b, const sg_so
   // 2. initial solve, 3. refinement
   bool converged = false;
   if (!status) {
-    e = sgk::launch_lu_solve(w.lu, c->lu.inv, n, c->lu.perm, bb, false, w.y, w.flags, ++epoch, w.tickets,
-                             w.dev_err, s, prof);
+    e = sgk::launch_lu_solve(w.lu, c->lu.inv, n, c->lu.perm, bb, w.y, w.flags, ++epoch, w.tickets,
+                             w.norms, w.dev_err, s, prof);
     if (e == cudaSuccess) e = sgk::launch_update(x, w.y, bb, n, true, w.norms, s);
     c->kernels += 4;
     double prev = -1.0;
     for (int it = 0; it < o.max_iter && e == cudaSuccess; ++it) {
-      e = cudaMemsetAsync(w.norms, 0, 3 * 8, s);
-      if (e == cudaSuccess) e = sgk::launch_residual(a, n, bb, x, w.r, w.norms, 0.0, nullptr, s, prof);
+      e = sgk::launch_residual(a, n, bb, x, w.r, w.norms, 0.0, nullptr, s, prof);
       if (e == cudaSuccess)
-        e = sgk::launch_lu_solve(w.lu, c->lu.inv, n, c->lu.perm, w.r, true, w.y, w.flags, ++epoch, w.tickets,
-                                 w.dev_err, s, prof);
+        e = sgk::launch_lu_solve(w.lu, c->lu.inv, n, c->lu.perm, w.r, w.y, w.flags, ++epoch,
+                                 w.tickets, w.norms, w.dev_err, s, prof);
       if (e == cudaSuccess) e = sgk::launch_update(x, w.y, bb, n, false, w.norms, s);
       c->kernels += 5;
       if (e != cudaSuccess || !sync_read()) break;
@@ -446,9 +452,10 @@ extern "C" sg_status sg_solve(sg_ctx* c, sg_matrix* A, sg_vector* b, const sg_so
 
   // 4. final residual and the postcondition
   if (!status) {
-    // the bound needs |A|_inf (norms[3]), max|x| (norms[2]) and max|b| (norms[4])
+    // the bound needs |A|_inf (norms[3]), max|x| (norms[2]) and max|b| (norms[4]),
+    // read back with the last step
     e = cudaMemsetAsync(w.norms, 0, 8, s);
-    if (e == cudaSuccess && sync_read()) {
+    if (e == cudaSuccess) {
       const double denom = hn[3] * hn[2] + hn[4];
       const bool check = c->mode >= SG_CONTRACTS_PRE_POST;
       e = cudaMemsetAsync(w.viol, 0, 8, s);
@@ -557,9 +564,10 @@ void LuCache::clear() {
   if (exec) cudaGraphExecDestroy(exec);
   if (exec_diag) cudaGraphExecDestroy(exec_diag);
   if (base) cudaFree(base);
+  if (host) cudaFreeHost(host);
   if (cap) cudaStreamDestroy(cap);
   exec = exec_diag = nullptr;
-  base = nullptr;
+  base = host = nullptr;
   cap = nullptr;
   lu = nullptr;
   piv = nullptr;
