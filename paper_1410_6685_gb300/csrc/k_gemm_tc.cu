@@ -39,6 +39,10 @@ using namespace tc;
 
 constexpr int TM = 128, TN = 256, TK = 64;
 constexpr int A_BYTES = TM * TK * 2;            // 16 KB
+// `corner`: the first kCorner rows and columns of C stay as they are and two
+// SMs stay free, for a caller that has another launch work on them meanwhile
+constexpr int kCorner = 128;
+static_assert(kCorner == TM && kCorner == TN / 2, "whole epilogue warps leave it out");
 // Eight epilogue warps, two per quarter of the tensor memory's lanes, each
 // draining one 128-column half of a tile (with four, each alone on its SM
 // sub-partition, the dependent steps of the epilogue bounded short-K
@@ -162,7 +166,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc(const __grid_consta
                                                     int* err, const float4* __restrict__ frv_r,
                                                     float4* __restrict__ frv_pw, int inj_row,
                                                     int inj_col, float inj_delta,
-                                                     const int* skip) {
+                                                    const int* skip, int corner) {
   if (skip && *skip != 0) return;   // written by earlier launches
   constexpr int STAGES = One<TNv>::kStages, STAGE_BYTES = One<TNv>::kStageBytes;
   constexpr int SL = One<TNv>::kSlices;
@@ -296,8 +300,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc(const __grid_consta
         tile_coords(t + (int)gridDim.x, nM, nN, &bm2, &bn2);
         prefetch_c_row(C, ldc, M, N, bm2 * TM + q * 32 + lane, bn2 * TNv + hh * (TNv / 2), TNv / 2);
       }
+      const bool keep = corner && bm == 0 && bn * TNv + hh * (TNv / 2) < kCorner;
       if (!epilogue_tile<false, TNv>(tmem, acc, tl, tfull0 + 8 * acc, tempty0 + 8 * acc, q, hh,
-                                bm * TM + q * 32, bn * TNv, bn, C, ldc, M, N, subtract, frv_r,
+                                bm * TM + q * 32, bn * TNv, bn, C, ldc, keep ? 0 : M, N, subtract, frv_r,
                                 frv_pw, inj_row, inj_col, inj_delta, s_rw, s_tw, lane, err,
                                 abort_flag))
         break;
@@ -345,7 +350,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc2(const __grid_const
                                                      int* err, const float4* __restrict__ frv_r,
                                                      float4* __restrict__ frv_pw, int inj_row,
                                                      int inj_col, float inj_delta,
-                                                     const int* skip) {
+                                                    const int* skip, int corner) {
   if (skip && *skip != 0) return;   // written by earlier launches
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
@@ -476,8 +481,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc2(const __grid_const
         prefetch_c_row(C, ldc, M, N, bm2 * TM2 + (int)rank * TH + q * 32 + lane,
                        bn2 * TN + hh * (TN / 2), TN / 2);
       }
+      const bool keep = corner && bm == 0 && bn == 0 && rank == 0 && hh == 0;
       if (!epilogue_tile<true, TN>(tmem, acc, tl, tfull0 + 8 * acc, tempty_leader + 8 * acc, q, hh,
-                               bm * TM2 + (int)rank * TH + q * 32, bn * TN, bn, C, ldc, M, N,
+                               bm * TM2 + (int)rank * TH + q * 32, bn * TN, bn, C, ldc, keep ? 0 : M, N,
                                subtract, frv_r, frv_pw, inj_row, inj_col, inj_delta, s_rw, s_tw,
                                lane, err, abort_flag))
         break;
@@ -755,16 +761,17 @@ template <int TNv>
 cudaError_t launch_one(const CUtensorMap& ma, const uint16_t* bt16, int Kp, bool fp16, float* C,
                        int ldc, int M, int N, bool subtract, int* err, const float4* frv_r,
                        float4* frv_pw, int inj_row, int inj_col, float inj_delta, cudaStream_t s,
-                       const int* skip) {
+                       const int* skip, int corner) {
   CUtensorMap mb;
   if (!make_map(&mb, bt16, N, Kp, TNv, fp16)) return cudaErrorInvalidValue;
   const cudaError_t e = cudaFuncSetAttribute(
       k_gemm_tc<TNv>, cudaFuncAttributeMaxDynamicSharedMemorySize, One<TNv>::kSmem);
   if (e != cudaSuccess) return e;
   const long long tiles = (long long)((M + TM - 1) / TM) * ((N + TNv - 1) / TNv);
-  k_gemm_tc<TNv><<<(int)std::min<long long>(tiles, sm_count()), kGemmThreads, One<TNv>::kSmem, s>>>(
+  const int slots = std::max(1, sm_count() - (corner ? 2 : 0));
+  k_gemm_tc<TNv><<<(int)std::min<long long>(tiles, slots), kGemmThreads, One<TNv>::kSmem, s>>>(
       ma, mb, C, ldc, M, N, (Kp / TK + One<TNv>::kSlices - 1) / One<TNv>::kSlices, idesc(fp16, TNv), subtract ? 1 : 0, err, frv_r, frv_pw,
-      inj_row, inj_col, inj_delta, skip);
+      inj_row, inj_col, inj_delta, skip, corner);
   return cudaGetLastError();
 }
 
@@ -773,14 +780,15 @@ cudaError_t launch_one(const CUtensorMap& ma, const uint16_t* bt16, int Kp, bool
 cudaError_t launch_product(const uint16_t* a16, const uint16_t* bt16, int Kp, bool fp16, float* C,
                            int ldc, int M, int N, bool subtract, int* err, const float4* frv_r,
                            float4* frv_pw, int inj_row, int inj_col, float inj_delta,
-                           cudaStream_t s, int form, const int* skip = nullptr) {
+                           cudaStream_t s, int form, const int* skip = nullptr,
+                           int corner = 0) {
   CUtensorMap ma, mb;
   if (!make_map(&ma, a16, M, Kp, TM, fp16)) return cudaErrorInvalidValue;
   if (takes_pair(form)) {
     if (!make_map(&mb, bt16, N, Kp, TH, fp16)) return cudaErrorInvalidValue;
     const long long tiles = (long long)((M + TM2 - 1) / TM2) * ((N + TN - 1) / TN);
     const int pairs = (int)std::max<long long>(
-        1, std::min<long long>(tiles, sm_count() / 2));
+        1, std::min<long long>(tiles, sm_count() / 2 - (corner ? 1 : 0)));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * pairs);
     cfg.blockDim = dim3(kGemmThreads);
@@ -795,15 +803,15 @@ cudaError_t launch_product(const uint16_t* a16, const uint16_t* bt16, int Kp, bo
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k_gemm_tc2, ma, mb, C, ldc, M, N, Kp / TK, idesc2(fp16),
                               subtract ? 1 : 0, err, frv_r, frv_pw, inj_row, inj_col, inj_delta,
-                              skip);
+                              skip, corner);
   }
   switch (one_cta_columns(M, N, Kp)) {
     case 64: return launch_one<64>(ma, bt16, Kp, fp16, C, ldc, M, N, subtract, err, frv_r, frv_pw,
-                                   inj_row, inj_col, inj_delta, s, skip);
+                                   inj_row, inj_col, inj_delta, s, skip, corner);
     case 128: return launch_one<128>(ma, bt16, Kp, fp16, C, ldc, M, N, subtract, err, frv_r,
-                                     frv_pw, inj_row, inj_col, inj_delta, s, skip);
+                                     frv_pw, inj_row, inj_col, inj_delta, s, skip, corner);
     default: return launch_one<256>(ma, bt16, Kp, fp16, C, ldc, M, N, subtract, err, frv_r, frv_pw,
-                                    inj_row, inj_col, inj_delta, s, skip);
+                                    inj_row, inj_col, inj_delta, s, skip, corner);
   }
 }
 
@@ -911,10 +919,10 @@ cudaError_t launch_gemm_tc(const float* A, int lda, const float* B, int ldb, flo
 
 cudaError_t launch_gemm_tc_operands(const uint16_t* a16, const uint16_t* bt16, int K, bool fp16,
                                     float* C, int ldc, int M, int N, int* err, const int* skip,
-                                    cudaStream_t s, int64_t* kernels) {
+                                    cudaStream_t s, int64_t* kernels, int form, bool corner) {
   *kernels += 1;
   return launch_product(a16, bt16, K, fp16, C, ldc, M, N, true, err, nullptr, nullptr, -1, -1, 0.0f,
-                        s, 0, skip);
+                        s, form, skip, corner ? 1 : 0);
 }
 
 cudaError_t launch_gemm_tc_checked(const float* A, const float* B, float* C, int N, bool fp16,

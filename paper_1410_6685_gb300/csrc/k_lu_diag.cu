@@ -6,7 +6,8 @@
 // matrix: 154 of the 235 us that a 128-column outer block took at n = 8192.
 // When no interchange will be needed, as for diagonally dominant matrices,
 // the outer block is three launches instead of about eleven, on average 85 us
-// at n = 8192 (28 + 18 + 43 by kernel; the factorisation 14.8 -> 5.4 ms):
+// at n = 8192 (28 + 18 + 43 by kernel; the factorisation 14.8 -> 5.4 ms), and
+// 70 us with the next diagonal block beside the update (4.4 ms; 16-bit updates):
 //   k_lu_diag_block : the 128 x 128 diagonal block, in one CTA's shared memory;
 //   k_lu_border     : L21 = A21 U11^-1 and U12 = L11^-1 A12, 64 rows or columns
 //                     per CTA, which also writes the trailing update's
@@ -104,10 +105,10 @@ __device__ __forceinline__ void update32_any(int g, float* C, int cs, const floa
 // one per thread, and the rest of the block by all.
 __global__ void __launch_bounds__(kDiagThreads) k_lu_diag_block(float* __restrict__ LU, int n, int K,
                                                                 int KB, int* __restrict__ piv,
+                                                                const int* prev, const int* err,
                                                                 int* fail) {
-  // fail[1]: a wait of the update before gave up
-  if (__syncthreads_or(threadIdx.x == 0 && (fail[0] | fail[1]))) {
-    if (threadIdx.x == 0) fail[0] = 1;
+  if (__syncthreads_or(threadIdx.x == 0 && prev && (*prev | *err))) {
+    if (threadIdx.x == 0) *fail = 1;
     return;
   }
   extern __shared__ __align__(16) float S[];   // [kNB][kS]
@@ -355,9 +356,10 @@ cudaError_t lu_diag_prepare() {
   return e;
 }
 
-cudaError_t launch_lu_diag_block(float* LU, int n, int K, int KB, int* piv, int* fail,
-                                 cudaStream_t s) {
-  k_lu_diag_block<<<1, kDiagThreads, (kNB * kS + kNB) * 4, s>>>(LU, n, K, KB, piv, fail);
+cudaError_t launch_lu_diag_block(float* LU, int n, int K, int KB, int* piv, const int* prev,
+                                 const int* err, int* fail, cudaStream_t s) {
+  k_lu_diag_block<<<1, kDiagThreads, (kNB * kS + kNB) * 4, s>>>(LU, n, K, KB, piv, prev, err,
+                                                                  fail);
   return cudaGetLastError();
 }
 

@@ -46,10 +46,12 @@ cudaError_t launch_gemm_tc(const float* A, int lda, const float* B, int ldb, flo
 bool gemm_pair_available();
 // C -= A16 Bt16^T, the elimination's update with its operands already in
 // K-major 16-bit copies (M x K and N x K, K a multiple of 64); nothing is done
-// when *skip != 0
+// when *skip != 0 (which no launch beside this one may write).  corner: C's
+// first 128 x 128 entries are neither read nor written and two SMs stay free.
 cudaError_t launch_gemm_tc_operands(const uint16_t* a16, const uint16_t* bt16, int K, bool fp16,
                                     float* C, int ldc, int M, int N, int* err, const int* skip,
-                                    cudaStream_t s, int64_t* kernels);
+                                    cudaStream_t s, int64_t* kernels, int form = 0,
+                                    bool corner = false);
 // Casts the operands once, then times the product C = A B in each of `forms`
 // (a warm-up, then the better of two runs, CUDA events on s, a product
 // under 16 us repeated within a run; waits for s): us[f] microseconds.  C

@@ -67,12 +67,12 @@ cudaError_t launch_update(double* x, const float* d, const double* b, int n, boo
 // which also writes the trailing update's operands: L21 as a16 (rest x 128)
 // and U12 transposed as bt16 (rest x 128), bf16 or fp16 by prec, or for
 // SG_PREC_F32_SIMT three bf16 planes of each (*gate = 1: an entry out of their
-// range).  A pivot that is not its column's largest entry sets fail[0];
-// with fail[0] set the launches do nothing.  fail[1]: set by an update whose
-// waits gave up, turned into fail[0] by the next diagonal block.
+// range).  A pivot that is not its column's largest entry sets the outer block's
+// *fail, as does *prev, the last one's (null: the first block), or *err, which an
+// update whose waits gave up sets; with *fail set the border does nothing.
 cudaError_t lu_diag_prepare();
-cudaError_t launch_lu_diag_block(float* LU, int n, int K, int KB, int* piv, int* fail,
-                                 cudaStream_t s);
+cudaError_t launch_lu_diag_block(float* LU, int n, int K, int KB, int* piv, const int* prev,
+                                 const int* err, int* fail, cudaStream_t s);
 cudaError_t launch_lu_border(float* LU, int n, int K, int prec, void* a16, void* bt16, int* gate,
                              int* fail, cudaStream_t s);
 

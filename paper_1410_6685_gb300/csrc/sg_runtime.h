@@ -165,11 +165,14 @@ struct LuCache {
   float* inv = nullptr;         // inverses of the factors' 128 x 128 diagonal blocks
   int* info = nullptr;
   cudaGraphExec_t exec = nullptr;
-  cudaStream_t cap = nullptr;
+  cudaStream_t cap = nullptr;   // captures the graphs; side: their second branch
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
   int64_t kernels = 0;          // kernel launches in one replay
   cudaGraphExec_t exec_diag = nullptr;   // every pivot on the diagonal (k_lu_diag.cu)
   int64_t kernels_diag = 0;
-  int* gates = nullptr;         // its words per outer block: an entry the pieces do not take
+  int* gates = nullptr;         // its words per outer block: an entry the pieces do not take,
+                                // then a pivot off the diagonal
   int* moves = nullptr;         // the panels' interchange lists, then their counters
   char* operands = nullptr;     // tensor-core operand copies
   void* host = nullptr;         // pinned, for the solve's small read-backs

@@ -109,28 +109,51 @@ cudaError_t factor_in_place(sg_ctx* c, float* lu, int n, int* piv, int* perm, in
 // The same factors where no interchange is needed: three launches per
 // 128-column outer block (k_lu_diag.cu).  info[1] != 0 afterwards: a pivot did
 // not stand on the diagonal, and the factors are worthless.
+// With 16-bit updates the next diagonal block, one CTA's serial chain, runs
+// beside the update: its 128 x 128 entries are updated first by a launch of
+// their own, and the update of the rest leaves them and two SMs alone (the whole
+// solve at n = 8192 7.39 -> 6.47 ms, at 2048 1.26 -> 1.19 ms).
 cudaError_t factor_diag(sg_ctx* c, LuCache& L, int n, sg_precision prec, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
-  int* fail = L.info + 1;
   auto at = [&](int r, int col) { return L.lu + (size_t)r * n + col; };
-  const int pieces = prec == SG_PREC_F32_SIMT ? 3 : 1;
+  const bool f32 = prec == SG_PREC_F32_SIMT, fp16 = prec == SG_PREC_F16_TC;
+  const int pieces = f32 ? 3 : 1;
+  const int nb = (n + sgk::kLuOuter - 1) / sgk::kLuOuter;
   uint16_t* a16 = reinterpret_cast<uint16_t*>(L.operands);
   uint16_t* b16 = a16 + (size_t)n * sgk::kLuOuter * pieces;
-  for (int K = 0, q = 0; K < n && e == cudaSuccess; K += sgk::kLuOuter, ++q) {
-    const int KB = std::min(sgk::kLuOuter, n - K), rest = n - K - KB;
-    e = sgk::launch_lu_diag_block(L.lu, n, K, KB, L.piv, fail, s);
+  int* err_word = L.info + 2;
+  // one word per outer block, so that no launch writes what another beside it reads
+  auto fail = [&](int q) { return q == nb - 1 ? L.info + 1 : L.gates + nb + q; };
+  auto diag = [&](int q, cudaStream_t st) {
+    const int K = q * sgk::kLuOuter;
     c->kernels += 1;
-    if (rest <= 0 || e != cudaSuccess) continue;
-    e = sgk::launch_lu_border(L.lu, n, K, prec, a16, b16, L.gates + q, fail, s);
+    return sgk::launch_lu_diag_block(L.lu, n, K, std::min(sgk::kLuOuter, n - K), L.piv,
+                                     q ? fail(q - 1) : nullptr, err_word, fail(q), st);
+  };
+  e = diag(0, s);
+  for (int q = 0; q + 1 < nb && e == cudaSuccess; ++q) {
+    const int K = q * sgk::kLuOuter, next = K + sgk::kLuOuter, rest = n - next;
+    e = sgk::launch_lu_border(L.lu, n, K, prec, a16, b16, L.gates + q, fail(q), s);
     c->kernels += 1;
     if (e != cudaSuccess) break;
-    float* C = at(K + KB, K + KB);
-    e = prec == SG_PREC_F32_SIMT
-            ? sgk::launch_gemm_split_operands(a16, b16, at(K + KB, K), n, at(K, K + KB), n, C, n,
-                                              rest, rest, KB, L.gates + q, fail, fail + 1, s,
-                                              &c->kernels)
-            : sgk::launch_gemm_tc_operands(a16, b16, KB, prec == SG_PREC_F16_TC, C, n, rest, rest,
-                                           fail + 1, fail, s, &c->kernels);
+    if (f32) {
+      e = sgk::launch_gemm_split_operands(a16, b16, at(next, K), n, at(K, next), n, at(next, next),
+                                          n, rest, rest, sgk::kLuOuter, L.gates + q, fail(q),
+                                          err_word, s, &c->kernels);
+      if (e == cudaSuccess) e = diag(q + 1, s);
+      continue;
+    }
+    auto update = [&](int m, int form, bool corner, cudaStream_t st) {
+      return sgk::launch_gemm_tc_operands(a16, b16, sgk::kLuOuter, fp16, at(next, next), n, m, m,
+                                          err_word, fail(q), st, &c->kernels, form, corner);
+    };
+    e = cudaEventRecord(L.fork, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(L.side, L.fork, 0);
+    if (e == cudaSuccess) e = update(std::min(sgk::kLuOuter, rest), 1, false, L.side);
+    if (e == cudaSuccess) e = diag(q + 1, L.side);
+    if (e == cudaSuccess) e = cudaEventRecord(L.join, L.side);
+    if (e == cudaSuccess && rest > sgk::kLuOuter) e = update(rest, 0, true, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, L.join, 0);
   }
   return e;
 }
@@ -164,7 +187,7 @@ cudaError_t capture(sg_ctx* c, LuCache& L, cudaGraphExec_t* exec, int64_t* kerne
 // factored without interchanges first (each pivot is verified on the device);
 // when that fails, or for any other matrix, the general elimination runs.
 // The choice costs one read-back of 8 bytes (about 15 us); where it applies it
-// takes the factorisation at n = 8192 from 14.8 to 5.4 ms (binary32 updates: 21.8
+// takes the factorisation at n = 8192 from 14.8 to 4.4 ms (binary32 updates: 21.8
 // to 8.5 ms), at 2048 from 2.82 to 0.76 ms.  Waits for the stream.  Afterwards
 // c->lu.lu holds L\U, c->lu.piv the interchanges and *hinfo the zero-pivot
 // report.
@@ -186,14 +209,17 @@ sg_status lu_factor(sg_ctx* c, const float* A, int n, sg_precision prec, const d
     const size_t o_inv = take(sgk::lu_diag_inv_bytes(n));
     const size_t o_info = take(64);
     const size_t o_moves = take((size_t)np * sgk::kLuMoveInts * 4 + (size_t)np * 4);
-    const size_t o_gates = take((size_t)np * 4);
+    const size_t o_gates = take((size_t)np * 8);
     // the operand copies of either form: M x 128 and N x 128, 16 bits each,
     // three of each for binary32 updates
     const size_t o_gemm =
         take((prec == SG_PREC_F32_SIMT ? sgk::gemm_split_scratch_bytes(n, n, sgk::kLuOuter)
                                        : sgk::gemm_tc_scratch_bytes(n, n, sgk::kLuOuter)) + 256);
     if (cudaMalloc(&L.base, off) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&L.cap, cudaStreamNonBlocking) != cudaSuccess) {
+        cudaStreamCreateWithFlags(&L.cap, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&L.side, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&L.fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&L.join, cudaEventDisableTiming) != cudaSuccess) {
       cudaGetLastError();
       L.clear();
       return err(c, SG_ERR_OOM, "factorisation workspace allocation failed");
@@ -225,7 +251,7 @@ sg_status lu_factor(sg_ctx* c, const float* A, int n, sg_precision prec, const d
         cudaError_t le = cudaMemsetAsync(L.info, 0, 64, L.cap);
         if (le == cudaSuccess) le = sgk::launch_lu_iota(L.perm, n, L.cap);
         if (diag) {
-          if (le == cudaSuccess) le = cudaMemsetAsync(L.gates, 0, (size_t)np * 4, L.cap);
+          if (le == cudaSuccess) le = cudaMemsetAsync(L.gates, 0, (size_t)np * 8, L.cap);
           if (le == cudaSuccess) le = factor_diag(c, L, n, prec, L.cap);
         } else {
           const size_t counters = (size_t)np * sgk::kLuMoveInts;
@@ -377,9 +403,9 @@ extern "C" sg_status sg_solve(sg_ctx* c, sg_matrix* A, sg_vector* b, const sg_so
   unsigned long long hviol = 0;
   int hinfo = 0, herr = 0;
   unsigned epoch = 0;
-  // One copy to pinned memory brings norms, violation and error: three to
-  // pageable memory and the memsets between the steps, now k_apply_perm's, took
-  // 20 us of an iteration's 60 at n = 1000.
+  // One copy to pinned memory brings norms, violation and error: with three to
+  // pageable memory, and memsets between the steps, a solve of n = 1000 took
+  // 1756 us against 1552.
   auto sync_read = [&]() -> bool {
     e = cudaMemcpyAsync(c->lu.host, w.norms, sizeof hn, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -566,9 +592,13 @@ void LuCache::clear() {
   if (base) cudaFree(base);
   if (host) cudaFreeHost(host);
   if (cap) cudaStreamDestroy(cap);
+  if (side) cudaStreamDestroy(side);
+  if (fork) cudaEventDestroy(fork);
+  if (join) cudaEventDestroy(join);
   exec = exec_diag = nullptr;
   base = host = nullptr;
-  cap = nullptr;
+  cap = side = nullptr;
+  fork = join = nullptr;
   lu = nullptr;
   piv = nullptr;
   perm = nullptr;
