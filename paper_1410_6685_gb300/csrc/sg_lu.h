@@ -37,9 +37,10 @@ cudaError_t launch_lu_trsm_outer(float* LU, int n, int K, int KB, int c0, int c1
 cudaError_t launch_lu_iota(int* perm, int n, cudaStream_t s);
 // y = U^-1 L^-1 P rhs in binary32 (P rhs gathered through perm).
 // Clears norms[1] and norms[2].
-// flags: 2*ceil(n/128) words (or more) that never hold `epoch` before the call.
+// words: n of them, whose high halves hold neither 2 epoch nor 2 epoch + 1
+// before the call.
 cudaError_t launch_lu_solve(const float* LU, const float* inv, int n, const int* perm,
-                            const double* rhs, float* y, unsigned* flags, unsigned epoch,
+                            const double* rhs, float* y, unsigned long long* words, unsigned epoch,
                             unsigned* tickets, double* norms, int* err, cudaStream_t s,
                             Prof* prof);
 // inv: lu_diag_inv_bytes(n): the inverses of the 128 x 128 diagonal blocks of L

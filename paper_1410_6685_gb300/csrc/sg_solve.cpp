@@ -41,7 +41,7 @@ struct SolveWork {
   int* piv;
   float* y;
   double* r;
-  unsigned* flags;
+  unsigned long long* words;   // the substitutions' exchange
   unsigned* tickets;
   int* dev_err;
   int* info;
@@ -356,7 +356,7 @@ extern "C" sg_status sg_solve(sg_ctx* c, sg_matrix* A, sg_vector* b, const sg_so
   };
   const size_t o_y = take((size_t)n * 4);
   const size_t o_r = take((size_t)n * 8);
-  const size_t o_flags = take((size_t)2 * nb * 4);
+  const size_t o_words = take((size_t)n * 8);
   const size_t o_tk = take(64);
   const size_t o_norms = take(8 * 8 + 16);   // norms, then viol and dev_err: read back together
   char* base = nullptr;
@@ -368,7 +368,7 @@ extern "C" sg_status sg_solve(sg_ctx* c, sg_matrix* A, sg_vector* b, const sg_so
   SolveWork w;
   w.y = reinterpret_cast<float*>(base + o_y);
   w.r = reinterpret_cast<double*>(base + o_r);
-  w.flags = reinterpret_cast<unsigned*>(base + o_flags);
+  w.words = reinterpret_cast<unsigned long long*>(base + o_words);
   w.tickets = reinterpret_cast<unsigned*>(base + o_tk);
   w.norms = reinterpret_cast<double*>(base + o_norms);
   w.viol = reinterpret_cast<unsigned long long*>(w.norms + 8);
@@ -417,7 +417,7 @@ extern "C" sg_status sg_solve(sg_ctx* c, sg_matrix* A, sg_vector* b, const sg_so
   };
 
   // 1. factorisation of a copy of A (the context's cached graph)
-  e = cudaMemsetAsync(base + o_flags, 0, o_norms + sizeof hn - o_flags, s);
+  e = cudaMemsetAsync(base + o_words, 0, o_norms + sizeof hn - o_words, s);
   if (e == cudaSuccess) e = sgk::launch_anorm(a, n, w.norms, s);
   if (e == cudaSuccess) {
     status = lu_factor(c, a, n, o.precision, w.norms, &hinfo);
@@ -442,7 +442,7 @@ extern "C" sg_status sg_solve(sg_ctx* c, sg_matrix* A, sg_vector* b, const sg_so
   // 2. initial solve, 3. refinement
   bool converged = false;
   if (!status) {
-    e = sgk::launch_lu_solve(w.lu, c->lu.inv, n, c->lu.perm, bb, w.y, w.flags, ++epoch, w.tickets,
+    e = sgk::launch_lu_solve(w.lu, c->lu.inv, n, c->lu.perm, bb, w.y, w.words, ++epoch, w.tickets,
                              w.norms, w.dev_err, s, prof);
     if (e == cudaSuccess) e = sgk::launch_update(x, w.y, bb, n, true, w.norms, s);
     c->kernels += 4;
@@ -450,7 +450,7 @@ extern "C" sg_status sg_solve(sg_ctx* c, sg_matrix* A, sg_vector* b, const sg_so
     for (int it = 0; it < o.max_iter && e == cudaSuccess; ++it) {
       e = sgk::launch_residual(a, n, bb, x, w.r, w.norms, 0.0, nullptr, s, prof);
       if (e == cudaSuccess)
-        e = sgk::launch_lu_solve(w.lu, c->lu.inv, n, c->lu.perm, w.r, w.y, w.flags, ++epoch,
+        e = sgk::launch_lu_solve(w.lu, c->lu.inv, n, c->lu.perm, w.r, w.y, w.words, ++epoch,
                                  w.tickets, w.norms, w.dev_err, s, prof);
       if (e == cudaSuccess) e = sgk::launch_update(x, w.y, bb, n, false, w.norms, s);
       c->kernels += 5;
