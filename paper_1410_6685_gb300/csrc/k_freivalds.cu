@@ -18,6 +18,29 @@
 
 namespace sgk {
 namespace {
+int sm_count() {
+  static const int sms = [] {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
+      v = 1;
+    return v;
+  }();
+  return sms;
+}
+}  // namespace
+
+// Groups of eight rows per CTA of the passes over A, B and C (a CTA loads its
+// vectors once): as many of four as leave a CTA for each SM.  N = 1000: 125
+// CTAs of one group 5.8 us (B) and 7.3 us (A and C), 32 CTAs of four 13.8 and 20.4
+// us; at 4096 four groups 18.0 and 39.8 us, one 23.1 and 42.9 us.
+int frv_row_groups(int stripes, int N) {
+  for (int g = 4; g > 1; g /= 2)
+    if ((long long)stripes * ((N + 8 * g - 1) / (8 * g)) >= sm_count()) return g;
+  return 1;
+}
+
+namespace {
 
 using frv::ldv;
 using frv::ldvec;
@@ -46,12 +69,6 @@ __global__ void k_frv_r(float4* r4, int N, int nvec, unsigned long long seed) {
   }
 }
 
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 constexpr int kRows = 8;            // rows per CTA (their loads issued together)
 constexpr int kWarps = 8;           // warps per CTA, side by side along a row
 constexpr int kWB = 256;            // columns per warp in the B pass (8 per lane)
@@ -59,12 +76,11 @@ constexpr int kWAC = 128;           // columns per warp in the A/C pass (4 per l
 constexpr int kSwB = kWarps * kWB;  // stripe width of a CTA, B pass
 constexpr int kSwAC = kWarps * kWAC;
 
-constexpr int kIters = 4;   // row groups of kRows per CTA (vectors loaded once)
-
 // partials over column stripes of B:  pb[s][k] = (sum_j B[k][j] r_v[j] for v<4,
 // sum_j B[k][j]^2), j in stripe s; the warps' shares are added in warp order
 __global__ void __launch_bounds__(256, 2) k_frv_b(const float* __restrict__ B, int N,
-                                                  const float4* __restrict__ r4, float* pb) {
+                                                  const float4* __restrict__ r4, float* pb,
+                                                  int iters) {
   __shared__ float red[2][kWarps][kRows][5];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int stripe = blockIdx.x;
@@ -75,8 +91,8 @@ __global__ void __launch_bounds__(256, 2) k_frv_b(const float* __restrict__ B, i
   for (int e = 0; e < 8; ++e) r[e] = ldvec(r4, c0 + e, N);
   const int slot = (lane >> 2) & 7;
 #pragma unroll 1
-  for (int it = 0; it < kIters; ++it) {
-    const long long row0 = ((long long)blockIdx.y * kIters + it) * kRows;
+  for (int it = 0; it < iters; ++it) {
+    const long long row0 = ((long long)blockIdx.y * iters + it) * kRows;
     if (row0 >= N) break;
     float4 b[kRows][2];
 #pragma unroll
@@ -120,6 +136,7 @@ __global__ void k_frv_b_reduce(const float* __restrict__ pb, int N, int nstripes
   const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (k >= N) return;
   float o[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
   for (int s = 0; s < nstripes; ++s) {
 #pragma unroll
     for (int t = 0; t < 5; ++t) o[t] += pb[((long long)s * N + k) * 5 + t];
@@ -134,7 +151,7 @@ __global__ void __launch_bounds__(256, 2) k_frv_ac(const float* __restrict__ A,
                                                    const float* __restrict__ C, int N,
                                                    const float4* __restrict__ r4,
                                                    const float4* __restrict__ br4,
-                                                   const float4* __restrict__ t4, float* pac) {
+                                                   const float4* __restrict__ t4, float* pac, int iters) {
   __shared__ float red[2][kWarps][kRows][12];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int stripe = blockIdx.x;
@@ -149,8 +166,8 @@ __global__ void __launch_bounds__(256, 2) k_frv_ac(const float* __restrict__ A,
   }
   const int slot = (lane >> 1) & 15;
 #pragma unroll 1
-  for (int it = 0; it < kIters; ++it) {
-    const long long row0 = ((long long)blockIdx.y * kIters + it) * kRows;
+  for (int it = 0; it < iters; ++it) {
+    const long long row0 = ((long long)blockIdx.y * iters + it) * kRows;
     if (row0 >= N) break;
     float4 av[kRows], cv[kRows];
 #pragma unroll
@@ -308,17 +325,30 @@ cudaError_t launch_freivalds(const float* A, const float* B, const float* C, int
   float* pb = reinterpret_cast<float*>(q);
   q += align256((size_t)nsb * N * 5 * sizeof(float));
   float* pac = reinterpret_cast<float*>(q);
-  const int rowblocks = (N + kRows * kIters - 1) / (kRows * kIters);
+  const int gb = frv_row_groups(nsb, N), ga = frv_row_groups(nsa, N);
+  auto blocks = [&](int groups) { return (N + kRows * groups - 1) / (kRows * groups); };
   prof_begin(prof, "freivalds", st);
   k_frv_r<<<(N + 255) / 256, 256, 0, st>>>(r4, N, nvec, seed);
-  k_frv_b<<<dim3(nsb, rowblocks), 256, 0, st>>>(B, N, r4, pb);
+  k_frv_b<<<dim3(nsb, blocks(gb)), 256, 0, st>>>(B, N, r4, pb, gb);
   k_frv_b_reduce<<<(N + 255) / 256, 256, 0, st>>>(pb, N, nsb, br4, t4);
-  k_frv_ac<<<dim3(nsa, rowblocks), 256, 0, st>>>(A, C, N, r4, br4, t4, pac);
+  k_frv_ac<<<dim3(nsa, blocks(ga)), 256, 0, st>>>(A, C, N, r4, br4, t4, pac, ga);
   k_frv_check<<<(N + 255) / 256, 256, 0, st>>>(pac, N, nsa, nvec, c, u_eff, res);
   prof_end(prof, st);
   *kernels += 5;
   return cudaGetLastError();
 }
+
+namespace {
+// Columns of B per CTA of its cast (with 64 rows): as many of kFrvStripeB as
+// leave CTAs for two thirds of the SMs, since each stripe is one more partial
+// sum per row (N = 1000: 512 / 256 / 128 / 64 columns 12.9 / 8.0 / 5.8 / 5.3 us;
+// 8192: 84.7 / 90.6 / 106 / 139 us).
+int stripe_b(int N) {
+  for (int w = kFrvStripeB; w > 64; w /= 2)
+    if (3LL * ((N + w - 1) / w) * ((N + 63) / 64) >= 2LL * sm_count()) return w;
+  return 64;
+}
+}  // namespace
 
 FrvFused frv_fused_layout(void* scratch, int N, int tile_c) {
   FrvFused f;
@@ -328,7 +358,8 @@ FrvFused frv_fused_layout(void* scratch, int N, int tile_c) {
   f.br4 = reinterpret_cast<float4*>(p + one);
   f.t4 = reinterpret_cast<float4*>(p + 2 * one);
   p += 3 * one;
-  f.nsb = (N + kFrvStripeB - 1) / kFrvStripeB;
+  f.stripe_b = stripe_b(N);
+  f.nsb = (N + f.stripe_b - 1) / f.stripe_b;
   f.nsa = (N + kFrvStripeA - 1) / kFrvStripeA;
   f.nsc = (N + tile_c - 1) / tile_c;
   f.pb = reinterpret_cast<float*>(p);

@@ -501,15 +501,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc2(const __grid_const
 }
 
 // Square B (N x N) -> Bt (N x Kp) 16-bit, with the fused Freivalds partial
-// sums of row k over this CTA's stripe of kFrvStripeB columns:
+// sums of row k over this CTA's stripe of `stripe` columns:
 // pb[stripe][k] = (sum_j B[k][j] r_v[j], v < 4;  sum_j B[k][j]^2).
-// CTA: 64 rows of B, eight 64-column sub-tiles in turn, each staged in
+// CTA: 64 rows of B, the stripe's 64-column sub-tiles in turn, each staged in
 // shared memory and written out transposed in 16-byte runs along k.
 template <bool FP16>
 __global__ void __launch_bounds__(256) k_cast_bt_frv(const float* __restrict__ B, int N, int Kp,
                                                      uint16_t* __restrict__ out,
                                                      const float4* __restrict__ r4,
-                                                     float* __restrict__ pb) {
+                                                     float* __restrict__ pb, int stripe) {
   __shared__ float t[64][65];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int k0 = blockIdx.y * 64;
@@ -541,10 +541,10 @@ __global__ void __launch_bounds__(256) k_cast_bt_frv(const float* __restrict__ B
     }
   };
   float nb0[8], nb1[8];
-  load(blockIdx.x * kFrvStripeB, nb0, nb1);
+  load(blockIdx.x * stripe, nb0, nb1);
 #pragma unroll 1
-  for (int st = 0; st < kFrvStripeB / 64; ++st) {
-    const int n0 = blockIdx.x * kFrvStripeB + st * 64;
+  for (int st = 0; st < stripe / 64; ++st) {
+    const int n0 = blockIdx.x * stripe + st * 64;
     if (n0 >= N) break;   // the same for the whole CTA
     const int nc = n0 + 2 * lane;
     const float4 r0 = frv::ldvec(r4, nc, N), r1 = frv::ldvec(r4, nc + 1, N);
@@ -554,7 +554,7 @@ __global__ void __launch_bounds__(256) k_cast_bt_frv(const float* __restrict__ B
       b0[i] = nb0[i];
       b1[i] = nb1[i];
     }
-    if (st + 1 < kFrvStripeB / 64) load(n0 + 64, nb0, nb1);
+    if (st + 1 < stripe / 64) load(n0 + 64, nb0, nb1);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       acc[i][0] = fmaf(b1[i], r1.x, fmaf(b0[i], r0.x, acc[i][0]));
@@ -598,13 +598,13 @@ __global__ void __launch_bounds__(256) k_cast_bt_frv(const float* __restrict__ B
 // partial sums of row i over this CTA's stripe of kFrvStripeA columns:
 // pzq[stripe][i] = (sum_k a_ik br_v[k], v < 4;  sum_k a_ik^2 t_v[k], v < 4).
 // Eight warps side by side along the row (4 columns per lane), 8 rows per
-// step, 4 steps per CTA.
+// step, `iters` steps per CTA.
 template <bool FP16>
 __global__ void __launch_bounds__(256, 2) k_cast_a_frv(const float* __restrict__ A, int N, int Kp,
                                                        uint16_t* __restrict__ out,
                                                        const float4* __restrict__ br4,
                                                        const float4* __restrict__ t4,
-                                                       float* __restrict__ pzq) {
+                                                       float* __restrict__ pzq, int iters) {
   __shared__ float red[2][8][8][8];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const long long c0 = (long long)blockIdx.x * kFrvStripeA + w * 128 + lane * 4;
@@ -626,15 +626,15 @@ __global__ void __launch_bounds__(256, 2) k_cast_a_frv(const float* __restrict__
     }
   };
   float4 nxt[8];
-  load8((long long)blockIdx.y * 32, nxt);
+  load8((long long)blockIdx.y * iters * 8, nxt);
 #pragma unroll 1
-  for (int it = 0; it < 4; ++it) {
-    const long long row0 = ((long long)blockIdx.y * 4 + it) * 8;
+  for (int it = 0; it < iters; ++it) {
+    const long long row0 = ((long long)blockIdx.y * iters + it) * 8;
     if (row0 >= N) break;
     float4 av[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) av[i] = nxt[i];
-    if (it < 3) load8(row0 + 8, nxt);
+    if (it + 1 < iters) load8(row0 + 8, nxt);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const long long row = row0 + i;
@@ -942,14 +942,15 @@ cudaError_t launch_gemm_tc_checked(const float* A, const float* B, float* C, int
   prof_begin(prof, "cast_operands", s);
   cudaError_t e = launch_frv_vectors(f, N, nvec, seed, s);
   if (e != cudaSuccess) return e;
-  const dim3 gb((N + kFrvStripeB - 1) / kFrvStripeB, Kp / 64);
-  const dim3 ga(f.nsa, (N + 31) / 32);
-  if (fp16) k_cast_bt_frv<true><<<gb, 256, 0, s>>>(B, N, Kp, bt16, f.r4, f.pb);
-  else k_cast_bt_frv<false><<<gb, 256, 0, s>>>(B, N, Kp, bt16, f.r4, f.pb);
+  const dim3 gb(f.nsb, Kp / 64);
+  const int groups = frv_row_groups(f.nsa, N);
+  const dim3 ga(f.nsa, (N + 8 * groups - 1) / (8 * groups));
+  if (fp16) k_cast_bt_frv<true><<<gb, 256, 0, s>>>(B, N, Kp, bt16, f.r4, f.pb, f.stripe_b);
+  else k_cast_bt_frv<false><<<gb, 256, 0, s>>>(B, N, Kp, bt16, f.r4, f.pb, f.stripe_b);
   e = launch_frv_b_reduce(f, N, s);
   if (e != cudaSuccess) return e;
-  if (fp16) k_cast_a_frv<true><<<ga, 256, 0, s>>>(A, N, Kp, a16, f.br4, f.t4, f.pzq);
-  else k_cast_a_frv<false><<<ga, 256, 0, s>>>(A, N, Kp, a16, f.br4, f.t4, f.pzq);
+  if (fp16) k_cast_a_frv<true><<<ga, 256, 0, s>>>(A, N, Kp, a16, f.br4, f.t4, f.pzq, groups);
+  else k_cast_a_frv<false><<<ga, 256, 0, s>>>(A, N, Kp, a16, f.br4, f.t4, f.pzq, groups);
   prof_end(prof, s);
   prof_begin(prof, fp16 ? "gemm_tc_f16" : "gemm_tc_bf16", s);
   e = launch_product(a16, bt16, Kp, fp16, C, N, N, N, false, err, f.r4, f.pw, inj_row, inj_col,

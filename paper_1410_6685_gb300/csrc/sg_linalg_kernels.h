@@ -85,7 +85,7 @@ cudaError_t launch_freivalds(const float* A, const float* B, const float* C, int
 // matrices: the cast of B also forms the partial sums of B r and |B_k|^2,
 // the cast of A those of A (B r) and (A.A) t, and the GEMM epilogue those of
 // C r, so the check reads no matrix a second time.  Partial sums are over
-// column stripes (kFrvStripeB of B, kFrvStripeA of A, tile_c of C) and are
+// column stripes (at most kFrvStripeB of B, kFrvStripeA of A, tile_c of C) and are
 // added in a fixed order by the final per-row test.
 constexpr int kFrvStripeB = 512;
 constexpr int kFrvStripeA = 1024;
@@ -97,9 +97,11 @@ struct FrvFused {
   float* pb;       // [nsb][N][5] partial B r and |B_k|^2
   float* pzq;      // [nsa][N][8] partial A (B r) and (A.A) t
   float4* pw;      // [nsc][N] partial C r
-  int nsb, nsa, nsc;
+  int nsb, nsa, nsc, stripe_b;
   size_t bytes;
 };
+// groups of eight rows per CTA where `stripes` CTAs stand side by side on N rows
+int frv_row_groups(int stripes, int N);
 FrvFused frv_fused_layout(void* scratch, int N, int tile_c);
 size_t frv_fused_scratch_bytes(int N);
 cudaError_t launch_frv_vectors(const FrvFused& f, int N, int nvec, unsigned long long seed,
