@@ -147,6 +147,7 @@ __device__ __forceinline__ void acc_one(Acc& a, float v, bool m) {
 )SGJIT";
 
 const char* kTemplateKernel = R"SGJIT(
+#define SG_U 2
 extern "C" __global__ void __launch_bounds__(256) sg_fused(const JitArgs a) {
   Acc acc;
   acc_init(acc);
@@ -161,13 +162,14 @@ extern "C" __global__ void __launch_bounds__(256) sg_fused(const JitArgs a) {
   if (a.vec4) {
     const long long nv = n >> 2;
     tail = nv << 2;
-    for (long long v = tid; v < nv; v += stride) {
-      float xs[SG_NX][4];
+    auto load = [&](long long v, float (&xs)[SG_NX][4]) {
 #pragma unroll
       for (int k = 0; k < SG_NIN; ++k) {
         const float4 t = __ldg(reinterpret_cast<const float4*>(a.in[k]) + v);
         xs[k][0] = t.x; xs[k][1] = t.y; xs[k][2] = t.z; xs[k][3] = t.w;
       }
+    };
+    auto eval = [&](long long v, const float (&xs)[SG_NX][4]) {
       float os[SG_NO][4];
       float rv[4];
       bool rm[4];
@@ -196,6 +198,20 @@ extern "C" __global__ void __launch_bounds__(256) sg_fused(const JitArgs a) {
 #pragma unroll
       for (int l = 0; l < 4; ++l) acc_one(acc, rv[l], rm[l]);
 #endif
+    };
+    // SG_U float4s of every input in flight per thread, side by side per CTA,
+    // once the grid has more than one each (a whole flush at n = 2^28 with one
+    // 503 us, two 494, four 498)
+    const int per = nv > stride ? SG_U : 1;
+    for (long long v = (long long)blockIdx.x * per * blockDim.x + threadIdx.x; v < nv;
+         v += stride * per) {
+      float xs[SG_U][SG_NX][4];
+#pragma unroll
+      for (int u = 0; u < SG_U; ++u)
+        if (u < per && v + u * blockDim.x < nv) load(v + u * blockDim.x, xs[u]);
+#pragma unroll
+      for (int u = 0; u < SG_U; ++u)
+        if (u < per && v + u * blockDim.x < nv) eval(v + u * blockDim.x, xs[u]);
     }
   }
   for (long long i = tail + tid; i < n; i += stride) {
@@ -235,6 +251,7 @@ extern "C" __global__ void __launch_bounds__(256) sg_fused(const JitArgs a) {
   __threadfence();
   Acc tot;
   acc_init(tot);
+#pragma unroll 4
   for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
     const PassResult* q = &a.partials[b];
     Acc p;

@@ -761,7 +761,7 @@ cudaError_t launch_stream_scheduled(sg_ctx* c, cudaKernel_t jk, const sgk::Strea
     } else {
       us.assign(cand.size(), 0.0);
       for (size_t i = 0; i < cand.size() && e == cudaSuccess; ++i) {
-        const int g = sg_stream_grid(w.n, cand[i], c->num_sms), b = (int)cand[i].chunk;
+        const int g = sg_stream_ctas(w.n, cand[i], c->num_sms), b = (int)cand[i].chunk;
         e = time_launch(c,
                         [&]() {
                           c->kernels += 1;
@@ -777,7 +777,7 @@ cudaError_t launch_stream_scheduled(sg_ctx* c, cudaKernel_t jk, const sgk::Strea
     }
   }
   sg_sched_note(c, SG_SCHED_STREAM, cand, us, def, learned, idx, pred);
-  return sgk::launch_jit_stream(jk, a, sg_stream_grid(w.n, cand[idx], c->num_sms),
+  return sgk::launch_jit_stream(jk, a, sg_stream_ctas(w.n, cand[idx], c->num_sms),
                                 (int)cand[idx].chunk, c->stream, &c->prof);
 }
 
@@ -883,7 +883,7 @@ sg_status run_flush(sg_ctx* c, bool fuse, bool commit, double* us) {
     for (Pass& P : passes) {
       switch (P.kind) {
         case PK::STREAM:
-          work = std::max(work, (size_t)std::max(stream_grid(c, P), c->num_sms * 8) *
+          work = std::max(work, (size_t)std::max(stream_grid(c, P), c->num_sms * 8 * kStreamWaves) *
                                     sizeof(sgk::PassResult));
           break;
         case PK::SORT: work = std::max(work, sgk::sort_scratch_bytes(P.n)); break;

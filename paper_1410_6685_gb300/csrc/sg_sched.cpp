@@ -96,6 +96,18 @@ int sg_stream_grid(long long n, const sg_sched_choice& ch, int num_sms) {
   return (int)std::max<long long>(1, std::min<long long>(want, (long long)num_sms * ch.blocks_per_sm));
 }
 
+// The launch's CTAs: the grid, or up to four times as many once each still has
+// sixteen steps.  The CTAs of one long wave drift apart, and the DRAM pages they
+// use with them: z = x + y alone at n = 2^28 takes 482-500 us with 1216 CTAs (8
+// per SM), 469 with two waves, 457 with seven, 449 with one step per CTA; with the
+// check and the sum, whose partial results are one per CTA, a whole flush takes
+// 524 us with one wave, 507 with two, 492-500 with three, four and seven.
+int sg_stream_ctas(long long n, const sg_sched_choice& ch, int num_sms) {
+  const int g = sg_stream_grid(n, ch, num_sms);
+  const long long steps = (n + 3) / 4 / ((long long)g * ch.chunk);
+  return g * (int)std::max<long long>(1, std::min<long long>(kStreamWaves, steps / 16));
+}
+
 std::vector<sg_sched_choice> sg_stream_candidates(long long n, int num_sms) {
   std::vector<sg_sched_choice> out;
   for (int t : kStreamThreads)

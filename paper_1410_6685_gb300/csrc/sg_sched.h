@@ -58,6 +58,9 @@ void sg_batch_features(const BatchStats& w, const sg_sched_choice& ch, int num_s
 std::vector<sg_sched_choice> sg_stream_candidates(long long n, int num_sms);
 sg_sched_choice sg_stream_default();
 int sg_stream_grid(long long n, const sg_sched_choice& ch, int num_sms);
+// the CTAs launched for it: at most kStreamWaves times the grid
+constexpr int kStreamWaves = 4;
+int sg_stream_ctas(long long n, const sg_sched_choice& ch, int num_sms);
 void sg_stream_features(const StreamWork& w, const sg_sched_choice& ch, int num_sms, float* f);
 
 // The filter: tile items; occ = resident CTAs per SM of that tile's kernel
