@@ -207,23 +207,31 @@ __device__ __forceinline__ void fp_flush(unsigned long long f1, unsigned long lo
 
 // ---------------------------------------------------------------------------
 // FP: also the input's multiset fingerprint (only the permutation check
-// needs it)
-template <bool FLT, bool FP>
-__global__ void __launch_bounds__(256) k_radix_hist(const int* __restrict__ in, long long n,
-                                                    SortHdr* h, SortResult* res) {
-  __shared__ unsigned sh[4][kRadix];
-  for (int i = threadIdx.x; i < 4 * kRadix; i += blockDim.x) (&sh[0][0])[i] = 0;
+// needs it).  LANES: a counter per digit and lane (128 KB, one CTA of 1024
+// threads per SM), so that no two lanes of a warp's shared-memory atomic meet in
+// a bank; with one counter per digit the four atomics of 32 uniform keys take
+// three to four turns each, which bounded the pass (2^26 keys: 105 -> 62 us; 2^22
+// 15.7 -> 12.6 us).  Below kLaneKeys clearing and adding up the counters costs more
+// than it saves.
+constexpr long long kLaneKeys = 1 << 22;
+template <bool FLT, bool FP, bool LANES>
+__global__ void __launch_bounds__(LANES ? 1024 : 256, 1) k_radix_hist(const int* __restrict__ in,
+                                                                      long long n, SortHdr* h,
+                                                                      SortResult* res) {
+  constexpr int kCopies = LANES ? 32 : 1, kThreads = LANES ? 1024 : 256;
+  extern __shared__ unsigned sh[];   // [4 * kRadix][kCopies]
+  for (int i = threadIdx.x; i < 4 * kRadix * kCopies; i += kThreads) sh[i] = 0;
   __syncthreads();
   unsigned long long f1 = 0, f2 = 0;
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long stride = (long long)gridDim.x * blockDim.x;
+  unsigned* const mine = sh + (LANES ? threadIdx.x & 31 : 0);
   long long start = 0;
   auto count = [&](int k) {
     const unsigned u = okey<FLT>(k);
-    atomicAdd(&sh[0][u & 0xFFu], 1u);
-    atomicAdd(&sh[1][(u >> 8) & 0xFFu], 1u);
-    atomicAdd(&sh[2][(u >> 16) & 0xFFu], 1u);
-    atomicAdd(&sh[3][u >> 24], 1u);
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+      atomicAdd(&mine[(p * kRadix + ((u >> (8 * p)) & 0xFFu)) * kCopies], 1u);
     if (FP) fp_add(f1, f2, k);
   };
   if (((uintptr_t)in & 15) == 0) {
@@ -231,11 +239,16 @@ __global__ void __launch_bounds__(256) k_radix_hist(const int* __restrict__ in, 
     start = nv << 2;
     const int4* in4 = reinterpret_cast<const int4*>(in);
     long long v = tid;
-    // two 16-byte loads in flight per thread before their keys are counted
-    for (; v + stride < nv; v += 2 * stride) {
-      const int4 q0 = __ldcs(in4 + v), q1 = __ldcs(in4 + v + stride);
-      count(q0.x); count(q0.y); count(q0.z); count(q0.w);
-      count(q1.x); count(q1.y); count(q1.z); count(q1.w);
+    // 64 KB of loads in flight per SM before their keys are counted
+    constexpr int kLoads = LANES ? 4 : 2;
+    for (; v + (kLoads - 1) * stride < nv; v += kLoads * stride) {
+      int4 q[kLoads];
+#pragma unroll
+      for (int i = 0; i < kLoads; ++i) q[i] = __ldcs(in4 + v + i * stride);
+#pragma unroll
+      for (int i = 0; i < kLoads; ++i) {
+        count(q[i].x); count(q[i].y); count(q[i].z); count(q[i].w);
+      }
     }
     for (; v < nv; v += stride) {
       const int4 q = __ldcs(in4 + v);
@@ -243,11 +256,13 @@ __global__ void __launch_bounds__(256) k_radix_hist(const int* __restrict__ in, 
     }
   }
   for (long long i = start + tid; i < n; i += stride) count(in[i]);
-  __shared__ unsigned long long s_fp[2 * 8];
+  __shared__ unsigned long long s_fp[2 * kThreads / 32];
   if (FP) fp_flush(f1, f2, res->fp_in, s_fp);
   __syncthreads();
-  for (int i = threadIdx.x; i < 4 * kRadix; i += blockDim.x) {
-    const unsigned c = (&sh[0][0])[i];
+  for (int i = threadIdx.x; i < 4 * kRadix; i += kThreads) {
+    unsigned c = 0;
+#pragma unroll
+    for (int q = 0; q < kCopies; ++q) c += sh[i * kCopies + ((q + i) & (kCopies - 1))];
     if (c) atomicAdd(&(&h->hist[0][0])[i], c);
   }
   __shared__ bool am_last;
@@ -258,14 +273,16 @@ __global__ void __launch_bounds__(256) k_radix_hist(const int* __restrict__ in, 
   if (!am_last) return;
   __threadfence();
   // per-digit start offsets: one exclusive scan over the block per histogram
-  // (thread d owns digit d)
-  __shared__ unsigned s_warp[kWarps];
+  // (thread d owns digit d; threads past the digits only keep the barriers)
+  __shared__ unsigned s_warp[kThreads / 32];
+  const bool own = threadIdx.x < kRadix;
   unsigned c[4];
 #pragma unroll
-  for (int p = 0; p < 4; ++p) c[p] = __ldcg(&h->hist[p][threadIdx.x]);
+  for (int p = 0; p < 4; ++p) c[p] = own ? __ldcg(&h->hist[p][threadIdx.x]) : 0u;
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
-    h->offs[p][threadIdx.x] = block_excl_scan(c[p], s_warp);
+    const unsigned o = block_excl_scan(c[p], s_warp);
+    if (own) h->offs[p][threadIdx.x] = o;
     __syncthreads();
   }
   if (threadIdx.x == 0) res->cnt_in = n;
@@ -668,6 +685,22 @@ size_t sort_scratch_bytes(long long n) { return layout(n).total; }
 
 namespace {
 
+template <bool FLT, bool FP>
+cudaError_t launch_hist(const int32_t* in, long long n, SortHdr* h, SortResult* res, int num_sms,
+                        cudaStream_t s) {
+  if (n < kLaneKeys) {
+    k_radix_hist<FLT, FP, false><<<grid_for((n + 3) / 4 / 8, num_sms, 8), 256,
+                                   4 * kRadix * sizeof(unsigned), s>>>(in, n, h, res);
+    return cudaGetLastError();
+  }
+  constexpr int kSmem = 4 * kRadix * 32 * (int)sizeof(unsigned);
+  const cudaError_t e = cudaFuncSetAttribute(k_radix_hist<FLT, FP, true>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  if (e != cudaSuccess) return e;
+  k_radix_hist<FLT, FP, true><<<num_sms, 1024, kSmem, s>>>(in, n, h, res);
+  return cudaGetLastError();
+}
+
 template <bool FLT, int KPT, int LOOK>
 cudaError_t sort_impl(const int32_t* in, int32_t* out, long long n, bool contracts,
                         void* scratch, SortResult* res, cudaStream_t s, int num_sms,
@@ -684,13 +717,12 @@ cudaError_t sort_impl(const int32_t* in, int32_t* out, long long n, bool contrac
   cudaError_t e = cudaMemsetAsync(base, 0, L.zero_bytes, s);
   if (e != cudaSuccess) return e;
   prof_begin(prof, "radix_hist", s);
-  if (contracts)
-    k_radix_hist<FLT, true><<<grid_for((n + 3) / 4 / 8, num_sms, 8), 256, 0, s>>>(in, n, h, res);
-  else
-    k_radix_hist<FLT, false><<<grid_for((n + 3) / 4 / 8, num_sms, 8), 256, 0, s>>>(in, n, h, res);
+  e = contracts ? launch_hist<FLT, true>(in, n, h, res, num_sms, s)
+                : launch_hist<FLT, false>(in, n, h, res, num_sms, s);
   prof_end(prof, s);
   constexpr int kTile = kSortBlock * KPT;
   const unsigned ntiles = (unsigned)((n + kTile - 1) / kTile);
+  if (e != cudaSuccess) return e;
   const unsigned ahead = (unsigned)num_sms * kSortMinBlocks;
   prof_begin(prof, "onesweep", s);
   k_onesweep<false, false, FLT, KPT, LOOK><<<ntiles, kSortBlock, 0, s>>>(in, tmp, n, 0, h, st32[0], st64, res, ahead, lb);
