@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool ok = true;
       for (int t = unit; t < ntiles && ok; t += nunits) {
         int bm, bn;
-        tile_coords(t, nM, nN, &bm, &bn);
+        tile_coords(t, nM, nN, &bm, &bn, SUB);
         const int m0 = bm * F::kTileM + (int)rank * 128;
         const int n0 = bn * TN + (int)rank * F::kBRows;
         for (int kb = 0; kb < KB; ++kb, ++it) {
@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool ok = true;
     for (int t = unit; t < ntiles && ok; t += nunits) {
       int bm, bn;
-      tile_coords(t, nM, nN, &bm, &bn);
+      tile_coords(t, nM, nN, &bm, &bn, SUB);
       const int m0q = bm * F::kTileM + (int)rank * 128 + q * 32, c0 = bn * TN + hh * HN;
       if (SUB) prefetch_c_row(C, ldc, M, N, m0q + lane, c0, HN);
       float sum[HN];
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint32_t r[32];
 #pragma unroll
         for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(sum[c * 32 + j]);
-        store_chunk(C, ldc, M, N, m0q, c0 + c * 32, r, s_tw, lane, SUB ? 1 : 0, cv);
+        store_chunk<SUB>(C, ldc, M, N, m0q, c0 + c * 32, r, s_tw, lane, cv);
       }
     }
   }

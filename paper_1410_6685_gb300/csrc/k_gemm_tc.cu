@@ -87,14 +87,14 @@ __host__ __device__ constexpr uint32_t idesc(bool fp16, int tn) {
 // its last chunk is read; the fused check's partial C r of its rows over its
 // half goes to column tile 2 bn + hh of frv_pw.  false: the wait for the
 // accumulator gave up.
-template <bool CL, int TNv>
+template <bool CL, int TNv, bool SUB>
 __device__ __forceinline__ bool epilogue_tile(
     uint32_t tmem, int acc, int tl, uint32_t tfull, uint32_t tempty, int q, int hh, int m0q,
-    int n0, int bn, float* __restrict__ C, int ldc, int M, int N, int subtract,
+    int n0, int bn, float* __restrict__ C, int ldc, int M, int N,
     const float4* __restrict__ frv_r, float4* __restrict__ frv_pw, int inj_row, int inj_col,
     float inj_delta, float4* s_rw, float* s_tw, int lane, int* err, volatile int* abort_flag) {
   const int c0 = n0 + hh * (TNv / 2);
-  if (frv_r) {
+  if (!SUB && frv_r) {
     // each epilogue warp keeps its own copy, so no barrier spans the warps
     __syncwarp();
     for (int j = lane; j < TNv / 2; j += 32)
@@ -109,7 +109,7 @@ __device__ __forceinline__ bool epilogue_tile(
   for (int c = 0; c < TNv / 64; ++c) {
     const int col0 = c0 + c * 32;
     float4 cv[8];
-    if (subtract) load_c(C, ldc, M, N, m0q, col0, lane, cv);
+    if (SUB) load_c(C, ldc, M, N, m0q, col0, lane, cv);
     uint32_t r[32];
     tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * TNv + col0 - n0), r);
     if (c == TNv / 64 - 1) {
@@ -125,12 +125,12 @@ __device__ __forceinline__ bool epilogue_tile(
     }
     // contract testing: a planted error in one product element, applied
     // before it is stored (and before the fused check sees it)
-    if (row == inj_row && inj_col >= col0 && inj_col < col0 + 32) {
+    if (!SUB && row == inj_row && inj_col >= col0 && inj_col < col0 + 32) {
 #pragma unroll
       for (int j = 0; j < 32; ++j)
         if (col0 + j == inj_col) r[j] = __float_as_uint(__uint_as_float(r[j]) + inj_delta);
     }
-    if (frv_r) {
+    if (!SUB && frv_r) {
       // r of columns past N is zero in s_r (their accumulator entries are too)
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
@@ -142,9 +142,9 @@ __device__ __forceinline__ bool epilogue_tile(
         wacc.w = fmaf(v, rj.w, wacc.w);
       }
     }
-    store_chunk(C, ldc, M, N, m0q, col0, r, s_tw, lane, subtract, cv);
+    store_chunk<SUB>(C, ldc, M, N, m0q, col0, r, s_tw, lane, cv);
   }
-  if (frv_r && row < M && c0 < N) frv_pw[(size_t)(2 * bn + hh) * M + row] = wacc;
+  if (!SUB && frv_r && row < M && c0 < N) frv_pw[(size_t)(2 * bn + hh) * M + row] = wacc;
   return true;
 }
 
@@ -158,11 +158,11 @@ __device__ __forceinline__ bool epilogue_tile(
 //                      and the column half (w - 2) / 4 of the tile;
 //                      after draining an accumulator they release it to the
 //                      MMA issuer through an mbarrier.
-template <int TNv>
+template <int TNv, bool SUB>
 __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc(const __grid_constant__ CUtensorMap ma,
                                                     const __grid_constant__ CUtensorMap mb,
                                                     float* __restrict__ C, int ldc, int M,
-                                                    int N, int KB, uint32_t id, int subtract,
+                                                    int N, int KB, uint32_t id,
                                                     int* err, const float4* __restrict__ frv_r,
                                                     float4* __restrict__ frv_pw, int inj_row,
                                                     int inj_col, float inj_delta,
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc(const __grid_consta
       bool ok = true;
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
         int bm, bn;
-        tile_coords(t, nM, nN, &bm, &bn);
+        tile_coords(t, nM, nN, &bm, &bn, SUB);
         const int m0 = bm * TM, n0 = bn * TNv;
         for (int kb = 0; kb < KB; ++kb, ++it) {
           const int s = it % STAGES;
@@ -293,16 +293,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc(const __grid_consta
     int tl = 0;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++tl) {
       int bm, bn;
-      tile_coords(t, nM, nN, &bm, &bn);
+      tile_coords(t, nM, nN, &bm, &bn, SUB);
       const int acc = tl & 1;
-      if (subtract && t + (int)gridDim.x < ntiles) {
+      if (SUB && t + (int)gridDim.x < ntiles) {
         int bm2, bn2;
-        tile_coords(t + (int)gridDim.x, nM, nN, &bm2, &bn2);
+        tile_coords(t + (int)gridDim.x, nM, nN, &bm2, &bn2, SUB);
         prefetch_c_row(C, ldc, M, N, bm2 * TM + q * 32 + lane, bn2 * TNv + hh * (TNv / 2), TNv / 2);
       }
-      const bool keep = corner && bm == 0 && bn * TNv + hh * (TNv / 2) < kCorner;
-      if (!epilogue_tile<false, TNv>(tmem, acc, tl, tfull0 + 8 * acc, tempty0 + 8 * acc, q, hh,
-                                bm * TM + q * 32, bn * TNv, bn, C, ldc, keep ? 0 : M, N, subtract, frv_r,
+      const bool keep = SUB && corner && bm == 0 && bn * TNv + hh * (TNv / 2) < kCorner;
+      if (!epilogue_tile<false, TNv, SUB>(tmem, acc, tl, tfull0 + 8 * acc, tempty0 + 8 * acc, q, hh,
+                                bm * TM + q * 32, bn * TNv, bn, C, ldc, keep ? 0 : M, N, frv_r,
                                 frv_pw, inj_row, inj_col, inj_delta, s_rw, s_tw, lane, err,
                                 abort_flag))
         break;
@@ -343,10 +343,11 @@ __host__ __device__ constexpr uint32_t idesc2(bool fp16) {
          ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(TM2 >> 4) << 24);
 }
 
+template <bool SUB>
 __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc2(const __grid_constant__ CUtensorMap ma,
                                                      const __grid_constant__ CUtensorMap mb,
                                                      float* __restrict__ C, int ldc, int M,
-                                                     int N, int KB, uint32_t id, int subtract,
+                                                     int N, int KB, uint32_t id,
                                                      int* err, const float4* __restrict__ frv_r,
                                                      float4* __restrict__ frv_pw, int inj_row,
                                                      int inj_col, float inj_delta,
@@ -403,7 +404,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc2(const __grid_const
       bool ok = true;
       for (int t = pair; t < ntiles && ok; t += npairs) {
         int bm, bn;
-        tile_coords(t, nM, nN, &bm, &bn);
+        tile_coords(t, nM, nN, &bm, &bn, SUB);
         const int m0 = bm * TM2 + (int)rank * TH, n0 = bn * TN + (int)rank * TH;
         for (int kb = 0; kb < KB; ++kb, ++it) {
           const int s = it % STAGES2;
@@ -473,19 +474,19 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_tc2(const __grid_const
     int tl = 0;
     for (int t = pair; t < ntiles; t += npairs, ++tl) {
       int bm, bn;
-      tile_coords(t, nM, nN, &bm, &bn);
+      tile_coords(t, nM, nN, &bm, &bn, SUB);
       const int acc = tl & 1;
-      if (subtract && t + npairs < ntiles) {
+      if (SUB && t + npairs < ntiles) {
         int bm2, bn2;
-        tile_coords(t + npairs, nM, nN, &bm2, &bn2);
+        tile_coords(t + npairs, nM, nN, &bm2, &bn2, SUB);
         prefetch_c_row(C, ldc, M, N, bm2 * TM2 + (int)rank * TH + q * 32 + lane,
                        bn2 * TN + hh * (TN / 2), TN / 2);
       }
-      const bool keep = corner && bm == 0 && bn == 0 && rank == 0 && hh == 0;
-      if (!epilogue_tile<true, TN>(tmem, acc, tl, tfull0 + 8 * acc, tempty_leader + 8 * acc, q, hh,
+      const bool keep = SUB && corner && bm == 0 && bn == 0 && rank == 0 && hh == 0;
+      if (!epilogue_tile<true, TN, SUB>(tmem, acc, tl, tfull0 + 8 * acc, tempty_leader + 8 * acc, q, hh,
                                bm * TM2 + (int)rank * TH + q * 32, bn * TN, bn, C, ldc, keep ? 0 : M, N,
-                               subtract, frv_r, frv_pw, inj_row, inj_col, inj_delta, s_rw, s_tw,
-                               lane, err, abort_flag))
+                               frv_r, frv_pw, inj_row, inj_col, inj_delta, s_rw, s_tw, lane,
+                               err, abort_flag))
         break;
     }
   }
@@ -717,7 +718,9 @@ bool use_pair() {
   static int v = -1;
   if (v < 0) {
     v = 0;
-    if (cudaFuncSetAttribute(k_gemm_tc2, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(k_gemm_tc2<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             SMEM2_BYTES) == cudaSuccess &&
+        cudaFuncSetAttribute(k_gemm_tc2<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              SMEM2_BYTES) == cudaSuccess) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(2);
@@ -731,7 +734,7 @@ bool use_pair() {
       cfg.attrs = at;
       cfg.numAttrs = 1;
       int nc = 0;
-      if (cudaOccupancyMaxActiveClusters(&nc, k_gemm_tc2, &cfg) == cudaSuccess && nc >= 1) v = 1;
+      if (cudaOccupancyMaxActiveClusters(&nc, k_gemm_tc2<true>, &cfg) == cudaSuccess && nc >= 1) v = 1;
     }
     cudaGetLastError();
   }
@@ -764,13 +767,14 @@ cudaError_t launch_one(const CUtensorMap& ma, const uint16_t* bt16, int Kp, bool
                        const int* skip, int corner) {
   CUtensorMap mb;
   if (!make_map(&mb, bt16, N, Kp, TNv, fp16)) return cudaErrorInvalidValue;
-  const cudaError_t e = cudaFuncSetAttribute(
-      k_gemm_tc<TNv>, cudaFuncAttributeMaxDynamicSharedMemorySize, One<TNv>::kSmem);
+  const auto fn = subtract ? k_gemm_tc<TNv, true> : k_gemm_tc<TNv, false>;
+  const cudaError_t e =
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, One<TNv>::kSmem);
   if (e != cudaSuccess) return e;
   const long long tiles = (long long)((M + TM - 1) / TM) * ((N + TNv - 1) / TNv);
   const int slots = std::max(1, sm_count() - (corner ? 2 : 0));
-  k_gemm_tc<TNv><<<(int)std::min<long long>(tiles, slots), kGemmThreads, One<TNv>::kSmem, s>>>(
-      ma, mb, C, ldc, M, N, (Kp / TK + One<TNv>::kSlices - 1) / One<TNv>::kSlices, idesc(fp16, TNv), subtract ? 1 : 0, err, frv_r, frv_pw,
+  fn<<<(int)std::min<long long>(tiles, slots), kGemmThreads, One<TNv>::kSmem, s>>>(
+      ma, mb, C, ldc, M, N, (Kp / TK + One<TNv>::kSlices - 1) / One<TNv>::kSlices, idesc(fp16, TNv), err, frv_r, frv_pw,
       inj_row, inj_col, inj_delta, skip, corner);
   return cudaGetLastError();
 }
@@ -801,8 +805,8 @@ cudaError_t launch_product(const uint16_t* a16, const uint16_t* bt16, int Kp, bo
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_gemm_tc2, ma, mb, C, ldc, M, N, Kp / TK, idesc2(fp16),
-                              subtract ? 1 : 0, err, frv_r, frv_pw, inj_row, inj_col, inj_delta,
+    return cudaLaunchKernelEx(&cfg, subtract ? k_gemm_tc2<true> : k_gemm_tc2<false>, ma, mb, C,
+                              ldc, M, N, Kp / TK, idesc2(fp16), err, frv_r, frv_pw, inj_row, inj_col, inj_delta,
                               skip, corner);
   }
   switch (one_cta_columns(M, N, Kp)) {

@@ -128,11 +128,28 @@ __device__ __forceinline__ void mbar_arrive_cl(uint32_t bar_cl) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar_cl) : "memory");
 }
 
+// An update's 32 x 32 chunk that lies inside M x N with 16-byte aligned rows, as
+// almost all do, is loaded and stored without a test or an address of its own
+// per access: with them a chunk took some 440 instructions of a warp, and the
+// updates, most of whose time the epilogue takes, were 7% slower.  (Products only
+// store; a second path cost them 5% at 1537 x 2049 x 1023.)
+__device__ __forceinline__ bool whole_chunk(const float* C, int ldc, int M, int N, int m0q,
+                                            int col0) {
+  return m0q + 32 <= M && col0 + 32 <= N &&
+         ((reinterpret_cast<uintptr_t>(C) | ((size_t)ldc * 4)) & 15) == 0;
+}
+
 // C rows m0q .. m0q + 31, columns col0 .. col0 + 31, as the epilogue's
 // stores take them: access it, lane l: row m0q + 4 it + l / 8, columns
 // col0 + 4 (l % 8) .. + 3 (zero outside M x N)
 __device__ __forceinline__ void load_c(const float* __restrict__ C, int ldc, int M, int N, int m0q,
                                        int col0, int lane, float4 (&cv)[8]) {
+  if (whole_chunk(C, ldc, M, N, m0q, col0)) {
+    const float* p = C + (size_t)(m0q + (lane >> 3)) * ldc + col0 + (lane & 7) * 4;
+#pragma unroll
+    for (int it = 0; it < 8; ++it) cv[it] = *reinterpret_cast<const float4*>(p + (size_t)it * 4 * ldc);
+    return;
+  }
 #pragma unroll
   for (int it = 0; it < 8; ++it) {
     const int grow = m0q + it * 4 + (lane >> 3), gcol = col0 + (lane & 7) * 4;
@@ -160,13 +177,15 @@ __device__ __forceinline__ void prefetch_c_row(const float* C, int ldc, int M, i
 }
 
 // One 32 x 32 chunk of the epilogue: lane l holds row m0q + l, columns
-// col0 .. col0 + 31 (r); C := chunk, or C := cv - chunk when subtracting (cv
-// from load_c), through the warp's transpose buffer s_tw (16 x 32 floats,
+// col0 .. col0 + 31 (r); C := chunk, or C := cv - chunk when SUB (cv from
+// load_c), through the warp's transpose buffer s_tw (16 x 32 floats,
 // rows 16 h .. 16 h + 15 in turn); rows outside M and columns outside N are
 // left alone.
+template <bool SUB>
 __device__ __forceinline__ void store_chunk(float* __restrict__ C, int ldc, int M, int N, int m0q,
                                             int col0, const uint32_t (&r)[32], float* s_tw,
-                                            int lane, int subtract, const float4 (&cv)[8]) {
+                                            int lane, const float4 (&cv)[8]) {
+  const bool whole = SUB && whole_chunk(C, ldc, M, N, m0q, col0);
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     if ((lane >> 4) == h) {
@@ -179,6 +198,21 @@ __device__ __forceinline__ void store_chunk(float* __restrict__ C, int ldc, int 
                                         __uint_as_float(r[4 * j + 3]));
     }
     __syncwarp();
+    if (whole) {
+      float* const p = C + (size_t)(m0q + 16 * h + (lane >> 3)) * ldc + col0 + (lane & 7) * 4;
+#pragma unroll
+      for (int it = 0; it < 4; ++it) {
+        const int rr = it * 4 + (lane >> 3);
+        const float4 v = reinterpret_cast<const float4*>(s_tw + rr * 32)[(lane & 7) ^ (rr & 7)];
+        const float4 c4 = cv[4 * h + it];
+        // an update's results are not needed again soon: they leave L2 first,
+        // which keeps the prefetched C there (4% of an update at n = 8192)
+        __stcs(reinterpret_cast<float4*>(p + (size_t)it * 4 * ldc),
+               make_float4(c4.x - v.x, c4.y - v.y, c4.z - v.z, c4.w - v.w));
+      }
+      __syncwarp();
+      continue;
+    }
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
       const int rr = it * 4 + (lane >> 3), g = lane & 7;
@@ -186,8 +220,7 @@ __device__ __forceinline__ void store_chunk(float* __restrict__ C, int ldc, int 
       const int grow = m0q + 16 * h + rr, gcol = col0 + 4 * g;
       if (grow >= M) continue;
       const float4 c4 = cv[4 * h + it];
-      const float4 o =
-          subtract ? make_float4(c4.x - v.x, c4.y - v.y, c4.z - v.z, c4.w - v.w) : v;
+      const float4 o = SUB ? make_float4(c4.x - v.x, c4.y - v.y, c4.z - v.z, c4.w - v.w) : v;
       float* cp = C + (size_t)grow * ldc + gcol;
       if (gcol + 4 <= N && ((reinterpret_cast<uintptr_t>(cp) & 15) == 0)) {
         *reinterpret_cast<float4*>(cp) = o;
@@ -206,9 +239,17 @@ __device__ __forceinline__ void store_chunk(float* __restrict__ C, int ldc, int 
 // group the row block varies fastest.  The 76 pairs' concurrent 256 x 256
 // tiles then span 8 row blocks x about 10 column blocks, whose A and B
 // slices (some 75 MB at K = 8192) stay in L2 instead of all of B (groups of
-// 8 measured 0.7% faster than 16, and 32 4% slower).
+// 8 measured 0.7% faster than 16, and 32 4% slower).  by_rows: the
+// elimination's updates, whose operands are narrow and whose traffic is C, go
+// along the rows of C (n = 8192: 1.5% faster than in groups).
 constexpr int kGroupM = 8;
-__device__ __forceinline__ void tile_coords(int t, int nM, int nN, int* mb, int* nb) {
+__device__ __forceinline__ void tile_coords(int t, int nM, int nN, int* mb, int* nb,
+                                            bool by_rows = false) {
+  if (by_rows) {
+    *mb = t / nN;
+    *nb = t - *mb * nN;
+    return;
+  }
   const int per_group = kGroupM * nN;
   const int g = t / per_group;
   const int first = g * kGroupM;
