@@ -2,10 +2,12 @@
 // partial pivoting) and the solve with iterative refinement (sm_103a).
 //
 // Right-looking blocked LU, panels of 32 columns:
-//   k_lu_panel_reg / k_lu_panel : a cluster of 16 CTAs (8 where the device
-//                  cannot schedule 16) holds the panel (rows k..n-1) -- in
-//                  registers (16 CTAs) or in shared memory (8 CTAs) -- and
-//                  eliminates it column by column.  Each
+//   k_lu_panel_rows : one CTA or a cluster of 8 or 16, one row of the panel per
+//                  thread (heights up to 4096);
+//   k_lu_panel_reg / k_lu_panel : above that a cluster of 16 CTAs, up to three
+//                  rows per thread in registers, or 8 CTAs with the panel in
+//                  shared memory where the device cannot schedule 16.  Each
+//                  eliminates its panel column by column.  Each
 //                  column costs one exchange: every CTA sends its best pivot
 //                  candidate (largest |a|, then the lowest current row
 //                  position) together with that row into every CTA's shared
@@ -25,14 +27,14 @@
 //   k_lu_trsm_outer  : U12 = L11^-1 A12 for the outer block (128 rows), L11
 //                  and a 32-column strip per CTA in shared memory.
 //   trailing update A22 -= L21 U12 (K = 128) : the tensor-core product
-//                  (bf16/fp16 operands, binary32 accumulate) or the binary32
-//                  SIMT form.
+//                  (bf16/fp16 operands, binary32 accumulate), or for binary32
+//                  updates three bf16 pieces per operand or the CUDA cores.
+// k_lu_diag.cu holds the form for matrices that need no interchange.
 // Solve: pivots on the right-hand side, then forward / backward substitution
 // by steps of 128 rows in one launch each: CTAs take steps in order
 // (ticket) and wait, with a bounded spin, for the steps they depend on; each
 // step's diagonal block is applied through its inverse (formed once per
-// factorisation), one short product
-// instead of 128 dependent steps.
+// factorisation), one short product instead of 128 dependent steps.
 // Refinement: residual r = b - A x in binary64 from the binary32 A, and the
 // update x += d with the norms the stopping test needs.
 #include <cooperative_groups.h>
