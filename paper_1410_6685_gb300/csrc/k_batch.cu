@@ -51,43 +51,45 @@ __global__ void __launch_bounds__(1024) k_batch_prep(const long long* __restrict
                                                      long long nseg, long long chunk,
                                                      long long capacity,
                                                      long long* chunk_start, BatchHdr* h) {
+  // one scan of the threads' totals, each over consecutive collections (a scan
+  // per 1024 collections, each behind its loads, took 14.5 us for 10,000)
   __shared__ long long s_warp[32];
   __shared__ long long s_carry;
-  if (threadIdx.x == 0) s_carry = 0;
-  __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (long long b = 0; b < nseg; b += blockDim.x) {
-    const long long s = b + threadIdx.x;
-    long long c = 0;
-    if (s < nseg) {
-      const long long L = off[s + 1] - off[s];
-      c = L > 0 ? (L + chunk - 1) / chunk : 1;
-    }
-    long long x = c;
+  const long long per = (nseg + blockDim.x - 1) / blockDim.x;
+  const long long first = threadIdx.x * per, end = first + per < nseg ? first + per : nseg;
+  auto chunks = [&](long long s) {
+    const long long L = off[s + 1] - off[s];
+    return L > 0 ? (L + chunk - 1) / chunk : 1;
+  };
+  long long own = 0;
+#pragma unroll 8
+  for (long long s = first; s < end; ++s) own += chunks(s);
+  long long x = own;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_warp[w] = x;
+  __syncthreads();
+  if (w == 0) {
+    const long long t = s_warp[lane];
+    long long ti = t;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const long long y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
+      const long long y = __shfl_up_sync(0xffffffffu, ti, o);
+      if (lane >= o) ti += y;
     }
-    if (lane == 31) s_warp[w] = x;
-    __syncthreads();
-    if (w == 0) {
-      const int nw = blockDim.x / 32;
-      long long t = lane < nw ? s_warp[lane] : 0;
-      long long ti = t;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const long long y = __shfl_up_sync(0xffffffffu, ti, o);
-        if (lane >= o) ti += y;
-      }
-      if (lane < nw) s_warp[lane] = ti - t;
-    }
-    __syncthreads();
-    const long long excl = s_carry + s_warp[w] + x - c;
-    if (s < nseg) chunk_start[s] = excl;
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) s_carry = excl + c;
-    __syncthreads();
+    s_warp[lane] = ti - t;
+    if (lane == 31) s_carry = ti;
+  }
+  __syncthreads();
+  long long excl = s_warp[w] + x - own;
+#pragma unroll 8
+  for (long long s = first; s < end; ++s) {
+    chunk_start[s] = excl;
+    excl += chunks(s);
   }
   if (threadIdx.x == 0) {
     chunk_start[nseg] = s_carry;
@@ -95,6 +97,71 @@ __global__ void __launch_bounds__(1024) k_batch_prep(const long long* __restrict
     h->total_chunks = s_carry <= capacity ? (unsigned long long)s_carry : 0ull;
     if (s_carry > capacity) h->any_violation |= 2u;
     h->ticket = 0;
+  }
+}
+
+// The lengths' statistics, one collection per thread in turn: partial sums per
+// CTA in a fixed order, added by the last CTA in theirs.
+constexpr int kStatThreads = 256;
+__global__ void __launch_bounds__(kStatThreads) k_batch_lengths(const long long* __restrict__ off,
+                                                                long long nseg, unsigned* counter,
+                                                                BatchLengths* part,
+                                                                BatchLengths* out) {
+  __shared__ BatchLengths sh[kStatThreads / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const auto add = [](BatchLengths& a, const BatchLengths& b) {
+    a.s += b.s;
+    a.s2 += b.s2;
+    a.mn = b.mn < a.mn ? b.mn : a.mn;
+    a.mx = b.mx > a.mx ? b.mx : a.mx;
+    a.negative |= b.negative;
+  };
+  const BatchLengths none{0.0, 0.0, 0x7fffffffffffffffLL, -1, 0, 0, 0};
+  BatchLengths v = none;
+  for (long long i = blockIdx.x * (long long)kStatThreads + threadIdx.x; i < nseg;
+       i += (long long)gridDim.x * kStatThreads) {
+    const long long L = off[i + 1] - off[i];
+    const double l = L < 0 ? 0.0 : log2((double)L + 1.0);
+    add(v, BatchLengths{l, l * l, L, L, 0, L < 0 ? 1 : 0, 0});
+  }
+  const auto warp_add = [&](BatchLengths& a) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      add(a, BatchLengths{__shfl_xor_sync(0xffffffffu, a.s, o), __shfl_xor_sync(0xffffffffu, a.s2, o),
+                          __shfl_xor_sync(0xffffffffu, a.mn, o),
+                          __shfl_xor_sync(0xffffffffu, a.mx, o), 0,
+                          __shfl_xor_sync(0xffffffffu, a.negative, o), 0});
+  };
+  warp_add(v);
+  if (lane == 0) sh[w] = v;
+  __syncthreads();
+  if (w != 0) return;
+  v = lane < kStatThreads / 32 ? sh[lane] : none;
+  warp_add(v);
+  unsigned last = 0;
+  if (lane == 0) {
+    part[blockIdx.x] = v;
+    __threadfence();
+    last = atomicAdd(counter, 1u) == gridDim.x - 1;
+  }
+  if (!__shfl_sync(0xffffffffu, last, 0)) return;
+  __threadfence();
+  BatchLengths q[kStatCtas / 32];
+#pragma unroll
+  for (int k = 0; k < kStatCtas / 32; ++k) {
+    const BatchLengths* p = part + lane + 32 * k;
+    q[k] = lane + 32 * k < (int)gridDim.x
+               ? BatchLengths{__ldcg(&p->s), __ldcg(&p->s2), __ldcg(&p->mn), __ldcg(&p->mx), 0,
+                              __ldcg(&p->negative), 0}
+               : none;
+  }
+#pragma unroll
+  for (int k = 1; k < kStatCtas / 32; ++k) add(q[0], q[k]);
+  warp_add(q[0]);
+  if (lane == 0) {
+    q[0].total = off[nseg] - off[0];
+    *out = q[0];
+    *counter = 0u;
   }
 }
 
@@ -268,6 +335,15 @@ size_t batch_scratch_bytes(long long nseg, long long capacity) {
   return sizeof(BatchHdr) + (size_t)(nseg + 1) * sizeof(long long) +
          (size_t)nseg * sizeof(unsigned) + (size_t)capacity * sizeof(ChunkPartial) +
          (size_t)capacity * sizeof(int) + 1280;
+}
+
+cudaError_t launch_batch_lengths(const long long* off, long long nseg, void* work,
+                                 BatchLengths* out, cudaStream_t s) {
+  const int g = (int)std::min<long long>((nseg + kStatThreads - 1) / kStatThreads, kStatCtas);
+  k_batch_lengths<<<g, kStatThreads, 0, s>>>(
+      off, nseg, static_cast<unsigned*>(work),
+      reinterpret_cast<BatchLengths*>(static_cast<char*>(work) + 256), out);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_batch(const BatchLaunch& L, cudaStream_t s, Prof* prof) {

@@ -28,4 +28,18 @@ size_t batch_scratch_bytes(long long nseg, long long capacity);
 cudaError_t launch_batch(const BatchLaunch& L, cudaStream_t s, Prof* prof);
 int batch_blocks_per_sm(int depth);
 
+// What the schedule chooser needs of the lengths L_i = off[i + 1] - off[i]:
+// sums of log2(L_i + 1) and of its square (fixed order), the extremes, the total
+// and whether a length is negative.  out and the work space (zeroed once by
+// the caller, left zeroed where it must be) on the device.
+struct BatchLengths {
+  double s, s2;
+  long long mn, mx, total;
+  int negative, pad;
+};
+constexpr int kStatCtas = 128;
+constexpr size_t kStatWorkBytes = 256 + kStatCtas * sizeof(BatchLengths);
+cudaError_t launch_batch_lengths(const long long* off, long long nseg, void* work,
+                                 BatchLengths* out, cudaStream_t s);
+
 }  // namespace sgk

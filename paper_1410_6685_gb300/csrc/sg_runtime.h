@@ -112,6 +112,8 @@ struct BatchPlanCache {
   std::vector<std::pair<BatchKey, BatchPlan>> plans;
   cudaStream_t capture_stream = nullptr;
   cudaEvent_t ev[2] = {nullptr, nullptr};   // timing of each batched run
+  void* stat_dev = nullptr;                 // the lengths' statistics: work space and record,
+  void* stat_host = nullptr;                // and the pinned copy of the record
   ~BatchPlanCache();
 };
 
