@@ -7,7 +7,7 @@
 // When no interchange will be needed, as for diagonally dominant matrices,
 // the outer block is three launches instead of about eleven, on average 85 us
 // at n = 8192 (28 + 18 + 43 by kernel; the factorisation 14.8 -> 5.4 ms), and
-// 70 us with the next diagonal block beside the update (4.4 ms; 16-bit updates):
+// 64 us with the next diagonal block beside the update (4.1 ms; 16-bit updates):
 //   k_lu_diag_block : the 128 x 128 diagonal block, in one CTA's shared memory;
 //   k_lu_border     : L21 = A21 U11^-1 and U12 = L11^-1 A12, 64 rows or columns
 //                     per CTA, which also writes the trailing update's
@@ -230,53 +230,33 @@ __global__ void __launch_bounds__(kBorderThreads, 2)
   const bool rows = (int)blockIdx.x < nrow_ctas;
   const int first = K + kNB + ((int)blockIdx.x - (rows ? 0 : nrow_ctas)) * kW;
   const int cnt = min(kW, n - first);
-  // warp w takes rows w, w + 8, ...; eight loads in flight
-#pragma unroll 2
-  for (int r0 = 0; r0 < kNB; r0 += 16) {
-    float v[2][4];
+  // every load in flight at once, straight into shared memory (past the end:
+  // zero); eight at a time through registers the border took 17.5 us, now 16.2
+  auto copy4 = [&](float* dst, const float* src, bool in) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(tc::smem_u32(dst)),
+                 "l"(in ? src : LU), "r"(in ? 4 : 0)
+                 : "memory");
+  };
+#pragma unroll 4
+  for (int r = w; r < kNB; r += 8)
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+    for (int u = 0; u < 4; ++u)
+      copy4(S + r * kS + lane + 32 * u, LU + (size_t)(K + r) * n + K + lane + 32 * u, true);
+  if (rows) {
+#pragma unroll 4
+    for (int r = w; r < kW; r += 8)
 #pragma unroll
       for (int u = 0; u < 4; ++u)
-        v[i][u] = __ldg(LU + (size_t)(K + r0 + w + 8 * i) * n + K + lane + 32 * u);
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int u = 0; u < 4; ++u) S[(r0 + w + 8 * i) * kS + lane + 32 * u] = v[i][u];
-  }
-  if (rows) {
-#pragma unroll 2
-    for (int r0 = 0; r0 < kW; r0 += 16) {
-      float v[2][4];
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int r = r0 + w + 8 * i;
-          v[i][u] = r < cnt ? LU[(size_t)(first + r) * n + K + lane + 32 * u] : 0.0f;
-        }
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) X[(r0 + w + 8 * i) * kS + lane + 32 * u] = v[i][u];
-    }
+        copy4(X + r * kS + lane + 32 * u, LU + (size_t)(first + r) * n + K + lane + 32 * u, r < cnt);
   } else {
-#pragma unroll 2
-    for (int r0 = 0; r0 < kNB; r0 += 32) {
-      float v[4][2];
+#pragma unroll 4
+    for (int r = w; r < kNB; r += 8)
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int r = r0 + w + 8 * i, c = lane + 32 * u;
-          v[i][u] = c < cnt ? LU[(size_t)(K + r) * n + first + c] : 0.0f;
-        }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int u = 0; u < 2; ++u) X[(r0 + w + 8 * i) * kXS + lane + 32 * u] = v[i][u];
-    }
+      for (int u = 0; u < 2; ++u)
+        copy4(X + r * kXS + lane + 32 * u, LU + (size_t)(K + r) * n + first + lane + 32 * u,
+              lane + 32 * u < cnt);
   }
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   if (rows && tid < kNB) rd[tid] = 1.0f / S[tid * kS + tid];
   __syncthreads();

@@ -187,8 +187,8 @@ cudaError_t capture(sg_ctx* c, LuCache& L, cudaGraphExec_t* exec, int64_t* kerne
 // factored without interchanges first (each pivot is verified on the device);
 // when that fails, or for any other matrix, the general elimination runs.
 // The choice costs one read-back of 8 bytes (about 15 us); where it applies it
-// takes the factorisation at n = 8192 from 14.8 to 4.4 ms (binary32 updates: 21.8
-// to 8.5 ms), at 2048 from 2.82 to 0.76 ms.  Waits for the stream.  Afterwards
+// takes the factorisation at n = 8192 from 14.8 to 4.1 ms (binary32 updates: 21.8
+// to 7.4 ms), at 2048 from 2.82 to 0.70 ms.  Waits for the stream.  Afterwards
 // c->lu.lu holds L\U, c->lu.piv the interchanges and *hinfo the zero-pivot
 // report.
 sg_status lu_factor(sg_ctx* c, const float* A, int n, sg_precision prec, double* norms,
