@@ -95,7 +95,8 @@ cudaError_t lengths_by_device(sg_ctx* c, const Job& j, sgk::BatchLengths* r) {
   if (!cache.stat_host) {
     cudaError_t e = cudaSuccess;
     if (!cache.stat_dev) e = cudaMalloc(&cache.stat_dev, sgk::kStatWorkBytes + sizeof *r);
-    if (e == cudaSuccess) e = cudaMemset(cache.stat_dev, 0, 256);
+    // on the context's stream: nothing orders the default one before it
+    if (e == cudaSuccess) e = cudaMemsetAsync(cache.stat_dev, 0, 256, c->stream);
     if (e == cudaSuccess) e = cudaMallocHost(&cache.stat_host, sizeof *r);
     if (e != cudaSuccess) return e;
   }
@@ -179,8 +180,10 @@ sg_status run_with(sg_ctx* c, const Job& j, const sg_sched_choice& sch, double* 
         cudaGetLastError();
         return bad(c, SG_ERR_OOM, "batch scratch allocation failed");
       }
-      // the per-collection counters start at zero and return to zero
-      cudaMemset(p.scratch, 0, sgk::batch_scratch_bytes(j.nseg, p.capacity));
+      // the per-collection counters start at zero and return to zero; cleared on
+      // the stream that the graph runs on (nothing orders the default one before it)
+      cudaError_t e =
+          cudaMemsetAsync(p.scratch, 0, sgk::batch_scratch_bytes(j.nseg, p.capacity), c->stream);
       sgk::BatchLaunch L{};
       L.data = j.data;
       L.offsets = reinterpret_cast<const long long*>(j.offsets);
@@ -198,7 +201,8 @@ sg_status run_with(sg_ctx* c, const Job& j, const sg_sched_choice& sch, double* 
       L.jit = c->codegen == SG_CODEGEN_SPECIALIZE ? sgk::jit_batch_kernel(j.prog, nullptr)
                                                   : nullptr;
       cudaGraph_t g = nullptr;
-      cudaError_t e = cudaStreamBeginCapture(cache.capture_stream, cudaStreamCaptureModeThreadLocal);
+      if (e == cudaSuccess)
+        e = cudaStreamBeginCapture(cache.capture_stream, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
         cudaError_t le = sgk::launch_batch(L, cache.capture_stream, nullptr);
         e = cudaStreamEndCapture(cache.capture_stream, &g);
