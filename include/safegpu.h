@@ -334,7 +334,8 @@ sg_status sg_solve(sg_ctx* ctx, sg_matrix* A, sg_vector* b,
  * An exactly singular A (a zero pivot) is not an error: sign = 0,
  * det = 0, log_abs = -inf, info = k+1 for the first zero pivot at step k.
  * Errors: SG_ERR_SHAPE (not square, n too large), SG_ERR_DTYPE,
- * SG_ERR_POISONED, SG_ERR_OOM, SG_ERR_CUDA. */
+ * SG_ERR_POISONED, SG_ERR_OOM, SG_ERR_CUDA, SG_ERR_TIMEOUT (a bounded wait of
+ * the elimination gave up). */
 typedef struct {
   int32_t sign;        /* +1, -1, or 0 for an exactly singular A            */
   int32_t info;        /* 0, or k+1 for the first exactly zero pivot        */
@@ -528,6 +529,16 @@ sg_status sg_debug_lookback(sg_ctx* ctx, uint32_t spin_limit, int64_t skip_tile)
  * ignore it.  Errors: SG_ERR_INVALID_ARG for indices below -1, one of them
  * negative, or above INT32_MAX. */
 sg_status sg_debug_inject_matmul(sg_ctx* ctx, int64_t row, int64_t col, float delta);
+
+/* Failure-detection testing of the elimination's trailing updates, whose
+ * kernels wait on their own loads and multiply-adds with bounded waits and
+ * raise a word in device memory when one gives up.  on != 0: the host raises
+ * that word behind the NEXT elimination with interchanges (sg_solve, sg_det) of
+ * this context, which must then return SG_ERR_TIMEOUT; 0 cancels.  Eliminations
+ * without interchanges take the word for a failed verification and are
+ * followed by the form with them.  Errors: SG_ERR_INVALID_ARG for a null
+ * context. */
+sg_status sg_debug_inject_update_timeout(sg_ctx* ctx, int on);
 
 /* Testing aid for the portable kernel forms.  On devices that schedule them,
  * tensor-core products run on CTA pairs (clusters of two, tcgen05

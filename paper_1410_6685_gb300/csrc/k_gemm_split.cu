@@ -470,10 +470,11 @@ size_t gemm_split_scratch_bytes(int M, int N, int K) {
 
 cudaError_t launch_gemm_split(const float* A, int lda, const float* B, int ldb, float* C, int ldc,
                               int M, int N, int K, bool subtract, void* scratch, cudaStream_t s,
-                              Prof* prof, int64_t* kernels, int form) {
+                              Prof* prof, int64_t* kernels, int* err) {
   const int Kp = ((K + 63) / 64) * 64;
   char* p = static_cast<char*>(scratch);
   int* gate = reinterpret_cast<int*>(p);   // [0] out of range, [1] a wait gave up
+  if (!err) err = gate + 1;
   uint16_t* a3 = reinterpret_cast<uint16_t*>(p + 256);
   uint16_t* b3 = reinterpret_cast<uint16_t*>(p + 256 + align256((size_t)M * Kp * 6));
   prof_begin(prof, "split_operands", s);
@@ -483,9 +484,9 @@ cudaError_t launch_gemm_split(const float* A, int lda, const float* B, int ldb, 
   if (e != cudaSuccess) return e;
   prof_end(prof, s);
   prof_begin(prof, "gemm_f32_split", s);
-  if (form < 0) form = choose_form(M, N, K, nullptr);
-  e = subtract ? launch_split<true>(form, a3, b3, Kp, C, ldc, M, N, K, gate, nullptr, gate + 1, s)
-               : launch_split<false>(form, a3, b3, Kp, C, ldc, M, N, K, gate, nullptr, gate + 1, s);
+  const int form = choose_form(M, N, K, nullptr);
+  e = subtract ? launch_split<true>(form, a3, b3, Kp, C, ldc, M, N, K, gate, nullptr, err, s)
+               : launch_split<false>(form, a3, b3, Kp, C, ldc, M, N, K, gate, nullptr, err, s);
   prof_end(prof, s);
   if (e != cudaSuccess) return e;
   *kernels += 3;

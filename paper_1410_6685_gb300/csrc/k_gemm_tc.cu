@@ -898,7 +898,7 @@ cudaError_t time_gemm_forms(const float* A, int lda, const float* B, int ldb, fl
 cudaError_t launch_gemm_tc(const float* A, int lda, const float* B, int ldb, float* C, int ldc,
                            int M, int N, int K, bool fp16, bool subtract, void* scratch,
                            cudaStream_t s, Prof* prof, int64_t* kernels, int inj_row,
-                           int inj_col, float inj_delta, int form) {
+                           int inj_col, float inj_delta, int form, int* err) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   if (K <= 0) {   // empty inner dimension: C = 0 (or C unchanged for C - A B)
     if (subtract) return cudaSuccess;
@@ -906,7 +906,7 @@ cudaError_t launch_gemm_tc(const float* A, int lda, const float* B, int ldb, flo
   }
   const int Kp = ((K + TK - 1) / TK) * TK;
   char* p = static_cast<char*>(scratch);
-  int* err = reinterpret_cast<int*>(p);
+  if (!err) err = reinterpret_cast<int*>(p);
   uint16_t* a16 = reinterpret_cast<uint16_t*>(p + 256);
   uint16_t* bt16 = reinterpret_cast<uint16_t*>(p + 256 + align256((size_t)M * Kp * 2));
   prof_begin(prof, "cast_operands", s);

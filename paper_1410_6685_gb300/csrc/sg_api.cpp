@@ -1059,6 +1059,12 @@ sg_status sg_debug_inject_matmul(sg_ctx* c, int64_t row, int64_t col, float delt
   return SG_OK;
 }
 
+sg_status sg_debug_inject_update_timeout(sg_ctx* c, int on) {
+  if (!c) return SG_ERR_INVALID_ARG;
+  c->inject_update_timeout = on != 0;
+  return SG_OK;
+}
+
 sg_status sg_debug_portable_kernels(sg_ctx* c, int on) {
   if (!c) return SG_ERR_INVALID_ARG;
   sgk::set_portable_kernels(on != 0);

@@ -15,20 +15,22 @@ cudaError_t launch_gemm_f32(const float* A, int lda, const float* B, int ldb, fl
 // split into three bf16 pieces each, six piece products, sums carried in
 // binary32 registers.  Operands outside its range, found on the device, fall
 // back to launch_gemm_f32 (queued behind, a no-op otherwise).  wanted: the
-// sizes that gain from it.  form: -1 by the sizes, else 0 / 1 / 2 (128 x 64,
-// 128 x 128, a CTA pair's 256 x 256 tiles).
+// sizes that gain from it.  A wait that gave up: C is computed by
+// launch_gemm_f32; a subtracting product has changed C by then and only raises
+// *err, which its caller reads.
 bool gemm_split_wanted(int M, int N, int K);
 size_t gemm_split_scratch_bytes(int M, int N, int K);
 cudaError_t launch_gemm_split(const float* A, int lda, const float* B, int ldb, float* C, int ldc,
                               int M, int N, int K, bool subtract, void* scratch, cudaStream_t s,
-                              Prof* prof, int64_t* kernels, int form = -1);
+                              Prof* prof, int64_t* kernels, int* err = nullptr);
 
 // Tensor-core product: operands rounded (nearest even) to bf16 or fp16,
 // binary32 accumulation in tensor memory.  beta = 0: C = A B; beta = 1:
 // C = C - A B (the elimination update).  a16 / bt16 are scratch operand
 // copies (M x Kp and N x Kp, K-major, Kp = K rounded up to 64).
 // inj_row / inj_col >= 0: contract testing, inj_delta is added to that
-// product element before it is stored.
+// product element before it is stored.  err: the word that a wait which gives up
+// raises (null: one of the scratch's).
 size_t gemm_tc_scratch_bytes(int M, int N, int K);
 // process-wide: use the portable kernel forms (one-CTA tensor-core product,
 // 8-CTA elimination panel) even where the device schedules the fast ones
@@ -42,7 +44,8 @@ void gemm_tc_prepare();
 cudaError_t launch_gemm_tc(const float* A, int lda, const float* B, int ldb, float* C, int ldc,
                            int M, int N, int K, bool fp16, bool subtract, void* scratch,
                            cudaStream_t s, Prof* prof, int64_t* kernels, int inj_row = -1,
-                           int inj_col = -1, float inj_delta = 0.0f, int form = 0);
+                           int inj_col = -1, float inj_delta = 0.0f, int form = 0,
+                           int* err = nullptr);
 bool gemm_pair_available();
 // C -= A16 Bt16^T, the elimination's update with its operands already in
 // K-major 16-bit copies (M x K and N x K, K a multiple of 64); nothing is done

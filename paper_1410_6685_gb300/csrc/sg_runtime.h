@@ -210,6 +210,7 @@ struct sg_ctx {
   bool host_res_mapped = false;        // kernels can store into host_res directly
   sgk::SortInject inject{};            // contract-test fault for the next sort
   sgk::LookbackCtl lookback{0, -1};    // testing switch of the look-back waits
+  bool inject_update_timeout = false;  // the next elimination's updates report a wait given up
   struct {
     int64_t row = -1, col = -1;
     float delta = 0.0f;

@@ -54,7 +54,8 @@ struct SolveWork {
 // the row interchanged with row k at step k, *info = k+1 at an exactly zero
 // pivot.  moves: ceil(n / kLuPanel) * kLuMoveInts ints, zero on entry.
 // gemm: tensor-core scratch (gemm_tc_scratch_bytes or, for binary32 updates,
-// gemm_split_scratch_bytes of (n, n, kLuOuter)).
+// gemm_split_scratch_bytes of (n, n, kLuOuter)).  info[2] = 1: a wait of a
+// trailing update gave up, and the factors are worthless.
 cudaError_t factor_in_place(sg_ctx* c, float* lu, int n, int* piv, int* perm, int* info,
                             int* moves, unsigned* counters, void* gemm, sg_precision prec,
                             cudaStream_t s, sgk::Prof* prof) {
@@ -92,10 +93,10 @@ cudaError_t factor_in_place(sg_ctx* c, float* lu, int n, int* piv, int* perm, in
       if (e == cudaSuccess && tc) {
         e = sgk::launch_gemm_tc(at(K + KB, K), n, at(K, K + KB), n, at(K + KB, K + KB), n, rest,
                                 rest, KB, prec == SG_PREC_F16_TC, true, gemm, s, prof,
-                                &c->kernels);
+                                &c->kernels, -1, -1, 0.0f, 0, info + 2);
       } else if (e == cudaSuccess && sgk::gemm_split_wanted(rest, rest, KB)) {
         e = sgk::launch_gemm_split(at(K + KB, K), n, at(K, K + KB), n, at(K + KB, K + KB), n, rest,
-                                   rest, KB, true, gemm, s, prof, &c->kernels);
+                                   rest, KB, true, gemm, s, prof, &c->kernels, info + 2);
       } else if (e == cudaSuccess) {
         e = sgk::launch_gemm_f32(at(K + KB, K), n, at(K, K + KB), n, at(K + KB, K + KB), n, rest,
                                  rest, KB, true, s, prof);
@@ -185,7 +186,8 @@ cudaError_t capture(sg_ctx* c, LuCache& L, cudaGraphExec_t* exec, int64_t* kerne
 // (the pass that forms its norms, all zero on entry, does so: a copy of its own took
 // 80 us at n = 8192) and replays a graph on the context's stream.  A matrix whose rows are all diagonally dominant is
 // factored without interchanges first (each pivot is verified on the device);
-// when that fails, or for any other matrix, the general elimination runs.
+// when that fails, or for any other matrix, the general elimination runs (and
+// SG_ERR_TIMEOUT is returned when one of its updates gave up a wait).
 // The choice costs one read-back of 8 bytes (about 15 us); where it applies it
 // takes the factorisation at n = 8192 from 14.8 to 4.1 ms (binary32 updates: 21.8
 // to 7.4 ms), at 2048 from 2.82 to 0.70 ms.  Waits for the stream.  Afterwards
@@ -272,11 +274,15 @@ sg_status lu_factor(sg_ctx* c, const float* A, int n, sg_precision prec, double*
         return err(c, SG_ERR_CUDA, "factorisation graph capture failed");
       }
     }
-    int hi[2] = {0, 0};
+    int hi[3] = {0, 0, 0};
     sgk::prof_begin(&c->prof, "lu_factor_graph", s);
     cudaError_t e = cudaGraphLaunch(exec, s);
     sgk::prof_end(&c->prof, s);
     c->kernels += kernels;
+    if (e == cudaSuccess && !diag && c->inject_update_timeout) {
+      c->inject_update_timeout = false;
+      e = cudaMemsetAsync(L.info + 2, 1, sizeof(int), s);
+    }
     if (e == cudaSuccess) e = cudaMemcpyAsync(L.host, L.info, sizeof hi, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
@@ -285,7 +291,8 @@ sg_status lu_factor(sg_ctx* c, const float* A, int n, sg_precision prec, double*
     }
     memcpy(hi, L.host, sizeof hi);
     *hinfo = hi[0];
-    return diag && hi[1] ? SG_ERR_NOT_CONVERGED : SG_OK;   // only seen below
+    if (diag) return hi[1] || hi[2] ? SG_ERR_NOT_CONVERGED : SG_OK;   // only seen below
+    return hi[2] ? err(c, SG_ERR_TIMEOUT, "trailing update's wait gave up") : SG_OK;
   };
   const size_t bytes = (size_t)n * n * 4;
   cudaError_t e = sgk::launch_anorm(A, n, norms, L.lu, s);
