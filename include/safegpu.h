@@ -266,11 +266,16 @@ sg_status sg_sort(sg_ctx* ctx, sg_vector* keys, sg_vector** out);
 
 /* ------------------------------------------------------------------------ */
 /* Matrix product (Sec. 3.4 `multiply`): C = A B.  A: M x K, B: K x N, SG_F32
- * storage; C: M x N SG_F32.  `precision` selects binary32 arithmetic (on the
- * CUDA cores, or for larger sizes on the tensor cores with every operand split
- * exactly into three bf16 pieces; products of binary32 accuracy either way) or
+ * storage; C: M x N SG_F32.  `precision` selects binary32 arithmetic or
  * bf16 / fp16 operands (rounded to nearest even) on the tensor cores with
- * binary32 accumulation.  Built-in postcondition (mode >= PRE_POST):
+ * binary32 accumulation.  Binary32 runs on the CUDA cores (one fused multiply-add
+ * after the other: every entry within K 2^-24 of sum_k |a_ik b_kj|), or for larger
+ * sizes with K > 64 on the tensor cores, every operand split exactly into three
+ * bf16 pieces: every entry within (24 + K / 16) 2^-24 of the same, on dense
+ * operands with a fifth to a quarter of the other's error; an entry that is a single
+ * product is off by up to 2^-23 of itself, by the mean square as if rounded once.
+ * The pieces take entries of magnitude 2^-50 to 2^55 and zero; with any other
+ * among them the product is the CUDA cores'.  Built-in postcondition (mode >= PRE_POST):
  * Freivalds' check with 4 Rademacher vectors (see sg_contract). */
 typedef enum {
   SG_PREC_F32_SIMT = 0,

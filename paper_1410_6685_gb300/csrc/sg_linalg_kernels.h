@@ -12,8 +12,8 @@ cudaError_t launch_gemm_f32(const float* A, int lda, const float* B, int ldb, fl
                             const int* only_if = nullptr);
 
 // The same binary32 product on the tensor cores (k_gemm_split.cu): operands
-// split into three bf16 pieces each, six piece products, sums carried in
-// binary32 registers.  Operands outside its range, found on the device, fall
+// split into three bf16 pieces each, six piece products, the largest's sums
+// carried in binary32 registers.  Operands outside its range, found on the device, fall
 // back to launch_gemm_f32 (queued behind, a no-op otherwise).  wanted: the
 // sizes that gain from it.  A wait that gave up: C is computed by
 // launch_gemm_f32; a subtracting product has changed C by then and only raises
