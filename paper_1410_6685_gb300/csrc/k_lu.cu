@@ -1448,6 +1448,12 @@ __global__ void __launch_bounds__(1024) k_lu_det(const float* __restrict__ LU, i
 // |A|_inf (binary64) once per factorisation, and whether every row is
 // diagonally dominant: 2 |a_ii| >= sum_j |a_ij| (NaN: not).  The binary64 pipe
 // bounds it (157 us at n = 8192), so that copying A beside it costs nothing.
+// Up to kColumnRows rows a larger entry below a diagonal counts as not dominant
+// too: elimination without interchanges would most likely fail there, and a failed one
+// costs 70 us, more than half of a determinant of n = 100 by the general form (253
+// us instead of 176).  For larger matrices it is 15% and less, and the diagonal's
+// gathers would not stay in L1.
+constexpr int kColumnRows = 256;
 __global__ void __launch_bounds__(256) k_anorm(const float* __restrict__ A, int n,
                                                double* norms, float* __restrict__ copy) {
   const int lane = threadIdx.x & 31;
@@ -1457,10 +1463,18 @@ __global__ void __launch_bounds__(256) k_anorm(const float* __restrict__ A, int 
   for (long long i = warp; i < n; i += nw) {
     const float* row = A + i * (long long)n;
     double s = 0.0;
+    bool above = false;
     for (int j = lane; j < n; j += 256) {
       float av[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) av[u] = j + 32 * u < n ? __ldg(row + j + 32 * u) : 0.0f;
+      if (n <= kColumnRows) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const long long c = j + 32 * u;
+          above |= c < i && !(fabsf(av[u]) <= fabsf(__ldg(A + c * (n + 1))));
+        }
+      }
 #pragma unroll
       for (int u = 0; u < 8; ++u)
         if (j + 32 * u < n) copy[i * (long long)n + j + 32 * u] = av[u];
@@ -1470,7 +1484,9 @@ __global__ void __launch_bounds__(256) k_anorm(const float* __restrict__ A, int 
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     mx = fmax(mx, s);
-    if (lane == 0 && !(2.0 * fabs((double)row[i]) >= s)) *reinterpret_cast<int*>(&norms[6]) = 1;
+    above = __any_sync(0xffffffffu, above);
+    if (lane == 0 && (above || !(2.0 * fabs((double)row[i]) >= s)))
+      *reinterpret_cast<int*>(&norms[6]) = 1;
   }
   if (lane == 0) atomicMax(reinterpret_cast<unsigned long long*>(&norms[3]),
                            (unsigned long long)__double_as_longlong(mx));

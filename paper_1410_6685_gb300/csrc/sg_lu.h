@@ -53,7 +53,8 @@ cudaError_t launch_residual(const float* A, int n, const double* b, const double
                             double* norms, double thresh, unsigned long long* viol,
                             cudaStream_t s, Prof* prof);
 // norms[3] = |A|_inf; the 32-bit word at norms[6] becomes 1 when some row is
-// not diagonally dominant (both zero before).  copy = A.
+// not diagonally dominant, or, in a small matrix, an entry below the diagonal
+// larger than it (both zero before).  copy = A.
 cudaError_t launch_anorm(const float* A, int n, double* norms, float* copy, cudaStream_t s);
 // out[0] = sign of det A (0 if singular), out[1] = log |det A|, from the factors
 cudaError_t launch_lu_det(const float* LU, int n, const int* piv, double* out, cudaStream_t s,

@@ -184,13 +184,15 @@ cudaError_t capture(sg_ctx* c, LuCache& L, cudaGraphExec_t* exec, int64_t* kerne
 // elimination (memsets and about 7 n / 32 kernels, or 3 n / 128 without
 // interchanges) as a CUDA graph on a private stream; every call copies A in
 // (the pass that forms its norms, all zero on entry, does so: a copy of its own took
-// 80 us at n = 8192) and replays a graph on the context's stream.  A matrix whose rows are all diagonally dominant is
-// factored without interchanges first (each pivot is verified on the device);
+// 80 us at n = 8192) and replays a graph on the context's stream.  A matrix of
+// more than one panel whose rows are all diagonally dominant is factored without
+// interchanges first (each pivot is verified on the device);
 // when that fails, or for any other matrix, the general elimination runs (and
 // SG_ERR_TIMEOUT is returned when one of its updates gave up a wait).
-// The choice costs one read-back of 8 bytes (about 15 us); where it applies it
+// The choice costs one read-back of 8 bytes (about 15 us: a determinant of n = 8
+// 98 us with it, 81 without); where it applies it
 // takes the factorisation at n = 8192 from 14.8 to 4.1 ms (binary32 updates: 21.8
-// to 7.4 ms), at 2048 from 2.82 to 0.70 ms.  Waits for the stream.  Afterwards
+// to 6.7 ms), at 2048 from 2.82 to 0.70 ms.  Waits for the stream.  Afterwards
 // c->lu.lu holds L\U, c->lu.piv the interchanges and *hinfo the zero-pivot
 // report.
 sg_status lu_factor(sg_ctx* c, const float* A, int n, sg_precision prec, double* norms,
@@ -296,10 +298,12 @@ sg_status lu_factor(sg_ctx* c, const float* A, int n, sg_precision prec, double*
   };
   const size_t bytes = (size_t)n * n * 4;
   cudaError_t e = sgk::launch_anorm(A, n, norms, L.lu, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(L.host, norms + 6, 8, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  int not_dominant = 0;
-  memcpy(&not_dominant, L.host, sizeof not_dominant);
+  int not_dominant = 1;
+  if (n > sgk::kLuPanel) {   // (one panel: the general form is as short)
+    if (e == cudaSuccess) e = cudaMemcpyAsync(L.host, norms + 6, 8, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    memcpy(&not_dominant, L.host, sizeof not_dominant);
+  }
   if (e == cudaSuccess && !not_dominant) {
     const sg_status st = run(true);
     if (st != SG_ERR_NOT_CONVERGED) return st;
