@@ -267,6 +267,8 @@ sg_status sg_destroy(sg_ctx* c) {
     cudaStreamDestroy(c->download);
     cudaEventDestroy(c->last_download);
     if (c->scratch) cudaFree(c->scratch);
+    if (c->pieces.own) cudaFreeAsync(c->pieces.own, c->stream);
+    if (c->pieces.pool) cudaMemPoolDestroy(c->pieces.pool);
     if (c->counter) cudaFree(c->counter);
     if (c->host_res) cudaFreeHost(c->host_res);
   }

@@ -878,52 +878,37 @@ sg_status run_flush(sg_ctx* c, bool fuse, bool commit, double* us) {
 
   // scratch: result records, then the largest per-pass work area
   const size_t res_bytes = round_up(std::max<size_t>(1, passes.size()) * sgk::kResultBytes, 256);
-  auto work_bytes = [&]() {
-    size_t work = 0;
-    for (Pass& P : passes) {
-      switch (P.kind) {
-        case PK::STREAM:
-          work = std::max(work, (size_t)std::max(stream_grid(c, P), c->num_sms * 8 * kStreamWaves) *
-                                    sizeof(sgk::PassResult));
-          break;
-        case PK::SORT: work = std::max(work, sgk::sort_scratch_bytes(P.n)); break;
-        case PK::FILTER: work = std::max(work, sgk::filter_jit_scratch_bytes(P.n)); break;
-        case PK::CHECK_SORTED:
-        case PK::CHECK_PERM: work = std::max(work, sgk::check_scratch_bytes()); break;
-        case PK::MATMUL:
-        case PK::FREIVALDS: work = std::max(work, sg_linalg_scratch(c, P.main, P.chk_frv)); break;
-        case PK::TRANSPOSE:
-        case PK::CONCAT:
-        case PK::FPRINT:
-        case PK::CHECK_SAME: break;
-        case PK::MATVEC: {
-          const Node* n = P.main;
-          const Value* A = P.vtrans ? P.vtrans->in[0].get() : n->left ? n->in[1].get() : nullptr;
-          if (A) work = std::max(work, sgk::vecmat_scratch_bytes((int)A->rows, (int)A->cols));
-          break;
-        }
+  size_t work = 0;
+  for (Pass& P : passes) {
+    switch (P.kind) {
+      case PK::STREAM:
+        work = std::max(work, (size_t)std::max(stream_grid(c, P), c->num_sms * 8 * kStreamWaves) *
+                                  sizeof(sgk::PassResult));
+        break;
+      case PK::SORT: work = std::max(work, sgk::sort_scratch_bytes(P.n)); break;
+      case PK::FILTER: work = std::max(work, sgk::filter_jit_scratch_bytes(P.n)); break;
+      case PK::CHECK_SORTED:
+      case PK::CHECK_PERM: work = std::max(work, sgk::check_scratch_bytes()); break;
+      case PK::MATMUL:
+      case PK::FREIVALDS: work = std::max(work, sg_linalg_scratch(c, P.main, P.chk_frv)); break;
+      case PK::TRANSPOSE:
+      case PK::CONCAT:
+      case PK::FPRINT:
+      case PK::CHECK_SAME: break;
+      case PK::MATVEC: {
+        const Node* n = P.main;
+        const Value* A = P.vtrans ? P.vtrans->in[0].get() : n->left ? n->in[1].get() : nullptr;
+        if (A) work = std::max(work, sgk::vecmat_scratch_bytes((int)A->rows, (int)A->cols));
+        break;
       }
     }
-    return work;
-  };
-  // a binary32 product takes scratch for its operands' pieces on the tensor
-  // cores and none on the CUDA cores: the latter while the stream is being
-  // captured (nothing may be allocated then) and where the scratch cannot be
-  // had
-  bool split = false;
-  for (Pass& P : passes)
-    if (P.kind == PK::MATMUL) split |= P.main->split = sg_linalg_split(P.main);
-  auto no_split = [&]() {
-    for (Pass& P : passes)
-      if (P.kind == PK::MATMUL) P.main->split = false;
-    split = false;
-  };
-  if (split && stream_capturing(c)) no_split();
-  sg_status st = ensure_scratch(c, res_bytes + work_bytes());
-  if (st && split) {
-    no_split();
-    st = ensure_scratch(c, res_bytes + work_bytes());
   }
+  // (a binary32 product on the tensor cores takes its operands' pieces from a
+  // pool of its own; not while the stream is being captured: nothing may be
+  // allocated then)
+  for (Pass& P : passes)
+    if (P.kind == PK::MATMUL) P.main->split = sg_linalg_split(P.main) && !stream_capturing(c);
+  sg_status st = ensure_scratch(c, res_bytes + work);
   if (!st) st = ensure_host_res(c, res_bytes);
   if (st) {
     if (commit) c->pending.clear();

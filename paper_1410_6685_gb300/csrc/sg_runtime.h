@@ -205,6 +205,11 @@ struct sg_ctx {
   unsigned int* counter = nullptr;     // last-block-done counter (stays zero)
   void* scratch = nullptr;             // per-flush scratch arena
   size_t scratch_bytes = 0;
+  struct {
+    cudaMemPool_t pool = nullptr;
+    void* own = nullptr;               // the block that stays
+    size_t bytes = 0;
+  } pieces;                            // memory for the binary32 products' operand pieces
   void* host_res = nullptr;            // pinned host copy of pass results
   size_t host_res_bytes = 0;
   bool host_res_mapped = false;        // kernels can store into host_res directly

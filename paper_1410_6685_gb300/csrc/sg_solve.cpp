@@ -190,7 +190,7 @@ cudaError_t capture(sg_ctx* c, LuCache& L, cudaGraphExec_t* exec, int64_t* kerne
 // when that fails, or for any other matrix, the general elimination runs (and
 // SG_ERR_TIMEOUT is returned when one of its updates gave up a wait).
 // The choice costs one read-back of 8 bytes (about 15 us: a determinant of n = 8
-// 98 us with it, 81 without); where it applies it
+// 97 us with it, 84 without); where it applies it
 // takes the factorisation at n = 8192 from 14.8 to 4.1 ms (binary32 updates: 21.8
 // to 6.7 ms), at 2048 from 2.82 to 0.70 ms.  Waits for the stream.  Afterwards
 // c->lu.lu holds L\U, c->lu.piv the interchanges and *hinfo the zero-pivot
