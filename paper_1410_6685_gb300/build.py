@@ -39,7 +39,8 @@ def _flags(src: str) -> list[str]:
 
 
 def _headers_mtime() -> float:
-    hs = glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
+    hs = [h for pat in (os.path.join(CSRC, "*.h"), os.path.join(CSRC, "*.cuh"),
+                        os.path.join(ROOT, "include", "*.h")) for h in glob.glob(pat)]
     return max(os.path.getmtime(h) for h in hs)
 
 
