@@ -15,10 +15,13 @@
 //   the trailing update A22 -= L21 U12 (k_gemm_tc.cu, k_gemm_split.cu).
 // Every entry goes through the same operations in the same order as in the
 // general form (a -= l_ik u_kj for increasing k, l = a (1 / u)), so the factors are
-// the same bits.  Every candidate a_ik is compared with its pivot before it is
-// scaled: one that is larger in magnitude (or NaN), or a zero pivot, raises
-// `fail`; what is queued behind then does nothing and the caller factors the
-// matrix by the general form.  k_lu_screen chooses the form beforehand.
+// the same bits, but for binary32 updates of trailing blocks that the general form
+// leaves to the CUDA cores (gemm_split_wanted: order 1537 to 1792 on 152 SMs); here
+// the border has written their pieces already.  Every candidate a_ik is compared
+// with its pivot before it is scaled: one that is larger in magnitude (or NaN), or a
+// zero pivot, raises `fail`; what is queued behind then does nothing and the caller
+// factors the matrix by the general form.  k_anorm (k_lu.cu) chooses the form
+// beforehand.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
