@@ -20,18 +20,6 @@
 #include "sg_linalg_kernels.h"
 
 namespace sgk {
-namespace {
-int sm_count() {
-  static const int sms = [] {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
-      v = 1;
-    return v;
-  }();
-  return sms;
-}
-}  // namespace
 
 // Groups of eight rows per CTA of the passes over A, B and C (a CTA loads its
 // vectors once): as many of four as leave a CTA for each SM.  N = 1000: 125
@@ -342,8 +330,6 @@ __global__ void __launch_bounds__(256) k_frv_check_fused(const float* __restrict
   }
   frv_worst(worst, res);
 }
-
-size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 }  // namespace
 

@@ -41,7 +41,6 @@
 // (subnormals, infinities, NaN, extreme scales); then this kernel does
 // nothing and the CUDA-core form, queued behind it, computes the product.
 #include <cuda.h>
-#include <cudaTypedefs.h>
 
 #include <algorithm>
 
@@ -408,19 +407,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (PAIR) cluster_sync();
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                         &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      p = nullptr;
-    return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  }();
-  return fn;
-}
-
 // the pieces [3][rows][Kp], boxes of TK x box_rows of one piece; rows past
 // the end read as zero
 bool make_map3(CUtensorMap* m, const void* base, int rows, int Kp, int box_rows) {
@@ -433,19 +419,6 @@ bool make_map3(CUtensorMap* m, const void* base, int rows, int Kp, int box_rows)
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
             es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
-
-int sm_count() {
-  static int sms = [] {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
-      v = 1;
-    return v;
-  }();
-  return sms;
 }
 
 template <bool PAIR, int TN, bool SUB>

@@ -21,7 +21,6 @@
 // Every mbarrier wait is bounded: on a timeout the kernel raises an error flag
 // and finishes without hanging.
 #include <cuda.h>
-#include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -672,19 +671,6 @@ __global__ void __launch_bounds__(256, 2) k_cast_a_frv(const float* __restrict__
   }
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                         &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  }
-  return fn;
-}
-
 bool make_map(CUtensorMap* m, const void* base, int rows, int Kp, int box_rows, bool fp16) {
   auto fn = encode_fn();
   if (!fn) return false;
@@ -696,20 +682,6 @@ bool make_map(CUtensorMap* m, const void* base, int rows, int Kp, int box_rows, 
             const_cast<void*>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
-
-// one CTA per SM (the pipeline's shared memory allows no second)
-int sm_count() {
-  static const int sms = [] {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
-      v = 1;
-    return v;
-  }();
-  return sms;
 }
 
 // the CTA-pair kernel where the device schedules clusters of two with its

@@ -242,18 +242,6 @@ __global__ void __launch_bounds__(256) k_vecmat_sum(const float* __restrict__ pa
   }
 }
 
-int sm_count() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        sms <= 0)
-      sms = 1;
-  }
-  return sms;
-}
-
 // row stripes of the left product: enough CTAs for about 4 per SM, at least
 // 16 rows per stripe
 int vecmat_stripes(int rows, int cols) {

@@ -5,6 +5,19 @@
 
 namespace sgk {
 
+inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+// the device's SMs (asked once)
+inline int sm_count() {
+  static const int sms = [] {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
+      v = 1;
+    return v;
+  }();
+  return sms;
+}
+
 // binary32 SIMT product C = A B (or C = C - A B), row-major with leading
 // dimensions (M x K, K x N, M x N).
 cudaError_t launch_gemm_f32(const float* A, int lda, const float* B, int ldb, float* C, int ldc,

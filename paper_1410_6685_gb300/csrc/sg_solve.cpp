@@ -356,7 +356,6 @@ extern "C" sg_status sg_solve(sg_ctx* c, sg_matrix* A, sg_vector* b, const sg_so
     if (info) *info = sg_solve_info{0, 0, 0.0, 0.0};
     return SG_OK;
   }
-  const int nb = (n + 31) / 32;
 
   // workspace (one allocation, freed at the end of the call)
   size_t off = 0;
