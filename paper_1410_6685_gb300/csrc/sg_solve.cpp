@@ -4,8 +4,8 @@
 //
 //   1. P A = L U in binary32 storage: panels of 32 columns factored by a
 //      thread-block cluster, trailing updates A22 -= L21 U12 on the tensor
-//      cores (bf16 / fp16 operands, binary32 accumulation) or in binary32 on
-//      the CUDA cores.
+//      cores (bf16 / fp16 operands, binary32 accumulation) or in binary32
+//      (three bf16 pieces per operand there, or the CUDA cores).
 //   2. x0 = U^-1 L^-1 P b (binary32 substitution of b rounded to binary32).
 //   3. repeat: r = b - A x in binary64 (A widened exactly), d = LU \ r in
 //      binary32, x += d in binary64, until max|d| <= refine_tol max|x|, or
@@ -65,7 +65,8 @@ cudaError_t factor_in_place(sg_ctx* c, float* lu, int n, int* piv, int* perm, in
   // columns and one fused kernel updates the block's columns to its right;
   // per outer block one launch applies its interchanges everywhere else, one
   // solves U12 for its 128 rows, and the trailing matrix is updated with
-  // K = 128 (tensor cores, or binary32 SIMT)
+  // K = 128 (tensor cores, or in binary32 where the pieces do not gain on them
+  // the CUDA cores)
   const bool tc = prec != SG_PREC_F32_SIMT;
   auto at = [&](int r, int col) { return lu + (size_t)r * n + col; };
   for (int K = 0; K < n && e == cudaSuccess; K += sgk::kLuOuter) {
@@ -192,7 +193,7 @@ cudaError_t capture(sg_ctx* c, LuCache& L, cudaGraphExec_t* exec, int64_t* kerne
 // The choice costs one read-back of 8 bytes (about 15 us: a determinant of n = 8
 // 97 us with it, 84 without); where it applies it
 // takes the factorisation at n = 8192 from 14.8 to 4.1 ms (binary32 updates: 21.8
-// to 6.7 ms), at 2048 from 2.82 to 0.70 ms.  Waits for the stream.  Afterwards
+// to 6.5 ms), at 2048 from 2.82 to 0.70 ms.  Waits for the stream.  Afterwards
 // c->lu.lu holds L\U, c->lu.piv the interchanges and *hinfo the zero-pivot
 // report.
 sg_status lu_factor(sg_ctx* c, const float* A, int n, sg_precision prec, double* norms,
